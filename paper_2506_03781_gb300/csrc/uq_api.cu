@@ -446,6 +446,11 @@ uq_status uq_check_device(void* stream) {
     if (e == cudaSuccess) e = uq::omni_error(true, &flag_omni);
     if (e == cudaSuccess) e = uq::awq_error(true, &flag_awq);
     if (e == cudaSuccess) e = uq::gemv_error(true, &flag_gemv);
+    if (e == cudaSuccess) {
+        unsigned int flag_tc = 0;
+        e = uq::bcq_tc_error(true, &flag_tc);
+        flag_gemv |= flag_tc;
+    }
     if (e != cudaSuccess) return fail(UQ_ERR_CUDA, "uq_check_device: %s", cudaGetErrorString(e));
     flag |= (flag_step << 4) | (flag_omni << 8) | (flag_awq << 12) | (flag_gemv << 16);
     const unsigned int drain_bits = 0x88888u;   // kDrainTimeoutBit of each kernel family

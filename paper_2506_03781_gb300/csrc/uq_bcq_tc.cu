@@ -1,0 +1,662 @@
+// BCQ product on the tensor cores: y = W~ x with
+// W~[r, i] = sum_j alpha*_{r,k,j} c_{j,r,i} + z*_{r,k} (k = i / g) from the
+// exported bit-planes, as one +-1 matrix product per plane and block of GB
+// columns of one group (GB = 32, 64, or 128 for larger groups):
+//   y_r += sum_j alpha*_j (C_j x)_r + z* S,   S = sum of x over the block.
+//
+// The +-1 entries are exact in bf16 and so are the activations: a bf16 token
+// is one column of the right-hand matrix, an fp32 token three (its value cut
+// into three bf16 pieces that add up to it exactly), so every product is
+// exact and the sums are taken in fp32 (tcgen05.mma kind::f16, 128 rows by N
+// columns, fp32 accumulators in tensor memory).
+//
+// A warpgroup owns 128 rows, one per thread.  For every plane and 128
+// columns a thread expands the row's four plane words to +-1 values in
+// registers and stores them to tensor memory, which is the left operand;
+// element k = 2 (16 word + p) + h of a row is bit p + 16 h of the word, so a
+// register holds the bits p and p + 16, moved to its two sign positions by
+// one product and one logic operation.  The block keeps the activations of
+// its column slice in shared memory in the same column order (K-major core
+// matrices of 8 tokens x 16 bytes, no swizzle).  The sums come back one row per thread and are scaled
+// by that row's alpha* in registers.  Operand and sums have two buffers each:
+// a plane is expanded while the products of the one before run.  One to three
+// warpgroups per block, each with its own rows and its own part of tensor
+// memory, cover each other's waits.  The products and copies of a warpgroup
+// are issued by one more warp of its own, so none of the four ever waits for
+// another one (one such warp for all warpgroups issued a plane every 500
+// clocks: its fence waits for the products that it issued before).
+//
+// The plane words come through a ring of shared-memory stages per warpgroup,
+// filled by tensor copies (box: 16 kTcSbs bytes of 128 rows of all planes,
+// swizzled so that one row per thread reads without bank conflicts); where
+// rows are not whole 128-column passes every thread loads its row's words.
+//
+// Split: block (slice, row block) keeps one column slice of all tokens of its
+// chunk and walks its 128-row tiles.  With one slice the result is y itself,
+// else the slices go to the caller's workspace [slice][token][row] and are
+// summed in order by a second kernel.  Every wait is bounded.  Deterministic;
+// no atomics on outputs.
+//
+// What bounds it: with 64 columns the tensor cores need 256 clocks for a
+// plane of 128 x 128 (measured 272) and the two warpgroups about 900 each,
+// the expansion (124 operations per thread, half of them on the half-rate
+// logic pipe) and the scaling of 64 sums; with 16 columns the products take
+// 197 clocks and three warpgroups about 550 each.  14336 x 4096, q = 3,
+// g = 128, bf16: 64 tokens 447 -> 39.4 us (per-token lookup tables before),
+// 16 tokens 114 -> 20.3 us, 4 tokens 30.4 -> 19.4 us; 8192 x 28672, 4 fp32
+// tokens: 99.8 -> 76.4 us.  The same product with mma.sync and fragments in
+// registers took 72.5, 28.2, 20.6 and 108 us: a fragment register holds the
+// same expanded pair, but every lane of a quad repeats the loads and the
+// scaling, and 64 columns are bound by that pipe (38 us).  Error against 64
+// bits: 0.8e-7 to 1.3e-7, the lookup tables' 0.7e-7 to 1.7e-7.
+#include <cuda.h>   // CUtensorMap
+
+#include <atomic>
+
+#include "uq_common.cuh"
+#include "uq_launch.h"
+#include "uq_pipe.cuh"
+
+namespace uq {
+
+static __device__ unsigned int g_tc_err = 0;
+
+// Tensor map of the bit-planes (uq_gemv.cu); false if the driver cannot encode it.
+bool bcq_planes_map(const uint32_t* planes, int64_t out, int n_in, int q, int box_words, int box_rows, CUtensorMap* map);
+
+constexpr int kTcCols = 128;                      // columns of one pass
+constexpr int kTcRows = 128;                      // rows of a tile: one per thread of a warpgroup
+constexpr int kTcMaxGroups = 3;                   // warpgroups per block
+constexpr int kTcSmem = 226 * 1024;               // dynamic shared memory a block may use
+constexpr int kTcMinSmem = 116 * 1024;            // more than half an SM: one block, one user of tensor memory, per SM
+
+// Passes of a stage, and stages of a warpgroup's ring.
+__host__ __device__ constexpr int tc_sbs(int n) { return n == 64 ? 2 : 4; }
+constexpr int kTcStages = 2;
+__host__ __device__ constexpr int tc_stage_bytes(int q, int n) { return q * kTcRows * 16 * tc_sbs(n); }
+// Tensor-memory columns of one warpgroup: two expanded planes (64 each) and
+// two buffers of the sums of a pass's blocks.
+__host__ __device__ constexpr int tc_tmem_cols(int gb, int n) { return 2 * (64 + kTcCols / gb * n); }
+__host__ __device__ constexpr int tc_groups(int gb, int n) {
+    return 512 / tc_tmem_cols(gb, n) < kTcMaxGroups ? 512 / tc_tmem_cols(gb, n) : kTcMaxGroups;
+}
+__host__ __device__ constexpr int tc_pass_bytes(int gb, int n) { return kTcCols * n * 2 + kTcCols / gb * n * 4; }
+
+namespace tc {
+
+__device__ __forceinline__ void alloc(uint32_t dst, uint32_t cols) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(dst), "r"(cols) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void dealloc(uint32_t addr, uint32_t cols) {
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(addr), "r"(cols) : "memory");
+}
+__device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
+__device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
+__device__ __forceinline__ void wait_store() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+// One lane of a converged warp.
+__device__ __forceinline__ uint32_t elect() {
+    uint32_t p;
+    asm volatile(
+        "{\n\t.reg .pred q;\n\t"
+        "elect.sync _|q, 0xffffffff;\n\t"
+        "selp.u32 %0, 1, 0, q;\n\t}"
+        : "=r"(p));
+    return p;
+}
+// d (128 x N, fp32) = a (128 x 16, tensor memory) b (16 x N, shared memory) + d if acc,
+// issued by the elected lane.  Called by the whole warp with uniform
+// arguments: inside a branch of one thread the operands cannot be uniform
+// registers, and an issue took 85 to 195 clocks instead of 25 (16 columns).
+__device__ __forceinline__ void mma(uint32_t d, uint32_t a, uint64_t b, uint32_t idesc, uint32_t acc, uint32_t elected) {
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "setp.ne.b32 q, %5, 0;\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d),
+        "r"(a), "l"(b), "r"(idesc), "r"(acc), "r"(elected)
+        : "memory");
+}
+__device__ __forceinline__ void load_box(uint32_t dst, const CUtensorMap* m, int x, int y, int z, uint32_t bar) {
+    asm volatile(
+        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], "
+        "[%5];" ::"r"(dst),
+        "l"(reinterpret_cast<uint64_t>(m)), "r"(x), "r"(y), "r"(z), "r"(bar)
+        : "memory");
+}
+__device__ __forceinline__ void commit(uint32_t bar) {
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+}
+// 16 words per thread: lane i of the warp holds row i of its 32 rows
+__device__ __forceinline__ void load(uint32_t addr, float (&r)[16]) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];\n\t"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=f"(r[0]), "=f"(r[1]), "=f"(r[2]), "=f"(r[3]), "=f"(r[4]), "=f"(r[5]), "=f"(r[6]), "=f"(r[7]), "=f"(r[8]), "=f"(r[9]), "=f"(r[10]), "=f"(r[11]), "=f"(r[12]), "=f"(r[13]), "=f"(r[14]), "=f"(r[15])
+        : "r"(addr)
+        : "memory");
+}
+
+__device__ __forceinline__ void store(uint32_t addr, const uint32_t (&r)[16]) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};" ::"r"(addr),
+                 "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
+                 : "memory");
+}
+
+
+// Instruction descriptor: fp32 sums, bf16 operands, both K-major, M = 128.
+__host__ __device__ constexpr uint32_t idesc(int n) {
+    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(kTcRows >> 4) << 24);
+}
+// Shared-memory descriptor without swizzle: core matrices of 8 rows x 16
+// bytes, 128 bytes apart over the rows and n * 16 bytes apart over K.
+__device__ __forceinline__ uint64_t desc(uint32_t addr, int n) {
+    return (uint64_t)((addr >> 4) & 0x3fffu) | ((uint64_t)(n) << 16) | ((uint64_t)(128 >> 4) << 32) | (1ull << 46);
+}
+
+}  // namespace tc
+
+// Bits p and p + 16 of w as two bf16 values, +1 where set and -1 where not:
+// moved to the sign positions by a product (the multiply pipe is idle here,
+// the logic pipe is what bounds the expansion) and one three-input logic
+// operation.  The factors 2^(15 - p) and the two masks come from the kernel's
+// arguments, so the compiler keeps the product and needs no second operation
+// for a second immediate.
+struct Pm1 {
+    uint32_t mul[16], mask, one;
+};
+__device__ __forceinline__ uint32_t pm1(uint32_t w, int p, const Pm1& c, uint32_t mask, uint32_t one) {
+    uint32_t r;
+    asm("lop3.b32 %0, %1, %2, %3, 0x6a;" : "=r"(r) : "r"(p == 15 ? w : w * c.mul[p]), "r"(mask), "r"(one));
+    return r;
+}
+
+// Piece 0, 1 or 2 of an fp32 value: three bf16 numbers that add up to it
+// exactly (8 significant bits each, cut and not rounded, so none overflows).
+// Infinities and NaN stay in piece 0.  Used for words that hold one.
+__device__ __forceinline__ uint32_t bf16_piece(float x, int piece) {
+    const uint32_t b = __float_as_uint(x);
+    if ((b & 0x7f800000u) == 0x7f800000u) return piece ? 0u : (b & 0x007fffffu) ? 0x7fc0u : b >> 16;
+    const uint32_t h0 = b & 0xffff0000u;
+    const float r = __fsub_rn(x, __uint_as_float(h0));
+    const uint32_t h1 = __float_as_uint(r) & 0xffff0000u;
+    if (piece == 0) return h0 >> 16;
+    if (piece == 1) return h1 >> 16;
+    return __float_as_uint(__fsub_rn(r, __uint_as_float(h1))) >> 16;
+}
+
+template <int Q, int GB, int N>
+__global__ void __launch_bounds__(tc_groups(GB, N) * 160, 1)
+bcq_tc_kernel(const __grid_constant__ CUtensorMap tm_planes, const uint32_t* __restrict__ PLANES,
+              const float* __restrict__ ASTAR, const float* __restrict__ ZSTAR, const void* __restrict__ X, int x_bf16,
+              float* __restrict__ DST, int64_t out, int n_in, int g, int batch, int n_ks, int sb_per, int tiles,
+              int tmem_cols, int staged, const __grid_constant__ Pm1 pm) {
+    constexpr int NB = kTcCols / GB;                       // scaling blocks of one pass
+    constexpr int SBS = tc_sbs(N), SB = tc_stage_bytes(Q, N);
+    extern __shared__ __align__(128) unsigned char tsm[];
+    // per warpgroup and buffer: plane expanded (its four warps), products done; per stage: copies landed
+    __shared__ __align__(8) unsigned long long ready[kTcMaxGroups][2], done[kTcMaxGroups][2], full[kTcMaxGroups][kTcStages];
+    __shared__ uint32_t tm_addr;
+    __shared__ volatile int dead;                          // a wait ran out: every warp stops
+    const int warp = __shfl_sync(kFull, threadIdx.x >> 5, 0), lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    // warps 0 .. 4 n_wg - 1: four of each warpgroup; then the issuing warp of each
+    const int n_wg = blockDim.x / 160, wt = threadIdx.x & 127;
+    const bool issuer = warp >= 4 * n_wg;
+    const int wg = issuer ? warp - 4 * n_wg : warp >> 2;
+    const int slice = (int)(blockIdx.x % n_ks);
+    const int64_t tile0 = (int64_t)(blockIdx.x / n_ks) * tiles;
+    const int words = n_in / 32, Gr = n_in / g;
+    const int n_sb = (n_in + kTcCols - 1) / kTcCols;
+    const int sb0 = slice * sb_per, sbn = n_sb - sb0 < sb_per ? n_sb - sb0 : sb_per;
+    const int tpc = x_bf16 ? N : N / 3;                    // tokens of a chunk
+    const int tok0 = (int)blockIdx.y * tpc, toks = batch - tok0 < tpc ? batch - tok0 : tpc;
+    // stages first (on a 1024-byte boundary), then the activations and the block sums
+    unsigned char* base = tsm + ((1024u - (tma::smem_addr(tsm) & 1023u)) & 1023u);
+    uint4* xs = reinterpret_cast<uint4*>(base + (staged ? (size_t)n_wg * kTcStages * SB : 0));      // [sb][16][N]
+    float* sums = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(xs) + (size_t)sb_per * kTcCols * N * 2);
+
+    // the slice sum (a programmatic dependent) may be scheduled now; it waits for this grid's results
+    asm volatile("griddepcontrol.launch_dependents;");
+    if (warp == 0) tc::alloc(tma::smem_addr(&tm_addr), (uint32_t)tmem_cols);
+    if (threadIdx.x < kTcMaxGroups) {
+        const int i = threadIdx.x;
+        for (int k = 0; k < 2; ++k) {
+            tma::bar_init(tma::smem_addr(&ready[i][k]), 4);
+            tma::bar_init(tma::smem_addr(&done[i][k]), 1);
+        }
+        for (int k = 0; k < kTcStages; ++k) tma::bar_init(tma::smem_addr(&full[i][k]), 1);
+        dead = 0;
+        tma::bar_init_fence();
+    }
+    __syncthreads();
+    // launched as a programmatic dependent itself: nothing global is touched before the work ahead has completed
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+
+    // stages of a warpgroup: tile-major, spt per tile
+    const int spt = (sbn + SBS - 1) / SBS;
+    const int64_t row_tiles = (out + kTcRows - 1) / kTcRows;
+    const int n_tiles = (int)(row_tiles - tile0 < tiles ? row_tiles - tile0 : tiles);
+    auto tiles_of = [&](int w) { return n_tiles > w ? (n_tiles - w + n_wg - 1) / n_wg : 0; };
+    auto copy = [&](int w, int i) {                        // stage i of warpgroup w
+        const int s = i & (kTcStages - 1), t = i / spt;
+        const uint32_t fb = tma::smem_addr(&full[w][s]);
+        tma::fence_async_smem();                           // the warpgroup's reads of this stage come first
+        tma::bar_arrive_tx(fb, (uint32_t)SB);
+        tc::load_box(tma::smem_addr(base + ((size_t)w * kTcStages + s) * SB), &tm_planes, (sb0 + (i - t * spt) * SBS) * 4,
+                     (int)((tile0 + w + (int64_t)t * n_wg) * kTcRows), 0, fb);
+    };
+    const int my_tiles = tiles_of(wg);
+    if (staged && issuer && lane == 0)
+        for (int i = 0; i < kTcStages && i < my_tiles * spt; ++i) copy(wg, i);
+
+    // --- the slice's activations in operand order, and their block sums ---
+    for (int it = warp; it < sbn * (N / 8); it += nw) {
+        const int sb = it / (N / 8), n8 = it - sb * (N / 8);
+        const int tig = lane & 3, col = n8 * 8 + (lane >> 2);
+        const int tok = x_bf16 ? col : col / 3, piece = x_bf16 ? 0 : col - tok * 3;
+        const int word = (sb0 + sb) * 4 + tig;
+        uint32_t pr[16];                                   // columns p and p + 16 of the word
+        float sum = 0.f;
+        if (tok < toks && word < words) {
+            const int64_t x0 = (int64_t)(tok0 + tok) * n_in + (int64_t)word * 32;
+            if (x_bf16) {
+                const uint4* p = reinterpret_cast<const uint4*>(static_cast<const uint16_t*>(X) + x0);
+                uint32_t u[16];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const uint4 v = __ldg(p + i);
+                    u[4 * i] = v.x; u[4 * i + 1] = v.y; u[4 * i + 2] = v.z; u[4 * i + 3] = v.w;
+                }
+#pragma unroll
+                for (int i = 0; i < 16; ++i) sum += __uint_as_float(u[i] << 16) + __uint_as_float(u[i] & 0xffff0000u);
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    pr[2 * i] = __byte_perm(u[i], u[i + 8], 0x5410);
+                    pr[2 * i + 1] = __byte_perm(u[i], u[i + 8], 0x7632);
+                }
+            } else {
+                const float4* p = reinterpret_cast<const float4*>(static_cast<const float*>(X) + x0);
+                // x less its upper 16 bits once for piece 1 and twice for piece 2, then cut
+                const uint32_t m1 = piece >= 1 ? 0xffff0000u : 0u, m2 = piece == 2 ? 0xffff0000u : 0u;
+                auto cut = [&](float v) {
+                    v = __fsub_rn(v, __uint_as_float(__float_as_uint(v) & m1));
+                    v = __fsub_rn(v, __uint_as_float(__float_as_uint(v) & m2));
+                    return __float_as_uint(v);
+                };
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    float lo[4], hi[4];
+                    f4_to(__ldg(p + i), lo);
+                    f4_to(__ldg(p + i + 4), hi);
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const uint32_t a = cut(lo[k]), b = cut(hi[k]);
+                        sum += __uint_as_float(a & 0xffff0000u) + __uint_as_float(b & 0xffff0000u);
+                        pr[4 * i + k] = __byte_perm(a, b, 0x7632);
+                    }
+                }
+                if (!(fabsf(sum) < __int_as_float(0x7f800000))) {      // an infinity or a NaN among them
+                    sum = 0.f;
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        float lo[4], hi[4];
+                        f4_to(__ldg(p + i), lo);
+                        f4_to(__ldg(p + i + 4), hi);
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            const uint32_t a = bf16_piece(lo[k], piece), b = bf16_piece(hi[k], piece);
+                            sum += __uint_as_float(a << 16) + __uint_as_float(b << 16);
+                            pr[4 * i + k] = a | (b << 16);
+                        }
+                    }
+                }
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < 16; ++i) pr[i] = 0u;
+        }
+        if (GB >= 64) sum += __shfl_xor_sync(kFull, sum, 1);
+        if (GB >= 128) sum += __shfl_xor_sync(kFull, sum, 2);
+        if (tig % (4 / NB) == 0) sums[(sb * NB + tig / (4 / NB)) * N + col] = sum;
+#pragma unroll
+        for (int v = 0; v < 4; ++v)
+            xs[(sb * 16 + tig * 4 + v) * N + col] = make_uint4(pr[4 * v], pr[4 * v + 1], pr[4 * v + 2], pr[4 * v + 3]);
+    }
+    tma::fence_async_smem();                               // the products read shared memory through the async proxy
+    tc::fence_before();
+    __syncthreads();
+    tc::fence_after();
+
+    const uint32_t xbase = tma::smem_addr(xs);
+    if (issuer) {
+        // --- products and copies of the warpgroup: the whole warp, uniformly; one lane issues ---
+        const uint32_t e = tc::elect();
+        const uint32_t tm = __shfl_sync(kFull, tm_addr, 0) + (uint32_t)(wg * tc_tmem_cols(GB, N));
+        const uint64_t xdesc = tc::desc(xbase, N);
+        uint32_t b = 0, ph = 0;                             // next buffer, parities of its barriers
+        int stage = 0;
+        bool go = true;
+        for (int t = 0; t < my_tiles && go; ++t)
+            for (int sb = 0; sb < sbn && go; ++sb) {
+                const uint64_t xd = xdesc + (uint32_t)(sb * 16 * N);               // 16-byte units
+#pragma unroll 1
+                for (int j = 0; j < Q; ++j) {
+                    if (!__all_sync(kFull, tma::bar_wait(tma::smem_addr(&ready[wg][b]), (ph >> b) & 1u))) {
+                        if (lane == 0) atomicOr(&g_tc_err, 4u);
+                        dead = 1;
+                    }
+                    if (__any_sync(kFull, dead)) { go = false; break; }
+                    tc::fence_after();
+#pragma unroll
+                    for (int k = 0; k < 8; ++k)             // 16 columns a step, 8 / NB steps a block
+                        tc::mma(tm + 128 + (b * NB + k / (8 / NB)) * N, tm + 64 * b + 8 * k, xd + 2 * k * N, tc::idesc(N),
+                                k % (8 / NB) ? 1u : 0u, e);
+                    if (e) tc::commit(tma::smem_addr(&done[wg][b]));
+                    __syncwarp();
+                    ph ^= 1u << b;
+                    b ^= 1u;
+                }
+                // the last plane of a stage has been read: its slot is free
+                if (staged && go && (sb == sbn - 1 || sb % SBS == SBS - 1)) {
+                    if (e && stage + kTcStages < my_tiles * spt) copy(wg, stage + kTcStages);
+                    __syncwarp();
+                    ++stage;
+                }
+            }
+    }
+    const uint32_t tmem = tm_addr + (uint32_t)(wg * tc_tmem_cols(GB, N));
+    const uint32_t tlane = tmem + ((uint32_t)((warp & 3) * 32) << 16);         // this warp's 32 rows
+    const unsigned char* ring = base + (size_t)wg * kTcStages * SB;
+    const int64_t pstride = out * words;
+    const int gdiv = g > kTcCols ? g / kTcCols : 1;        // passes per group
+    const bool vec = g <= kTcCols && (Gr & 3) == 0;        // four groups of a row are 16-byte aligned
+    uint32_t phase = 0;                                    // bit b: parity of buffer b's next completion
+    int buf = 0, waited = 0;                               // buffer of the next plane; stages waited for
+    bool alive = true;
+    const uint32_t mask = pm.mask, one = pm.one;
+
+    for (int mt = 0; mt < my_tiles && alive && !issuer; ++mt) {
+        const int64_t row_raw = (tile0 + wg + (int64_t)mt * n_wg) * kTcRows + wt;
+        const int64_t row = row_raw < out ? row_raw : out - 1;     // rows past the last one are not stored
+        float acc[N], v[N];
+#pragma unroll
+        for (int n = 0; n < N; ++n) acc[n] = 0.f;
+
+        // alpha* and z* of four blocks of the row at a time
+        float pa[4][Q], pz[4];
+        auto params = [&](int b0) {                        // blocks b0 .. b0 + 3 of the row
+            if (vec) {
+                if (b0 < Gr) {
+                    const float4* a4 = reinterpret_cast<const float4*>(ASTAR + (row * Gr + b0) * Q);
+                    float f[4 * Q];
+#pragma unroll
+                    for (int i = 0; i < Q; ++i) f4_to(__ldg(a4 + i), f + 4 * i);
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+#pragma unroll
+                        for (int j = 0; j < Q; ++j) pa[k][j] = f[k * Q + j];
+                    f4_to(__ldg(reinterpret_cast<const float4*>(ZSTAR + row * Gr + b0)), pz);
+                }
+            } else {
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const int grp = (b0 + k) / gdiv;
+                    const bool in = grp < Gr;
+                    pz[k] = in ? __ldg(ZSTAR + row * Gr + grp) : 0.f;
+#pragma unroll
+                    for (int j = 0; j < Q; ++j) pa[k][j] = in ? __ldg(ASTAR + (row * Gr + grp) * Q + j) : 0.f;
+                }
+            }
+        };
+        // expands the warp's rows of plane j of pass sb into operand buffer b
+        auto expand = [&](int sb, int j, int b) {
+            if (staged && j == 0 && sb % SBS == 0) {
+                const int s = waited & (kTcStages - 1);
+                if (!tma::bar_wait(tma::smem_addr(&full[wg][s]), (uint32_t)(waited / kTcStages) & 1u)) {
+                    atomicOr(&g_tc_err, 2u);
+                    dead = 1;
+                }
+                ++waited;
+                __syncwarp();
+            }
+            uint4 w4;
+            if (staged) {
+                const unsigned char* st = ring + ((waited - 1) & (kTcStages - 1)) * SB + j * (kTcRows * 16 * SBS);
+                const int c = sb % SBS, x = SBS == 4 ? (wt >> 1) & 3 : (wt >> 2) & 1;      // the copy's swizzle
+                w4 = *reinterpret_cast<const uint4*>(st + wt * 16 * SBS + ((c ^ x) << 4));
+            } else {
+                const int word = (sb0 + sb) * 4;
+                const uint32_t* p = PLANES + row * words + j * pstride + word;
+                w4.x = __ldg(p);
+                w4.y = word + 1 < words ? __ldg(p + 1) : 0u;
+                w4.z = word + 2 < words ? __ldg(p + 2) : 0u;
+                w4.w = word + 3 < words ? __ldg(p + 3) : 0u;
+            }
+            const uint32_t w[4] = {w4.x, w4.y, w4.z, w4.w};
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                uint32_t a[16];
+#pragma unroll
+                for (int p = 0; p < 16; ++p) a[p] = pm1(w[i], p, pm, mask, one);
+                tc::store(tlane + 64 * b + 16 * i, a);
+            }
+            tc::wait_store();
+            tc::fence_before();
+            __syncwarp();
+            if (lane == 0) tma::bar_arrive(tma::smem_addr(&ready[wg][b]));
+        };
+        expand(0, 0, buf);
+        int left = 0;                                      // blocks of pa, pz not yet used
+        for (int sb = 0; sb < sbn && alive; ++sb) {
+            if (left == 0) {
+                const int b0 = ((sb0 + sb) * NB) & ~3, skip = (sb0 + sb) * NB - b0;
+                params(b0);
+                left = 4 - skip;
+                for (int i = 0; i < skip; i += NB) {        // the slice begins inside the four
+#pragma unroll
+                    for (int k = 0; k + NB < 4; ++k) {
+                        pz[k] = pz[k + NB];
+#pragma unroll
+                        for (int j = 0; j < Q; ++j) pa[k][j] = pa[k + NB][j];
+                    }
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < Q; ++j) {
+                if (j + 1 < Q) expand(sb, j + 1, buf ^ 1);
+                else if (sb + 1 < sbn) expand(sb + 1, 0, buf ^ 1);
+                if (!tma::bar_wait(tma::smem_addr(&done[wg][buf]), (phase >> buf) & 1u)) {
+                    atomicOr(&g_tc_err, 1u);
+                    dead = 1;
+                }
+                phase ^= 1u << buf;
+                __syncwarp();
+                tc::fence_after();
+#pragma unroll
+                for (int h = 0; h < NB; ++h) {
+                    const float* S = sums + (sb * NB + h) * N;
+#pragma unroll
+                    for (int n0 = 0; n0 < N; n0 += 16) {
+                        float d[16];
+                        tc::load(tlane + 128 + (buf * NB + h) * N + n0, d);
+#pragma unroll
+                        for (int n = 0; n < 16; ++n) {
+                            // the block's terms first, then the running sum: one rounding per pass at its size
+                            if (j == 0) v[n0 + n] = h == 0 ? __fmul_rn(pz[h], S[n0 + n]) : fmaf(pz[h], S[n0 + n], v[n0 + n]);
+                            v[n0 + n] = fmaf(pa[h][j], d[n], v[n0 + n]);
+                            if (j == Q - 1 && h == NB - 1) acc[n0 + n] += v[n0 + n];
+                        }
+                    }
+                }
+                buf ^= 1;
+            }
+            if (__any_sync(kFull, dead)) alive = false;
+            left -= NB;
+            if (NB < 4) {
+#pragma unroll
+                for (int k = 0; k + NB < 4; ++k) {
+                    pz[k] = pz[k + NB];
+#pragma unroll
+                    for (int j = 0; j < Q; ++j) pa[k][j] = pa[k + NB][j];
+                }
+            }
+        }
+        if (alive && row_raw < out) {
+            float* dst = DST + ((int64_t)slice * batch + tok0) * out + row;
+            if (x_bf16) {
+#pragma unroll
+                for (int n = 0; n < N; ++n)
+                    if (n < toks) dst[(int64_t)n * out] = acc[n];
+            } else {
+#pragma unroll
+                for (int t = 0; t < N / 3; ++t)
+                    if (t < toks) dst[(int64_t)t * out] = (acc[3 * t] + acc[3 * t + 1]) + acc[3 * t + 2];
+            }
+        }
+    }
+    // after a wait ran out: bounded waits for copies and products in flight before the block leaves
+    __syncthreads();
+    if (dead && wt == 0 && !issuer) {
+        const bool gone = tma::bar_wait(tma::smem_addr(&full[wg][waited & (kTcStages - 1)]), (uint32_t)(waited / kTcStages) & 1u, 1ll << 24) &
+                          tma::bar_wait(tma::smem_addr(&done[wg][buf]), (phase >> buf) & 1u, 1ll << 24);
+        if (!gone) atomicOr(&g_tc_err, kDrainTimeoutBit);
+    }
+    tc::fence_before();
+    __syncthreads();
+    if (warp == 0) tc::dealloc(tm_addr, (uint32_t)tmem_cols);
+}
+
+cudaError_t bcq_tc_error(bool clear, unsigned int* flag) {
+    unsigned int v = 0;
+    cudaError_t e = cudaMemcpyFromSymbol(&v, g_tc_err, sizeof(v));
+    if (e != cudaSuccess) return e;
+    *flag = v;
+    if (clear && v) {
+        const unsigned int z = 0;
+        e = cudaMemcpyToSymbol(g_tc_err, &z, sizeof(z));
+    }
+    return e;
+}
+
+namespace {
+
+struct TcPlan {
+    int n_ks, sb_per, n_rb, tiles, groups;
+};
+
+// Slices, tiles per block and warpgroups for the least estimated time (in SM
+// clocks): the waves of blocks, each with the operands it builds and its
+// rounds of tiles, and the slice sum where there is more than one slice.
+template <int Q, int GB, int N>
+TcPlan tc_plan(int64_t out, int n_in, int chunks, bool staged) {
+    const int sms = sm_count();
+    const int n_sb = (n_in + kTcCols - 1) / kTcCols;
+    const int64_t all = (out + kTcRows - 1) / kTcRows;
+    const int most_ks = (n_in + 511) / 512;                // the workspace holds this many partials of every output
+    // a pass of one plane: alone (waits included), and what it takes of the SM among others
+    const double alone = 450.0 + 7.0 * N, busy = 4.5 * N > 200.0 ? 4.5 * N : 200.0;
+    TcPlan best{};
+    double best_cost = -1.0;
+    for (int w = 1; w <= tc_groups(GB, N); ++w) {
+        const int fit = (kTcSmem - 1024 - (staged ? w * kTcStages * tc_stage_bytes(Q, N) : 0)) / tc_pass_bytes(GB, N);
+        const int least = (n_sb + fit - 1) / fit;
+        for (int ks = least; ks <= most_ks && ks < least + 16; ++ks) {
+            const int per = (n_sb + ks - 1) / ks, n_ks = (n_sb + per - 1) / per;
+            for (int waves = 1; waves <= 2; ++waves) {
+                int64_t n_rb = (int64_t)sms * waves / ((int64_t)n_ks * chunks);
+                n_rb = n_rb < 1 ? 1 : n_rb > all ? all : n_rb;
+                const int64_t tiles = (all + n_rb - 1) / n_rb;
+                n_rb = (all + tiles - 1) / tiles;
+                const int64_t wv = (n_rb * n_ks * chunks + sms - 1) / sms;
+                const int ww = tiles < w ? (int)tiles : w;
+                const int64_t rounds = (tiles + ww - 1) / ww;
+                const double pass = alone > ww * busy ? alone : ww * busy;
+                const double cost = (double)wv * (2500.0 + per * N * 12.0 / ww + (double)rounds * per * Q * pass) +
+                                    (n_ks > 1 ? 3000.0 : 0.0);
+                if (best_cost < 0.0 || cost < best_cost) {
+                    best_cost = cost;
+                    best = TcPlan{n_ks, per, (int)n_rb, (int)tiles, ww};
+                }
+            }
+        }
+    }
+    return best;
+}
+
+template <int Q, int GB, int N>
+cudaError_t run_tc(const uint32_t* planes, const float* astar, const float* zstar, int64_t out, int n_in, int g,
+                   const void* x, int x_bf16, int batch, float* y, float* work, cudaStream_t st) {
+    const int tpc = x_bf16 ? N : N / 3, chunks = (batch + tpc - 1) / tpc;
+    // whole passes: the planes come through tensor copies
+    CUtensorMap map = {};
+    const bool staged = n_in % kTcCols == 0 && bcq_planes_map(planes, out, n_in, Q, 4 * tc_sbs(N), kTcRows, &map);
+    const TcPlan p = tc_plan<Q, GB, N>(out, n_in, chunks, staged);
+    Pm1 pm;
+    for (int i = 0; i < 16; ++i) pm.mul[i] = 1u << (15 - i);
+    pm.mask = 0x80008000u;
+    pm.one = 0xbf80bf80u;
+    auto kern = bcq_tc_kernel<Q, GB, N>;
+    static std::atomic<int> ready[kMaxDevices] = {};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= kMaxDevices || ready[dev].load(std::memory_order_relaxed) == 0) {
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcSmem);
+        if (e != cudaSuccess) return e;
+        if (dev >= 0 && dev < kMaxDevices) ready[dev].store(1, std::memory_order_relaxed);
+    }
+    int cols = 32;
+    while (cols < p.groups * tc_tmem_cols(GB, N)) cols *= 2;
+    int smem = 1024 + p.sb_per * tc_pass_bytes(GB, N) + (staged ? p.groups * kTcStages * tc_stage_bytes(Q, N) : 0);
+    if (smem < kTcMinSmem) smem = kTcMinSmem;
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = dim3((unsigned)(p.n_ks * p.n_rb), (unsigned)chunks);
+    cfg.blockDim = dim3(p.groups * 160);
+    cfg.dynamicSmemBytes = (size_t)smem;
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    e = cudaLaunchKernelEx(&cfg, kern, map, planes, astar, zstar, x, x_bf16, p.n_ks > 1 ? work : y, out, n_in, g, batch,
+                           p.n_ks, p.sb_per, p.tiles, cols, staged ? 1 : 0, pm);
+    if (e != cudaSuccess || p.n_ks == 1) return e;
+    return gemv_reduce(work, y, (int64_t)batch * out, p.n_ks, st);
+}
+
+template <int Q, int GB>
+cudaError_t tc_n(const uint32_t* planes, const float* astar, const float* zstar, int64_t out, int n_in, int g,
+                 const void* x, int x_bf16, int batch, float* y, float* work, cudaStream_t st) {
+    // columns of one pass; more go in chunks of tokens, each reading the planes
+    // again.  64 columns only where a pass is one block: the sums of more
+    // blocks leave tensor memory for one warpgroup alone.
+    const int cols = batch * (x_bf16 ? 1 : 3);
+    if (cols <= 16) return run_tc<Q, GB, 16>(planes, astar, zstar, out, n_in, g, x, x_bf16, batch, y, work, st);
+    if constexpr (GB == 128)
+        if (cols > 32) return run_tc<Q, GB, 64>(planes, astar, zstar, out, n_in, g, x, x_bf16, batch, y, work, st);
+    return run_tc<Q, GB, 32>(planes, astar, zstar, out, n_in, g, x, x_bf16, batch, y, work, st);
+}
+
+template <int Q>
+cudaError_t tc_g(const uint32_t* planes, const float* astar, const float* zstar, int64_t out, int n_in, int g,
+                 const void* x, int x_bf16, int batch, float* y, float* work, cudaStream_t st) {
+    if (g == 32) return tc_n<Q, 32>(planes, astar, zstar, out, n_in, g, x, x_bf16, batch, y, work, st);
+    if (g == 64) return tc_n<Q, 64>(planes, astar, zstar, out, n_in, g, x, x_bf16, batch, y, work, st);
+    return tc_n<Q, 128>(planes, astar, zstar, out, n_in, g, x, x_bf16, batch, y, work, st);
+}
+
+}  // namespace
+
+cudaError_t launch_bcq_tc(const uint32_t* planes, const float* astar, const float* zstar, int64_t out, int n_in, int q,
+                          int g, const void* x, int xdtype, int batch, float* y, float* work, cudaStream_t st) {
+    const int b16 = xdtype == UQ_W_BF16 ? 1 : 0;
+    switch (q) {
+        case 1: return tc_g<1>(planes, astar, zstar, out, n_in, g, x, b16, batch, y, work, st);
+        case 2: return tc_g<2>(planes, astar, zstar, out, n_in, g, x, b16, batch, y, work, st);
+        case 3: return tc_g<3>(planes, astar, zstar, out, n_in, g, x, b16, batch, y, work, st);
+        default: return tc_g<4>(planes, astar, zstar, out, n_in, g, x, b16, batch, y, work, st);
+    }
+}
+
+}  // namespace uq

@@ -852,6 +852,21 @@ static bool gemv_tensor_maps(const uint32_t* planes, const float* astar, const f
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// Tensor map of the bit-planes with boxes of box_words x box_rows x q, the
+// 16-byte pieces of a row swizzled over its 32 or 64 bytes.  in a multiple of
+// 128; false as above.
+bool bcq_planes_map(const uint32_t* planes, int64_t out, int n_in, int q, int box_words, int box_rows, CUtensorMap* map) {
+    const TensorMapEncode enc = tensor_map_encoder();
+    const cuuint64_t words = (cuuint64_t)n_in / 32, rows = (cuuint64_t)out;
+    if (enc == nullptr || words * 4 * rows >= (1ull << 40)) return false;
+    const cuuint64_t dim[3] = {words, rows, (cuuint64_t)q};
+    const cuuint64_t stride[2] = {words * 4, words * 4 * rows};
+    const cuuint32_t box[3] = {(cuuint32_t)box_words, (cuuint32_t)box_rows, (cuuint32_t)q}, one[3] = {1, 1, 1};
+    return enc(map, CU_TENSOR_MAP_DATA_TYPE_UINT32, 3, const_cast<uint32_t*>(planes), dim, stride, box, one,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, box_words == 16 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B,
+               CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 // Opts a kernel into `smem` bytes of dynamic shared memory and returns its
 // resident blocks per SM, once per device (Tag: one cache per kernel).
 template <typename Tag, typename KERN>
@@ -896,7 +911,7 @@ static void gemv_row_blocks(int64_t out, int n_tiles, int per_sm, int64_t& n_rb,
 // The tile sum is launched with programmatic stream serialization, so its
 // launch overlaps the end of the product kernel (it waits for that grid's
 // results with griddepcontrol.wait before reading them).
-static cudaError_t gemv_reduce(const float* work, float* y, int64_t n, int n_tiles, cudaStream_t st) {
+cudaError_t gemv_reduce(const float* work, float* y, int64_t n, int n_tiles, cudaStream_t st) {
     int64_t blocks = (n + 255) / 256;
     const int64_t cap = (int64_t)sm_count() * 8;
     if (blocks > cap) blocks = cap;
@@ -1038,6 +1053,16 @@ static cudaError_t gemv_x(const uint32_t* planes, const float* astar, const floa
 
 cudaError_t launch_gemv(const uint32_t* planes, const float* astar, const float* zstar, int64_t out, int n_in, int q,
                         int g, const void* x, int xdtype, int batch, float* y, float* work, cudaStream_t st) {
+    // The lookup tables hold one token, so their kernels build them and read
+    // the planes once per token; the tensor-core product reads the planes once
+    // for up to 64 columns.  Three tokens and more: 23.6 vs 19.4 us on
+    // 14336 x 4096 (2 tokens: 16.5 vs 19.3), 77 vs 74 on 8192 x 28672 (53 vs
+    // 74), 9.5 vs 8.9 on 1024 x 4096 q = 4 (7.0 vs 8.9), 7.5 vs 6.2 on 256 x
+    // 512 (5.9 vs 6.2).  Two tokens where the 512-column kernels would run:
+    // 31.6 vs 20.4 us on 4096 x 11008, but 8.4 vs 9.0 on 1024 x 8192 g = 512.
+    const bool wide = n_in % kWideCols == 0 && g <= 256;
+    if (batch >= 3 || (batch == 2 && !wide && out * n_in >= (int64_t(1) << 24)))
+        return launch_bcq_tc(planes, astar, zstar, out, n_in, q, g, x, xdtype, batch, y, work, st);
     switch (q) {
         case 1: return gemv_x<1>(planes, astar, zstar, out, n_in, g, x, xdtype, batch, y, work, st);
         case 2: return gemv_x<2>(planes, astar, zstar, out, n_in, g, x, xdtype, batch, y, work, st);

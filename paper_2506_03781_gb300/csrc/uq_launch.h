@@ -61,6 +61,12 @@ cudaError_t gemv_static_workspace(float** work);
 cudaError_t gemv_error(bool clear, unsigned int* flag);
 cudaError_t launch_gemv(const uint32_t* planes, const float* astar, const float* zstar, int64_t out, int n_in, int q,
                         int g, const void* x, int xdtype, int batch, float* y, float* work, cudaStream_t st);
+// y[i] = the n_parts partials work[p][i], summed in order (uq_gemv.cu).
+cudaError_t gemv_reduce(const float* work, float* y, int64_t n, int n_parts, cudaStream_t st);
+// The same product on the tensor cores (uq_bcq_tc.cu), same workspace, and its bounded-wait flag.
+cudaError_t bcq_tc_error(bool clear, unsigned int* flag);
+cudaError_t launch_bcq_tc(const uint32_t* planes, const float* astar, const float* zstar, int64_t out, int n_in, int q,
+                          int g, const void* x, int xdtype, int batch, float* y, float* work, cudaStream_t st);
 // UniQuan with OmniQuant's maps (uq_omni.cu); omni_ok: the group sizes it takes.
 bool omni_ok(const Shape& sh);
 cudaError_t launch_omni_fwd(const Shape& sh, const void* W, uq_params_omni p, uint8_t* codes, int mode, float* what,

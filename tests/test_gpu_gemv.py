@@ -70,7 +70,7 @@ def check(planes, a_star, z_star, x, g, xdtype="f32", label=""):
 # in: one ragged tile, several tiles, a non-multiple of 512.  In a multiple of 1024 with
 # g <= 256 takes the wide-lane kernel (1024-column tiles, 4 to 32 groups per tile); other
 # whole 512-column tiles with 4, 8 and 16 groups per tile the tensor-copy staging, the
-# rest the per-lane copies
+# rest the per-lane copies (one token)
 @pytest.mark.parametrize("out,n_in,g", [(40, 256, 32), (33, 512, 64), (17, 1536, 128), (64, 4096, 128),
                                         (9, 4096 + 32 * 3, 32), (5, 8192, 256), (3, 28672, 128), (300, 1024, 512),
                                         (24, 1024, 32), (13, 2560, 64), (11, 3072, 1024), (6, 4096, 2048)])
@@ -99,6 +99,44 @@ def test_gemv_many_rows(out, n_in, g, q):
     planes, a_star, z_star = random_export(out, n_in, q, g, seed=9 + out)
     x = np.random.default_rng(0).standard_normal((2, n_in)).astype(F32)
     check(planes, a_star, z_star, x, g, label=f"{out} rows {n_in} g{g} q{q}")
+
+
+# The tensor-core product (3 tokens and more): row tiles of 128 with a remainder, one row, columns that are
+# no whole 128-column pass (per-thread loads), slices that begin inside a pass's four groups, every group
+# size class; 16, 32 and 64 matrix columns and several chunks of tokens (an fp32 token takes three columns)
+@pytest.mark.parametrize("out,n_in,g,q", [(1, 32, 32, 3), (127, 96, 32, 1), (129, 192, 64, 2), (300, 320, 64, 4),
+                                          (128, 128, 128, 3), (257, 640, 128, 2), (65, 11008, 128, 3),
+                                          (40, 1280, 256, 4), (31, 3072, 1024, 1), (2500, 6080, 32, 2)])
+@pytest.mark.parametrize("batch,xdtype", [(3, "bf16"), (5, "f32"), (6, "f32"), (17, "bf16"), (22, "f32"),
+                                          (33, "bf16"), (64, "f32"), (64, "bf16")])
+def test_gemv_tensor_core_product(out, n_in, g, q, batch, xdtype):
+    planes, a_star, z_star = random_export(out, n_in, q, g, seed=out + batch)
+    x = np.random.default_rng(batch + q).standard_normal((batch, n_in)).astype(F32)
+    check(planes, a_star, z_star, x, g, xdtype, label=f"{out}x{n_in} g{g} q{q} batch {batch} {xdtype}")
+
+
+@pytest.mark.parametrize("xdtype", ["f32", "bf16"])
+def test_gemv_extreme_activations_stay_in_their_token(xdtype):
+    """Largest, smallest and tiny activations keep the bound; an infinity and
+    a NaN make their own token's outputs non-finite and no other's."""
+    out, n_in, g, q = 130, 1024, 64, 3
+    planes, a_star, z_star = random_export(out, n_in, q, g, seed=3)
+    x = np.random.default_rng(1).standard_normal((6, n_in)).astype(F32)
+    x[1] *= F32(1e34)
+    x[2] *= F32(1e-30)
+    x[3, ::7] *= F32(1e12)
+    check(planes, a_star, z_star, x, g, xdtype, label="extreme")
+    x[4, 5], x[5, 77] = np.inf, np.nan
+    if xdtype == "bf16":
+        raw, _ = synth.bf16_round(np.where(np.isfinite(x), x, 0))
+        raw[4, 5], raw[5, 77] = 0x7F80, 0x7FC0
+        xd = api.weights_tensor(raw, C.dev())
+    else:
+        xd = torch.from_numpy(x).to(C.dev())
+    y = torch.empty(6, out, device=C.dev())
+    api.uq_bcq_gemv(torch.from_numpy(planes.view(np.int32)).to(C.dev()), torch.from_numpy(a_star).to(C.dev()),
+                    torch.from_numpy(z_star).to(C.dev()), xd, y, g)
+    assert torch.isfinite(y[:4]).all() and not torch.isfinite(y[4:]).any()
 
 
 def test_gemv_deterministic():
