@@ -147,6 +147,30 @@ def test_init_singular_gram_groups_match_the_oracle_bit_for_bit(q, g, clip):
     C.check_init(W, q, g, 7, clip, got, gc, ref, errs, chosen, f"singular q={q} g={g} clip={clip}")
 
 
+@pytest.mark.parametrize("q,g", [(1, 32), (2, 64), (3, 128), (4, 128), (3, 256)])
+def test_init_groups_outside_the_fast_paths(q, g):
+    """Groups whose sums are no integers of one scale (values over 12 decades),
+    whose squared errors leave fp32's range, one-sided groups, and groups of
+    two or three values (equal levels, far fewer values than levels), between
+    ordinary groups of the same warp."""
+    rng = np.random.default_rng(31 * q + g)
+    out, Gr = 7, 10
+    W = (rng.standard_t(4, (out, Gr, g)) * 0.014).astype(np.float32)
+    W[1] = np.exp(rng.uniform(np.log(1e-12), np.log(1.0), (Gr, g))) * rng.choice([-1.0, 1.0], (Gr, g))
+    W[2] *= 1e-24
+    W[3] *= 1e20
+    W[4] = np.abs(W[4]) + np.float32(1e-7)
+    W[5] = rng.choice(np.float32([-0.02, 0.01, 0.03]), (Gr, g))
+    W[6, :, 1:] = np.float32(0.005)
+    W = W.reshape(out, Gr * g).astype(np.float32)
+    p = api.empty_params(out, Gr * g, q, g, C.dev())
+    codes = torch.empty(out, Gr * g, dtype=torch.uint8, device=C.dev())
+    api.uq_init_params(torch.from_numpy(W).to(C.dev()), q, g, p, codes, G=9, T=6)
+    ref, errs, chosen = O.unified_init(W, q, g, G=9, T=6, return_errors=True)
+    got = {k: C.host(v) for k, v in p.items()}
+    C.check_init(W, q, g, 9, api.CLIP_FIXED_MIN, got, C.host(codes), ref, errs, chosen, f"outside q={q} g={g}")
+
+
 def test_edge_level_ties_negative_alpha_and_high_code_bits():
     """alpha_1 == alpha_2 makes two code words share a level (ties in the sort
     and in the mapping); a negative alpha reverses part of the order; code
