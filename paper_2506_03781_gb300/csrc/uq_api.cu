@@ -437,6 +437,11 @@ uq_status uq_check_device(void* stream) {
     if (e != cudaSuccess) return fail(UQ_ERR_CUDA, "uq_check_device: %s", cudaGetErrorString(e));
     unsigned int flag = 0, flag_step = 0, flag_omni = 0, flag_awq = 0, flag_gemv = 0;
     e = uq::stream_error(true, &flag);
+    for (auto more : {uq::ragged_fwd_error, uq::ragged_bwd_error}) {
+        unsigned int flag_ragged = 0;
+        if (e == cudaSuccess) e = more(true, &flag_ragged);
+        flag |= flag_ragged;
+    }
     if (e == cudaSuccess) e = uq::step_error(true, &flag_step);
     if (e == cudaSuccess) {
         unsigned int flag_step_bf16 = 0;

@@ -287,7 +287,7 @@ awq_stream_fwd_kernel(const void* __restrict__ W, const float* __restrict__ SA, 
     constexpr int L = 1 << Q, LPG = St::LPG, NG = St::NG, NV = St::NV, UE = St::UE, NST = St::NST;
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ __align__(8) unsigned long long bars[kWarps][NST];
-    __shared__ MapTab<Q, NG> tabs[kWarps];
+    __shared__ SortTab<Q, NG> tabs[kWarps];
     constexpr int NIV = MODE == FWD_REMAP ? NG : 1;              // remap intervals only on remap steps
     __shared__ float4 ivs[kWarps][NIV][L];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -295,7 +295,7 @@ awq_stream_fwd_kernel(const void* __restrict__ W, const float* __restrict__ SA, 
     const int U = n_in / UE, Gr = n_in / G_;
     const Items it(U, R, n_rb, warp);
     unsigned char* wsm = smem + (size_t)warp * St::WARP_BYTES;
-    MapTab<Q, NG>& t = tabs[warp];
+    SortTab<Q, NG>& t = tabs[warp];
 
     if (lane == 0) {
         for (int s = 0; s < NST; ++s) tma::bar_init(tma::smem_addr(&bars[warp][s]), 1);

@@ -1,6 +1,9 @@
 // Backward of the quantizer: straight-through estimator with gradient
 // filtering (App. C.1) through Eq. 3.
 //
+// The kernel here takes the groups of more than 512 elements and of 384; the
+// pipelined kernels of uq_stream.cu and uq_ragged_bwd.cu take every other g.
+//
 // Per element (NV vectors of 4 per lane and group, see uq_common.cuh):
 // recompute x = T_F(w) and m = l(code), filter f = |x - m| <= tau (fp32
 // decision), write ds = -(Delta G f u) / s.  Per group, with G = dL/dW^:
@@ -158,31 +161,21 @@ static cudaError_t run_bwd(const Shape& sh, const void* W, uq_params p, const ui
     return cudaGetLastError();
 }
 
-template <int Q, typename WT, bool ELEM>
-static cudaError_t bwd_gf(const Shape& sh, const void* W, uq_params p, const uint8_t* codes, const float* gup,
-                          uq_grads gr, cudaStream_t st) {
-    switch (lanes_per_group(sh.g)) {
-        case 4: return run_bwd<Q, WT, 4, ELEM>(sh, W, p, codes, gup, gr, st);
-        case 8: return run_bwd<Q, WT, 8, ELEM>(sh, W, p, codes, gup, gr, st);
-        case 16: return run_bwd<Q, WT, 16, ELEM>(sh, W, p, codes, gup, gr, st);
-        default: return run_bwd<Q, WT, 32, ELEM>(sh, W, p, codes, gup, gr, st);
-    }
-}
-
 template <int Q>
 static cudaError_t bwd_w(const Shape& sh, const void* W, uq_params p, const uint8_t* codes, const float* gup,
                          uq_grads gr, int filter, cudaStream_t st) {
     const bool elem = filter == UQ_FILTER_ELEMENT;
     if (sh.wdtype == UQ_W_BF16)
-        return elem ? bwd_gf<Q, WBF16, true>(sh, W, p, codes, gup, gr, st)
-                    : bwd_gf<Q, WBF16, false>(sh, W, p, codes, gup, gr, st);
-    return elem ? bwd_gf<Q, WF32, true>(sh, W, p, codes, gup, gr, st)
-                : bwd_gf<Q, WF32, false>(sh, W, p, codes, gup, gr, st);
+        return elem ? run_bwd<Q, WBF16, 32, true>(sh, W, p, codes, gup, gr, st)
+                    : run_bwd<Q, WBF16, 32, false>(sh, W, p, codes, gup, gr, st);
+    return elem ? run_bwd<Q, WF32, 32, true>(sh, W, p, codes, gup, gr, st)
+                : run_bwd<Q, WF32, 32, false>(sh, W, p, codes, gup, gr, st);
 }
 
 cudaError_t launch_bwd(const Shape& sh, const void* W, uq_params p, const uint8_t* codes, const float* gup,
                        uq_grads gr, cudaStream_t st, int filter) {
     if (stream_path_ok(sh)) return launch_bwd_stream(sh, W, p, codes, gup, gr, st, filter);
+    if (ragged_path_ok(sh)) return launch_bwd_ragged(sh, W, p, codes, gup, gr, st, filter);
     switch (sh.q) {
         case 1: return bwd_w<1>(sh, W, p, codes, gup, gr, filter, st);
         case 2: return bwd_w<2>(sh, W, p, codes, gup, gr, filter, st);

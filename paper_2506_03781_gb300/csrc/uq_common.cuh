@@ -110,13 +110,17 @@ struct LvTab {                       // levels by code word and tau per slot
 };
 
 template <int Q, int NS>
-struct MapTab {                      // + sorted order and local-mapping neighbours
+struct SortTab {                     // + sorted order
     static constexpr int L = 1 << Q;
-    float lv[NS][L];
+    alignas(16) float lv[NS][L];
     float srt[NS][L];
-    float4 nb[NS][L];
     uint8_t cor[NS][L];
     uint8_t rk[NS][L];
+};
+
+template <int Q, int NS>
+struct MapTab : SortTab<Q, NS> {     // + local-mapping neighbours
+    float4 nb[NS][1 << Q];
 };
 
 // Levels l(c) of the NS groups grp0 + k (k < n_ok), tau = min_j |alpha_j| and,
@@ -159,8 +163,8 @@ __device__ __forceinline__ void unit_levels(TAB& t, float* tau, int lane, const 
 
 // Sorted order (ascending, ties by code word) and, if NB, the neighbour
 // triples of the local mapping.  Requires t.lv; ends with __syncwarp().
-template <int Q, int NS, bool NB>
-__device__ __forceinline__ void unit_sort(MapTab<Q, NS>& t, int lane) {
+template <int Q, int NS, bool NB, typename TAB>
+__device__ __forceinline__ void unit_sort(TAB& t, int lane) {
     constexpr int L = 1 << Q;
     constexpr int E = NS * L;
 #pragma unroll
@@ -168,10 +172,20 @@ __device__ __forceinline__ void unit_sort(MapTab<Q, NS>& t, int lane) {
         const int k = e / L, c = e % L;
         const float v = t.lv[k][c];
         int r = 0;
+        if constexpr (L >= 4) {
 #pragma unroll
-        for (int c2 = 0; c2 < L; ++c2) {
-            const float v2 = t.lv[k][c2];
-            r += (v2 < v) || (v2 == v && c2 < c);
+            for (int c4 = 0; c4 < L; c4 += 4) {
+                float v4[4];
+                f4_to(*reinterpret_cast<const float4*>(&t.lv[k][c4]), v4);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) r += (v4[i] < v) || (v4[i] == v && c4 + i < c);
+            }
+        } else {
+#pragma unroll
+            for (int c2 = 0; c2 < L; ++c2) {
+                const float v2 = t.lv[k][c2];
+                r += (v2 < v) || (v2 == v && c2 < c);
+            }
         }
         t.srt[k][r] = v;
         t.cor[k][r] = static_cast<uint8_t>(c);
@@ -358,7 +372,7 @@ __device__ __forceinline__ void bwd_vec4(const float w[4], const float s4[4], co
 // a NaN (all comparisons false) -- takes the exact path: transform_x and
 // the three distances.
 template <int Q, int NS>
-__device__ __forceinline__ void unit_remap_iv(const MapTab<Q, NS>& t, float4 (*iv)[1 << Q], int lane,
+__device__ __forceinline__ void unit_remap_iv(const SortTab<Q, NS>& t, float4 (*iv)[1 << Q], int lane,
                                               const float* pd, const float* pz) {
     constexpr int L = 1 << Q;
     constexpr int E = NS * L;
@@ -387,7 +401,7 @@ __device__ __forceinline__ void unit_remap_iv(const MapTab<Q, NS>& t, float4 (*i
 // Every lane of the warp must call it (the fallback verdicts are warp-wide).
 template <int Q, int NS>
 __device__ __forceinline__ uint32_t remap_vec4(const float w[4], const float s4[4], uint32_t cv,
-                                               const MapTab<Q, NS>& t, const float4 (*iv)[1 << Q], int sub,
+                                               const SortTab<Q, NS>& t, const float4 (*iv)[1 << Q], int sub,
                                                float dl, float sr, float zu, float o[4]) {
     constexpr int L = 1 << Q;
     uint32_t nc = 0;
@@ -417,6 +431,115 @@ __device__ __forceinline__ uint32_t remap_vec4(const float w[4], const float s4[
             const float dhi = fabsf(__fsub_rn(x, hi));
             if (dhi < best) { m = hi; code = t.cor[sub][rh]; }
             o[kq] = __fmul_rn(dl, __fsub_rn(m, zu));
+        }
+        nc |= code << (8 * kq);
+    }
+    return nc;
+}
+
+// Full mapping M_B from the reciprocal, with a proof: a search over the
+// midpoints th of the sorted levels finds the rank r of x' (formed as above):
+// every fourth midpoint from registers, then one 16-byte load of the three
+// between two of those.  The rank only has to be right where
+// iv[r] = (a, b, w^, code) confirms it, as in the remap: x' in (a, b) puts the IEEE
+// x more than m / 2 beyond the midpoints to the next lower and the next higher
+// distinct level (m as above).  The scan of the exact path takes the lowest
+// rank among equal distances, so against a lower level the distances have to
+// stay different after rounding: between the levels they differ by more than
+// m; above l_r by the gap of the two, which must exceed 2^-20 of the
+// distances -- that gap is at least 2^-20 M for the ranks below the top (|x| <=
+// M there), and at the top b caps x at 2^20 gaps; where this fails a = +inf
+// sends every element to the exact path.  Equal levels share the lowest one's
+// interval, W^ and code, whichever of their ranks the search finds.
+// groups k >= ng get an interval nothing lies in.
+template <int Q, int NS>
+__device__ __forceinline__ void unit_full_iv(const SortTab<Q, NS>& t, float4 (*iv)[1 << Q], float (*th)[1 << Q], int lane,
+                                             const float* pd, const float* pz, int ng) {
+    constexpr int L = 1 << Q;
+    constexpr int E = NS * L;
+    const float inf = __int_as_float(0x7f800000);
+#pragma unroll
+    for (int e = lane; e < E; e += 32) {
+        const int k = e / L, r = e % L;
+        if (k >= ng) {
+            iv[k][r] = make_float4(inf, -inf, 0.f, 0.f);
+            th[k][r] = 0.f;
+            continue;
+        }
+        const float y = t.srt[k][r], zu = pz[k];
+        th[k][r] = r < L - 1 ? __fmul_rn(0.5f, __fadd_rn(y, t.srt[k][r + 1])) : inf;
+        int lo = r, hi = r;                                   // lowest and highest rank of this level
+        while (lo > 0 && t.srt[k][lo - 1] == y) --lo;
+        while (hi < L - 1 && t.srt[k][hi + 1] == y) ++hi;
+        const float M = fmaxf(fabsf(t.srt[k][0]), fabsf(t.srt[k][L - 1]));
+        const float base = __fadd_rn(fabsf(zu), M);
+        float a = -inf, b = inf;
+        if (lo > 0) {
+            const float p = t.srt[k][lo - 1], mid = __fmul_rn(0.5f, __fadd_rn(p, y)), gap = __fsub_rn(y, p);
+            a = gap > __fmul_rn(M, 0x1p-20f) ? __fadd_rn(mid, __fmaf_rn(__fadd_rn(fabsf(mid), base), 0x1p-18f, 0x1p-126f)) : inf;
+            b = __fmul_rn(gap, 0x1p20f);
+        }
+        if (hi < L - 1) {
+            const float mid = __fmul_rn(0.5f, __fadd_rn(y, t.srt[k][hi + 1]));
+            b = __fsub_rn(mid, __fmaf_rn(__fadd_rn(fabsf(mid), base), 0x1p-18f, 0x1p-126f));
+        }
+        iv[k][r] = make_float4(a, b, __fmul_rn(pd[k], __fsub_rn(y, zu)), __uint_as_float((uint32_t)t.cor[k][lo]));
+    }
+    __syncwarp();
+}
+
+// Every fourth midpoint of a group (none for L <= 4).
+template <int L>
+struct FullKeys {
+    float k[L > 4 ? L / 4 - 1 : 1];
+    __device__ __forceinline__ void load(const float* th) {
+#pragma unroll
+        for (int i = 0; i + 1 < L / 4; ++i) k[i] = th[4 * i + 3];
+    }
+};
+
+// Full mapping of 4 consecutive elements of group slot `sub`: W^ into o[],
+// returns the 4 code words packed as bytes.
+template <int Q, int NS>
+__device__ __forceinline__ uint32_t full_vec4(const float w[4], const float s4[4], const SortTab<Q, NS>& t,
+                                              const float4 (*iv)[1 << Q], const float (*th)[1 << Q],
+                                              const FullKeys<(1 << Q)>& keys, int sub, float dl, float sr, float zu,
+                                              float o[4]) {
+    constexpr int L = 1 << Q;
+    uint32_t nc = 0;
+#pragma unroll
+    for (int kq = 0; kq < 4; ++kq) {
+        const float den = __fmul_rn(__fmul_rn(dl, s4[kq]), sr);
+        const float xa = __fadd_rn(__fmul_rn(w[kq], rcp_approx(den)), zu);
+        int r = 0;
+        if constexpr (L == 16) {
+            const bool h = xa > keys.k[1];
+            r = (h ? 8 : 0) + (xa > (h ? keys.k[2] : keys.k[0]) ? 4 : 0);
+        } else if constexpr (L == 8) {
+            r = xa > keys.k[0] ? 4 : 0;
+        }
+        if constexpr (L >= 4) {
+            const float4 m = *reinterpret_cast<const float4*>(&th[sub][r]);
+            const bool h = xa > m.y;
+            r += (h ? 2 : 0) + (xa > (h ? m.z : m.x) ? 1 : 0);
+        } else {
+            r = xa > th[sub][0] ? 1 : 0;
+        }
+        const float4 v = iv[sub][r];
+        o[kq] = v.z;
+        uint32_t code = __float_as_uint(v.w);
+        if (!((xa > v.x) & (xa < v.y) & (fabsf(den) < 0x1p125f))) {
+            float uu, m = t.srt[sub][0];
+            const float x = transform_x(w[kq], s4[kq], dl, sr, zu, uu);
+            float best = fabsf(__fsub_rn(x, m));
+            int br = 0;
+#pragma unroll 1
+            for (int k = 1; k < L; ++k) {
+                const float l = t.srt[sub][k], d = fabsf(__fsub_rn(x, l));
+                if (d < best) { best = d; br = k; m = l; }
+            }
+            o[kq] = __fmul_rn(dl, __fsub_rn(m, zu));
+            code = t.cor[sub][br];
         }
         nc |= code << (8 * kq);
     }

@@ -37,6 +37,17 @@ cudaError_t launch_fwd_stream(const Shape& sh, const void* W, uq_params p, uint8
                               float* what, cudaStream_t st);
 cudaError_t launch_bwd_stream(const Shape& sh, const void* W, uq_params p, const uint8_t* codes,
                               const float* gup, uq_grads gr, cudaStream_t st, int filter = UQ_FILTER_STE);
+// The same pipelines for rows that are no whole number of units and for g =
+// 256, 512 (uq_ragged_fwd.cu, uq_ragged_bwd.cu), and their bounded-wait flags.
+inline bool ragged_path_ok(const Shape& sh) {
+    return sh.g == 32 || sh.g == 64 || sh.g == 128 || sh.g == 256 || sh.g == 512;
+}
+cudaError_t launch_fwd_ragged(const Shape& sh, const void* W, uq_params p, uint8_t* codes, int mode, float* what,
+                              cudaStream_t st);
+cudaError_t launch_bwd_ragged(const Shape& sh, const void* W, uq_params p, const uint8_t* codes, const float* gup,
+                              uq_grads gr, cudaStream_t st, int filter);
+cudaError_t ragged_fwd_error(bool clear, unsigned int* flag);
+cudaError_t ragged_bwd_error(bool clear, unsigned int* flag);
 // Fused optimisation step (uq_step.cu): backward of step t, SGD update,
 // forward of step t + 1 in `mode` (a FWD_* value).  step_path_ok tells
 // whether the shape is one the fused kernel handles.

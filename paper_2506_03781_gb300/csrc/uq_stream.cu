@@ -283,15 +283,15 @@ fwd_stream_kernel(const void* __restrict__ W, const float* __restrict__ S, const
     constexpr int L = 1 << Q, LPG = St::LPG, NG = St::NG, NV = St::NV, UE = St::UE, NST = St::NST;
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ __align__(8) unsigned long long bars[kWarps][NST];
-    __shared__ MapTab<Q, NG> tabs[kWarps];
-    constexpr int NIV = mode == FWD_REMAP ? NG : 1;              // remap intervals only on remap steps
-    __shared__ float4 ivs[kWarps][NIV][L];
+    __shared__ SortTab<Q, NG> tabs[kWarps];
+    __shared__ float4 ivs[kWarps][NG][L];                        // intervals of the remap or of the full mapping
+    __shared__ __align__(16) float ths[kWarps][mode == FWD_FULL ? NG : 1][L];      // midpoints of the full mapping
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int sub = lane / LPG, li = lane % LPG;
     const int U = n_in / UE, Gr = n_in / G_;
     const Items it(U, R, n_rb, warp);
     unsigned char* wsm = smem + (size_t)warp * St::WARP_BYTES;
-    MapTab<Q, NG>& t = tabs[warp];
+    SortTab<Q, NG>& t = tabs[warp];
     constexpr uint32_t TX = St::TX;
 
     if (lane == 0) {
@@ -341,15 +341,13 @@ fwd_stream_kernel(const void* __restrict__ W, const float* __restrict__ S, const
                 unit_remap_iv<Q, NG>(t, ivs[warp], lane, pd, pz);
             } else if constexpr (mode == FWD_FULL) {
                 unit_sort<Q, NG, false>(t, lane);
+                unit_full_iv<Q, NG>(t, ivs[warp], ths[warp], lane, pd, pz, NG);
             }
             const float dl = pd[sub], zu = pz[sub];
             const float sr = __ldg(SR + row);
             const int64_t ebase = row * n_in + (int64_t)it.unit(cc.j) * UE;
-            float srt[L];
-            if constexpr (mode == FWD_FULL) {
-#pragma unroll
-                for (int r = 0; r < L; ++r) srt[r] = t.srt[sub][r];
-            }
+            FullKeys<L> keys;
+            if constexpr (mode == FWD_FULL) keys.load(ths[warp][sub]);
 #pragma unroll
             for (int v = 0; v < NV; ++v) {
                 const int el = sub * G_ + 4 * li + 4 * LPG * v;
@@ -364,14 +362,7 @@ fwd_stream_kernel(const void* __restrict__ W, const float* __restrict__ S, const
                     if constexpr (mode == FWD_REMAP) {
                         nc = remap_vec4<Q, NG>(w, s4, cv, t, ivs[warp], sub, dl, sr, zu, o);
                     } else {
-#pragma unroll
-                        for (int kq = 0; kq < 4; ++kq) {
-                            float uu, m;
-                            const float x = transform_x(w[kq], s4[kq], dl, sr, zu, uu);
-                            const int r = nearest_rank<L>(x, srt, m);
-                            o[kq] = __fmul_rn(dl, __fsub_rn(m, zu));
-                            nc |= uint32_t(t.cor[sub][r]) << (8 * kq);
-                        }
+                        nc = full_vec4<Q, NG>(w, s4, t, ivs[warp], ths[warp], keys, sub, dl, sr, zu, o);
                     }
                     *reinterpret_cast<uint32_t*>(CODES + ebase + el) = nc;
                 }

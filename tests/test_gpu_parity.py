@@ -246,6 +246,46 @@ def test_remap_near_level_midpoints_is_bit_exact(q, g, n_in):
     assert (r_codes != codes0).mean() > 0.05         # many decisions go to the neighbour
 
 
+@pytest.mark.parametrize("q,g,n_in", [(1, 32, 1024), (2, 64, 1024), (3, 128, 2048), (4, 128, 1024), (4, 64, 1024),
+                                      (3, 256, 1024), (4, 128, 640), (2, 32, 352)])
+def test_full_mapping_near_level_midpoints_and_equal_levels_is_bit_exact(q, g, n_in):
+    """Full mapping of elements within 4 ulps of the midpoints, in groups of
+    which some have equal levels (two equal alpha, one zero alpha), levels a
+    few ulps apart (the distances round to equal values far from them: the
+    lower rank wins) and weights far outside the levels."""
+    out = 12
+    _, W0, P, codes0, _ = C.make_inputs(out, n_in, q, g, seed=900 + 10 * q + g, wdtype="f32")
+    if q > 1:
+        P["alpha"][1::4, :, 1] = P["alpha"][1::4, :, 0]
+        P["alpha"][2::4, :, 0] = 0.0
+        P["alpha"][3::4, :, 0] = P["alpha"][3::4, :, 1] * np.float32(2.0 ** -22)
+    W = C.midpoint_weights(P, codes0, g, seed=q + g)
+    W[::3, ::5] *= np.float32(1e6)
+    what, codes = C.gpu_fwd(W, P, None, q, g, api.MAP_FULL, 0, 2)
+    r_what, r_codes = O.quantize_fwd(W, P["s"], P["sr"], P["delta"], P["zu"], P["alpha"], P["zb"], None, g, O.MAP_FULL)
+    C.assert_fwd_equal(what, codes, r_what, r_codes, f"full midpoints q={q} g={g} in={n_in}")
+
+
+# rows that are no whole number of work units: one group, remainders 1..3 of the 16-byte parameter pieces for
+# every g and q, the last row's groups that no whole piece covers, and the larger groups
+@pytest.mark.parametrize("out,n_in,g", [(1, 32, 32), (3, 32 * 11, 32), (5, 64 * 13, 64), (2, 128, 128), (9, 128 * 7, 128),
+                                        (4, 128 * 86, 128), (3, 256 * 3, 256), (1, 256, 256), (2, 512 * 3, 512),
+                                        (1, 512, 512), (300, 64 * 3, 64)])
+@pytest.mark.parametrize("q,wd", [(1, "bf16"), (2, "f32"), (3, "bf16"), (4, "f32")])
+def test_rows_of_partial_units(out, n_in, g, q, wd):
+    raw, W, P, codes0, Gup = C.make_inputs(out, n_in, q, g, seed=out + n_in + q, wdtype=wd, init_G=3, init_T=2)
+    args = (P["s"], P["sr"], P["delta"], P["zu"], P["alpha"], P["zb"])
+    for mode, step in ((api.MAP_FULL, 0), (api.MAP_LOCAL_PERIODIC, 0), (api.MAP_LOCAL_PERIODIC, 1)):
+        what, codes = C.gpu_fwd(raw, P, codes0, q, g, mode, step, 2)
+        r_what, r_codes = O.quantize_fwd(W, *args, None if mode == api.MAP_FULL else codes0, g,
+                                         O.MAP_FULL if mode == api.MAP_FULL else O.MAP_LOCAL_PERIODIC, step, 2)
+        C.assert_fwd_equal(what, codes, r_what, r_codes, f"{out}x{n_in} g{g} q{q} mode {mode} step {step}")
+    gr = C.gpu_bwd(raw, P, codes0, Gup, q, g)
+    ref, mass = C.oracle_bwd(W, P, codes0, Gup, g)
+    C.assert_grads_close(gr, ref, mass, f"{out}x{n_in} g{g} q{q}")
+    api.uq_check_device()
+
+
 def test_deterministic_and_in_bounds():
     """Two identical calls give identical bits; outputs written into the middle
     of larger buffers leave the sentinel margins untouched."""
