@@ -149,7 +149,23 @@ def uq_check_device(stream=None, device=None):
 # marshalling helpers
 # ---------------------------------------------------------------------------
 
+# The current device and a device's current stream, without the Stream and
+# device objects that torch.cuda builds on every call (a call on a small matrix
+# is shorter than its marshalling).
+_current_device = torch._C._cuda_getDevice
+_current_raw_stream = torch._C._cuda_getCurrentRawStream
+
+
 def _check(t, name, shape, dtype, device):
+    # one pass for a tensor that is as it should be; _refuse says what is wrong with any other
+    if (t.__class__ is torch.Tensor and t.is_cuda and t.dtype is dtype and t.shape == shape and t.is_contiguous()
+            and t.device == device and device.index == _current_device()):
+        return t.data_ptr()
+    return _refuse(t, name, shape, dtype, device)
+
+
+def _refuse(t, name, shape, dtype, device):
+    """The checks one by one, each with its message (subclasses of Tensor and device=None pass here too)."""
     if not isinstance(t, torch.Tensor):
         raise TypeError(f"{name} must be a torch.Tensor")
     if t.device.type != "cuda" or (device is not None and t.device != device):
@@ -176,24 +192,39 @@ def _wdtype(W):
 
 def _stream(stream, device):
     if stream is None:
-        return torch.cuda.current_stream(device).cuda_stream
+        return _current_raw_stream(device.index)
     if isinstance(stream, torch.cuda.Stream):
         return stream.cuda_stream
     return int(stream)
 
 
+_PARAM_LABELS = tuple(f"params['{n}']" for n in PARAM_NAMES)
+_GRAD_LABELS = tuple(f"grads['{n}']" for n in GRAD_NAMES)
+_OMNI_LABELS, _AWQ_LABELS = (tuple(f"params['{n}']" for n in names) for names in (OMNI_PARAM_NAMES, AWQ_PARAM_NAMES))
+_OMNI_GRAD_LABELS, _AWQ_GRAD_LABELS = (tuple(f"grads['{n}']" for n in names) for names in (OMNI_GRAD_NAMES, AWQ_GRAD_NAMES))
+
+
+def _fields(d, names, labels, shapes, device):
+    return [_check(d[n], label, shape, torch.float32, device) for n, label, shape in zip(names, labels, shapes)]
+
+
 def _params(p, out, n_in, q, g, device, need=PARAM_NAMES):
     Gr = n_in // g
-    shapes = {"delta": (out, Gr), "zu": (out, Gr), "s": (out, n_in), "sr": (out,),
-              "alpha": (out, Gr, q), "zb": (out, Gr)}
-    ptrs = {}
-    for n in PARAM_NAMES:
-        if n in need:
-            ptrs[n] = _check(p[n], f"params['{n}']", shapes[n], torch.float32, device)
-        else:
-            t = p.get(n) if p is not None else None
-            ptrs[n] = _check(t, f"params['{n}']", shapes[n], torch.float32, device) if t is not None else None
-    return uq_params(**ptrs)
+    grp = (out, Gr)
+    shapes = (grp, grp, (out, n_in), (out,), (out, Gr, q), grp)
+    if need is PARAM_NAMES:
+        return uq_params(*_fields(p, PARAM_NAMES, _PARAM_LABELS, shapes, device))
+    ptrs = []
+    for n, label, shape in zip(PARAM_NAMES, _PARAM_LABELS, shapes):
+        t = p[n] if n in need else (p.get(n) if p is not None else None)
+        ptrs.append(_check(t, label, shape, torch.float32, device) if n in need or t is not None else None)
+    return uq_params(*ptrs)
+
+
+def _grads(gr, out, n_in, q, g, device):
+    Gr = n_in // g if g > 0 and n_in % g == 0 else 0
+    grp = (out, Gr)
+    return uq_grads(*_fields(gr, GRAD_NAMES, _GRAD_LABELS, (grp, grp, (out, n_in), (out,), (out, Gr, q), grp), device))
 
 
 def _raise(status):
@@ -247,10 +278,7 @@ def uq_quantize_bwd(W, q, g, params, codes, dL_dWhat, grads, stream=None):
     """Backward (App. C.1 STE with gradient filtering); overwrites every tensor of ``grads``."""
     out, n_in = _dims(W, g)
     dev = W.device
-    Gr = n_in // g if g > 0 and n_in % g == 0 else 0
-    shapes = {"ddelta": (out, Gr), "dzu": (out, Gr), "ds": (out, n_in), "dsr": (out,),
-              "dalpha": (out, Gr, q), "dzb": (out, Gr)}
-    gp = uq_grads(**{n: _check(grads[n], f"grads['{n}']", shapes[n], torch.float32, dev) for n in GRAD_NAMES})
+    gp = _grads(grads, out, n_in, q, g, dev)
     st = lib().uq_quantize_bwd(
         W.data_ptr(), _wdtype(W), out, n_in, q, g, _params(params, out, n_in, q, g, dev),
         _check(codes, "codes", (out, n_in), torch.uint8, dev),
@@ -292,10 +320,7 @@ def uq_quantize_bwd_ex(W, q, g, params, codes, dL_dWhat, grads, filter=FILTER_ST
     """uq_quantize_bwd with a choice of gradient filter (FILTER_STE or FILTER_ELEMENT)."""
     out, n_in = _dims(W, g)
     dev = W.device
-    Gr = n_in // g if g > 0 and n_in % g == 0 else 0
-    shapes = {"ddelta": (out, Gr), "dzu": (out, Gr), "ds": (out, n_in), "dsr": (out,),
-              "dalpha": (out, Gr, q), "dzb": (out, Gr)}
-    gp = uq_grads(**{n: _check(grads[n], f"grads['{n}']", shapes[n], torch.float32, dev) for n in GRAD_NAMES})
+    gp = _grads(grads, out, n_in, q, g, dev)
     st = lib().uq_quantize_bwd_ex(
         W.data_ptr(), _wdtype(W), out, n_in, q, g, _params(params, out, n_in, q, g, dev),
         _check(codes, "codes", (out, n_in), torch.uint8, dev),
@@ -343,9 +368,8 @@ def uq_export_bcq(W, q, g, params, codes, bitplanes, alpha_star, zb_star, mode=E
 
 def _omni_params(p, out, n_in, q, g, device):
     Gr = n_in // g if g > 0 and n_in % g == 0 else 0
-    shapes = {"beta": (out, Gr), "gamma": (out, Gr), "alpha": (out, Gr, q), "zb": (out, Gr)}
-    return uq_params_omni(**{n: _check(p[n], f"params['{n}']", shapes[n], torch.float32, device)
-                             for n in OMNI_PARAM_NAMES})
+    grp = (out, Gr)
+    return uq_params_omni(*_fields(p, OMNI_PARAM_NAMES, _OMNI_LABELS, (grp, grp, (out, Gr, q), grp), device))
 
 
 def uq_quantize_fwd_omni(W, q, g, params, codes, W_hat, map_mode=MAP_LOCAL_PERIODIC, step=0, p_period=2,
@@ -365,9 +389,8 @@ def uq_quantize_bwd_omni(W, q, g, params, codes, dL_dWhat, grads, stream=None):
     out, n_in = _dims(W, g)
     dev = W.device
     Gr = n_in // g if g > 0 and n_in % g == 0 else 0
-    shapes = {"dbeta": (out, Gr), "dgamma": (out, Gr), "dalpha": (out, Gr, q), "dzb": (out, Gr)}
-    gp = uq_grads_omni(**{n: _check(grads[n], f"grads['{n}']", shapes[n], torch.float32, dev)
-                          for n in OMNI_GRAD_NAMES})
+    gp = uq_grads_omni(*_fields(grads, OMNI_GRAD_NAMES, _OMNI_GRAD_LABELS,
+                                ((out, Gr), (out, Gr), (out, Gr, q), (out, Gr)), dev))
     st = lib().uq_quantize_bwd_omni(
         W.data_ptr(), _wdtype(W), out, n_in, q, g, _omni_params(params, out, n_in, q, g, dev),
         _check(codes, "codes", (out, n_in), torch.uint8, dev),
@@ -387,11 +410,10 @@ def uq_omni_scales(W, q, g, beta, gamma, delta, zo, stream=None):
     _raise(st)
 
 
-def _awq_params(p, out, n_in, q, g, device, need=AWQ_PARAM_NAMES):
+def _awq_params(p, out, n_in, q, g, device):
     Gr = n_in // g if g > 0 and n_in % g == 0 else 0
-    shapes = {"sa": (n_in,), "delta": (out, Gr), "za": (out, Gr), "alpha": (out, Gr, q), "zb": (out, Gr)}
-    return uq_params_awq(**{n: _check(p[n], f"params['{n}']", shapes[n], torch.float32, device)
-                            for n in AWQ_PARAM_NAMES})
+    grp = (out, Gr)
+    return uq_params_awq(*_fields(p, AWQ_PARAM_NAMES, _AWQ_LABELS, ((n_in,), grp, grp, (out, Gr, q), grp), device))
 
 
 def uq_quantize_fwd_awq(W, q, g, params, codes, W_hat, map_mode=MAP_LOCAL_PERIODIC, step=0, p_period=2,
@@ -416,9 +438,8 @@ def uq_quantize_bwd_awq(W, q, g, params, codes, dL_dWhat, grads, workspace=None,
     out, n_in = _dims(W, g)
     dev = W.device
     Gr = n_in // g if g > 0 and n_in % g == 0 else 0
-    shapes = {"dsa": (n_in,), "ddelta": (out, Gr), "dza": (out, Gr), "dalpha": (out, Gr, q), "dzb": (out, Gr)}
-    gp = uq_grads_awq(**{n: _check(grads[n], f"grads['{n}']", shapes[n], torch.float32, dev)
-                         for n in AWQ_GRAD_NAMES})
+    gp = uq_grads_awq(*_fields(grads, AWQ_GRAD_NAMES, _AWQ_GRAD_LABELS,
+                               ((n_in,), (out, Gr), (out, Gr), (out, Gr, q), (out, Gr)), dev))
     if workspace is None:
         nbytes = uq_awq_bwd_workspace_bytes(out, n_in, q, g)
         workspace = torch.empty(max(nbytes // 4, 4), dtype=torch.float32, device=dev)
@@ -737,17 +758,13 @@ class Quantizer:
         self.codes = _check(codes, "codes", (self.out, self.n_in), torch.uint8, dev)
         self.what = _check(W_hat, "W_hat", (self.out, self.n_in), torch.float32, dev)
         self.G = _check(dL_dWhat, "dL_dWhat", (self.out, self.n_in), torch.float32, dev)
-        Gr = self.n_in // g
-        shapes = {"ddelta": (self.out, Gr), "dzu": (self.out, Gr), "ds": (self.out, self.n_in),
-                  "dsr": (self.out,), "dalpha": (self.out, Gr, q), "dzb": (self.out, Gr)}
         # grads may be None when only the fused train_step is used (it writes no gradients)
-        self.gr = None if grads is None else uq_grads(
-            **{n: _check(grads[n], f"grads['{n}']", shapes[n], torch.float32, dev) for n in GRAD_NAMES})
+        self.gr = None if grads is None else _grads(grads, self.out, self.n_in, q, g, dev)
         self.wptr = W.data_ptr()
         self.L = lib()
 
     def _st(self, stream):
-        if self.device.index != torch.cuda.current_device():
+        if self.device.index != _current_device():
             raise ValueError(f"this Quantizer's tensors are on {self.device} but the current device is "
                              f"cuda:{torch.cuda.current_device()} (call it under torch.cuda.device(...))")
         return _stream(stream, self.device)

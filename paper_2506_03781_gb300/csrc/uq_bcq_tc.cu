@@ -560,7 +560,7 @@ TcPlan tc_plan(int64_t out, int n_in, int chunks, bool staged) {
     for (int w = 1; w <= tc_groups(GB, N); ++w) {
         const int fit = (kTcSmem - 1024 - (staged ? w * kTcStages * tc_stage_bytes(Q, N) : 0)) / tc_pass_bytes(GB, N);
         const int least = (n_sb + fit - 1) / fit;
-        for (int ks = least; ks <= most_ks && ks < least + 16; ++ks) {
+        for (int ks = least; ks <= most_ks && ks < least + 8; ++ks) {
             const int per = (n_sb + ks - 1) / ks, n_ks = (n_sb + per - 1) / per;
             for (int waves = 1; waves <= 2; ++waves) {
                 int64_t n_rb = (int64_t)sms * waves / ((int64_t)n_ks * chunks);

@@ -888,7 +888,9 @@ static cudaError_t gemv_blocks_per_sm(KERN kern, size_t smem, int& per_sm, int t
 
 // Row blocks (of whole 8-row batches): the count that minimises
 // waves x (one table build, worth about 32 rows, + rows per block), where
-// a wave is one block per resident slot.
+// a wave is one block per resident slot.  For a number of waves that is the
+// largest count it holds; up to 8 waves are compared (a scan of every count
+// took 15 us of host time on a call whose kernels take 9.5).
 static void gemv_row_blocks(int64_t out, int n_tiles, int per_sm, int64_t& n_rb, int64_t& rpb,
                             double table_rows = 32.0) {
     const int64_t slots = (int64_t)sm_count() * per_sm;
@@ -896,14 +898,16 @@ static void gemv_row_blocks(int64_t out, int n_tiles, int per_sm, int64_t& n_rb,
     n_rb = 1;
     rpb = max_rb * kBatchRows;
     double best = -1.0;
-    const int64_t lim = max_rb < 8 * slots ? max_rb : 8 * slots;
-    for (int64_t cand = 1; cand <= lim; ++cand) {
+    for (int w = 1; w <= 8; ++w) {
+        int64_t cand = slots * w / n_tiles;
+        cand = cand < 1 ? 1 : cand > max_rb ? max_rb : cand;
         int64_t r = (out + cand - 1) / cand;
         r = (r + kBatchRows - 1) / kBatchRows * kBatchRows;
         const int64_t nb = (out + r - 1) / r;
         const int64_t waves = (nb * n_tiles + slots - 1) / slots;
         const double cost = (double)waves * (table_rows + (double)r);
         if (best < 0.0 || cost < best) { best = cost; n_rb = nb; rpb = r; }
+        if (cand == max_rb) break;
     }
 }
 
