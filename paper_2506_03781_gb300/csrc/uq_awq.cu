@@ -35,6 +35,8 @@ awq_fwd_kernel(const void* __restrict__ W, const float* __restrict__ SA, const f
                const float* __restrict__ ZA, const float* __restrict__ ALPHA, const float* __restrict__ ZB,
                uint8_t* __restrict__ CODES, float* __restrict__ WHAT, int64_t out, int n_in, int g,
                int64_t rows_per_range) {
+    dependents_may_start();
+    inputs_ready();
     constexpr int L = 1 << Q;
     constexpr int NG = 32 / LPG;
     __shared__ MapTab<Q, NG> tabs[kWarps];
@@ -125,6 +127,8 @@ awq_bwd_kernel(const void* __restrict__ W, const float* __restrict__ SA, const f
                const uint8_t* __restrict__ CODES, const float* __restrict__ GUP, float* __restrict__ DDELTA,
                float* __restrict__ DZA, float* __restrict__ DALPHA, float* __restrict__ DZB,
                float* __restrict__ PART, int64_t out, int n_in, int g, int64_t rows_per_range) {
+    dependents_may_start();
+    inputs_ready();
     constexpr int L = 1 << Q;
     constexpr int NG = 32 / LPG;
     using SR8 = SegReduce<LPG>;
@@ -283,6 +287,7 @@ __global__ void __launch_bounds__(kThreads, 3)
 awq_stream_fwd_kernel(const void* __restrict__ W, const float* __restrict__ SA, const float* __restrict__ DELTA,
                       const float* __restrict__ ZA, const float* __restrict__ ALPHA, const float* __restrict__ ZB,
                       uint8_t* __restrict__ CODES, float* __restrict__ WHAT, int64_t out, int n_in, int R, int n_rb) {
+    dependents_may_start();
     using St = AwqFwdStage<Q, WT, G_, MODE>;
     constexpr int L = 1 << Q, LPG = St::LPG, NG = St::NG, NV = St::NV, UE = St::UE, NST = St::NST;
     extern __shared__ __align__(128) unsigned char smem[];
@@ -302,6 +307,7 @@ awq_stream_fwd_kernel(const void* __restrict__ W, const float* __restrict__ SA, 
         tma::bar_init_fence();
     }
     __syncwarp();
+    inputs_ready();
     auto issue = [&](const Cursor& c, int s) {          // lane 0 only
         awq_issue<Q, St>(it, c, s, tma::smem_addr(&bars[warp][s]), wsm, W, SA, CODES, DELTA, ZA, ZB, ALPHA, out, n_in,
                          Gr);
@@ -395,8 +401,7 @@ static cudaError_t run_awq_stream_fwd(const Shape& sh, const void* W, uq_params_
     int grid = 0;
     cudaError_t e = grid_for<AwqTag<St, MODE>>(kern, dyn, n_rb, grid);
     if (e != cudaSuccess) return e;
-    kern<<<grid, kThreads, dyn, st>>>(W, p.sa, p.delta, p.za, p.alpha, p.zb, codes, what, sh.out, sh.n_in, R, n_rb);
-    return cudaGetLastError();
+    return launch_dependent(kern, grid, kThreads, dyn, st, W, p.sa, p.delta, p.za, p.alpha, p.zb, codes, what, sh.out, sh.n_in, R, n_rb);
 }
 
 template <int Q, typename WT, int G_>
@@ -480,6 +485,7 @@ awq_stream_bwd_kernel(const void* __restrict__ W, const float* __restrict__ SA, 
                       const uint8_t* __restrict__ CODES, const float* __restrict__ GUP, float* __restrict__ DDELTA,
                       float* __restrict__ DZA, float* __restrict__ DALPHA, float* __restrict__ DZB,
                       float* __restrict__ PART, int64_t out, int n_in, int R, int n_rb) {
+    dependents_may_start();
     using St = AwqBwdStage<Q, WT, G_>;
     constexpr int L = 1 << Q, LPG = St::LPG, NG = St::NG, NV = St::NV, UE = St::UE, NST = St::NST;
     using SR8 = SegReduce<LPG>;
@@ -497,6 +503,7 @@ awq_stream_bwd_kernel(const void* __restrict__ W, const float* __restrict__ SA, 
         tma::bar_init_fence();
     }
     __syncwarp();
+    inputs_ready();
     auto issue = [&](const Cursor& c, int s) {          // lane 0 only
         awq_bwd_issue<Q, St>(it, c, s, tma::smem_addr(&bars[warp][s]), wsm, W, SA, GUP, CODES, DELTA, ZA, ZB, ALPHA,
                              out, n_in, Gr);
@@ -635,6 +642,8 @@ cudaError_t awq_error(bool clear, unsigned int* flag) {
 constexpr int kColsumSlices = 8;
 __global__ void __launch_bounds__(32 * kColsumSlices)
 awq_colsum_kernel(const float* __restrict__ PART, float* __restrict__ DSA, int n_in, int ranges) {
+    dependents_may_start();
+    inputs_ready();
     __shared__ float part[kColsumSlices][32];
     const int lane = threadIdx.x & 31, slice = threadIdx.x >> 5;
     const int c = blockIdx.x * 32 + lane;
@@ -690,12 +699,10 @@ static cudaError_t run_awq_stream_bwd(const Shape& sh, const void* W, uq_params_
     auto kern = awq_stream_bwd_kernel<Q, WT, G_>;
     cudaError_t e = grid_for<AwqTag<St, 9>>(kern, dyn, n_rb, unused);    // shared-memory attribute (once)
     if (e != cudaSuccess) return e;
-    kern<<<grid, kThreads, dyn, st>>>(W, p.sa, p.delta, p.za, p.alpha, p.zb, codes, gup, gr.ddelta, gr.dza,
+    e = launch_dependent(kern, grid, kThreads, dyn, st, W, p.sa, p.delta, p.za, p.alpha, p.zb, codes, gup, gr.ddelta, gr.dza,
                                       gr.dalpha, gr.dzb, work, sh.out, sh.n_in, R, n_rb);
-    e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    awq_colsum_kernel<<<(sh.n_in + 31) / 32, 32 * kColsumSlices, 0, st>>>(work, gr.dsa, sh.n_in, grid * R);
-    return cudaGetLastError();
+    return launch_dependent(awq_colsum_kernel, (sh.n_in + 31) / 32, 32 * kColsumSlices, 0, st, work, gr.dsa, sh.n_in, grid * R);
 }
 
 template <int Q, typename WT>
@@ -714,24 +721,20 @@ static cudaError_t awq_lpg(bool bwd, int mode, const Shape& sh, const void* W, u
     awq_grid(sh, LPG, cb, ranges, rpr);
     const dim3 grid(cb, (unsigned)ranges);
     if (bwd) {
-        awq_bwd_kernel<Q, WT, LPG><<<grid, kThreads, 0, st>>>(W, p.sa, p.delta, p.za, p.alpha, p.zb, codes, gup,
+        cudaError_t e = launch_dependent(awq_bwd_kernel<Q, WT, LPG>, grid, kThreads, 0, st, W, p.sa, p.delta, p.za, p.alpha, p.zb, codes, gup,
                                                              gr.ddelta, gr.dza, gr.dalpha, gr.dzb, work, sh.out,
                                                              sh.n_in, sh.g, rpr);
-        cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
-        awq_colsum_kernel<<<(sh.n_in + 31) / 32, 32 * kColsumSlices, 0, st>>>(work, gr.dsa, sh.n_in, (int)ranges);
-        return cudaGetLastError();
+        return launch_dependent(awq_colsum_kernel, (sh.n_in + 31) / 32, 32 * kColsumSlices, 0, st, work, gr.dsa, sh.n_in, (int)ranges);
     }
     if (mode == FWD_KEEP)
-        awq_fwd_kernel<Q, WT, LPG, FWD_KEEP><<<grid, kThreads, 0, st>>>(W, p.sa, p.delta, p.za, p.alpha, p.zb, codes,
-                                                                        what, sh.out, sh.n_in, sh.g, rpr);
-    else if (mode == FWD_REMAP)
-        awq_fwd_kernel<Q, WT, LPG, FWD_REMAP><<<grid, kThreads, 0, st>>>(W, p.sa, p.delta, p.za, p.alpha, p.zb, codes,
-                                                                         what, sh.out, sh.n_in, sh.g, rpr);
-    else
-        awq_fwd_kernel<Q, WT, LPG, FWD_FULL><<<grid, kThreads, 0, st>>>(W, p.sa, p.delta, p.za, p.alpha, p.zb, codes,
-                                                                        what, sh.out, sh.n_in, sh.g, rpr);
-    return cudaGetLastError();
+        return launch_dependent(awq_fwd_kernel<Q, WT, LPG, FWD_KEEP>, grid, kThreads, 0, st, W, p.sa, p.delta, p.za,
+                                p.alpha, p.zb, codes, what, sh.out, sh.n_in, sh.g, rpr);
+    if (mode == FWD_REMAP)
+        return launch_dependent(awq_fwd_kernel<Q, WT, LPG, FWD_REMAP>, grid, kThreads, 0, st, W, p.sa, p.delta, p.za,
+                                p.alpha, p.zb, codes, what, sh.out, sh.n_in, sh.g, rpr);
+    return launch_dependent(awq_fwd_kernel<Q, WT, LPG, FWD_FULL>, grid, kThreads, 0, st, W, p.sa, p.delta, p.za, p.alpha,
+                            p.zb, codes, what, sh.out, sh.n_in, sh.g, rpr);
 }
 
 template <int Q, typename WT>

@@ -216,7 +216,7 @@ bcq_tc_kernel(const __grid_constant__ CUtensorMap tm_planes, const uint32_t* __r
     float* sums = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(xs) + (size_t)sb_per * kTcCols * N * 2);
 
     // the slice sum (a programmatic dependent) may be scheduled now; it waits for this grid's results
-    asm volatile("griddepcontrol.launch_dependents;");
+    dependents_may_start();
     if (warp == 0) tc::alloc(tma::smem_addr(&tm_addr), (uint32_t)tmem_cols);
     if (threadIdx.x < kTcMaxGroups) {
         const int i = threadIdx.x;
@@ -230,7 +230,7 @@ bcq_tc_kernel(const __grid_constant__ CUtensorMap tm_planes, const uint32_t* __r
     }
     __syncthreads();
     // launched as a programmatic dependent itself: nothing global is touched before the work ahead has completed
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    inputs_ready();
 
     // stages of a warpgroup: tile-major, spt per tile
     const int spt = (sbn + SBS - 1) / SBS;
@@ -609,17 +609,7 @@ cudaError_t run_tc(const uint32_t* planes, const float* astar, const float* zsta
     while (cols < p.groups * tc_tmem_cols(GB, N)) cols *= 2;
     int smem = 1024 + p.sb_per * tc_pass_bytes(GB, N) + (staged ? p.groups * kTcStages * tc_stage_bytes(Q, N) : 0);
     if (smem < kTcMinSmem) smem = kTcMinSmem;
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.gridDim = dim3((unsigned)(p.n_ks * p.n_rb), (unsigned)chunks);
-    cfg.blockDim = dim3(p.groups * 160);
-    cfg.dynamicSmemBytes = (size_t)smem;
-    cfg.stream = st;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    e = cudaLaunchKernelEx(&cfg, kern, map, planes, astar, zstar, x, x_bf16, p.n_ks > 1 ? work : y, out, n_in, g, batch,
+    e = launch_dependent(kern, dim3((unsigned)(p.n_ks * p.n_rb), (unsigned)chunks), dim3(p.groups * 160), (size_t)smem, st, map, planes, astar, zstar, x, x_bf16, p.n_ks > 1 ? work : y, out, n_in, g, batch,
                            p.n_ks, p.sb_per, p.tiles, cols, staged ? 1 : 0, pm);
     if (e != cudaSuccess || p.n_ks == 1) return e;
     return gemv_reduce(work, y, (int64_t)batch * out, p.n_ks, st);

@@ -36,6 +36,8 @@ bwd_kernel(const void* __restrict__ W, const float* __restrict__ S, const float*
            const float* __restrict__ ZB, const uint8_t* __restrict__ CODES, const float* __restrict__ GUP,
            float* __restrict__ DS, float* __restrict__ DSR, float* __restrict__ DDELTA, float* __restrict__ DZU,
            float* __restrict__ DZB, float* __restrict__ DALPHA, int64_t out, int n_in, int g, int R) {
+    dependents_may_start();
+    inputs_ready();
     constexpr int L = 1 << Q;
     constexpr int NG = 32 / LPG;                 // groups per unit
     using SR8 = SegReduce<LPG>;
@@ -155,10 +157,9 @@ static cudaError_t run_bwd(const Shape& sh, const void* W, uq_params p, const ui
     const int Gr = sh.n_in / sh.g;
     const int R = rows_per_block((Gr + NG - 1) / NG);
     const int64_t blocks = (sh.out + R - 1) / R;
-    bwd_kernel<Q, WT, LPG, ELEM><<<dim3((unsigned)blocks), kThreads, 0, st>>>(
+    return launch_dependent(bwd_kernel<Q, WT, LPG, ELEM>, dim3((unsigned)blocks), kThreads, 0, st, 
         W, p.s, p.sr, p.delta, p.zu, p.alpha, p.zb, codes, gup, gr.ds, gr.dsr, gr.ddelta, gr.dzu, gr.dzb, gr.dalpha,
         sh.out, sh.n_in, sh.g, R);
-    return cudaGetLastError();
 }
 
 template <int Q>

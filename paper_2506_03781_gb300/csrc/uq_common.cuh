@@ -26,6 +26,17 @@ constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
 constexpr unsigned kFull = 0xffffffffu;
 
+// Programmatic dependent launch: a kernel lets the next one on the stream
+// be scheduled while it runs (dependents_may_start, first thing) and itself
+// waits for the work ahead of it before its first access to global memory
+// (inputs_ready; returns at once when it was not launched as a dependent).
+// What overlaps is the launch and the set-up of shared memory.  Four kernels of
+// a 1024 x 1024 matrix: 30.5 -> 19.0 us queued, of 14336 x 4096: 441 -> 427 us.
+// Not for the initialization (one long launch) and the clusters of the fused
+// step (slower: see its launch).
+__device__ __forceinline__ void dependents_may_start() { asm volatile("griddepcontrol.launch_dependents;"); }
+__device__ __forceinline__ void inputs_ready() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // Weight-storage adaptors: 4 consecutive weights per lane.
 struct WF32 {
     using raw = float4;

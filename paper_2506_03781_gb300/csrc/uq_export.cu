@@ -38,6 +38,8 @@ export_kernel(const void* __restrict__ W, const float* __restrict__ DELTA, const
               const float* __restrict__ ALPHA, const float* __restrict__ ZB, const uint8_t* __restrict__ CODES,
               uint32_t* __restrict__ PLANES, typename OT::T* __restrict__ ASTAR, typename OT::T* __restrict__ ZSTAR,
               int64_t out, int n_in, int g) {
+    dependents_may_start();
+    inputs_ready();
     constexpr int L = 1 << Q;
     constexpr uint32_t kMask = uint32_t(L - 1) * 0x01010101u;
     const int words = n_in / 32;
@@ -167,9 +169,8 @@ static cudaError_t run_export(const Shape& sh, const void* W, uq_params p, const
                               typename OT::T* astar, typename OT::T* zstar, cudaStream_t st) {
     const int64_t words = sh.n_in / 32;
     const int grid = export_grid(sh.out * (!EQ4 && (words & 3) == 0 ? words / 4 : words));
-    export_kernel<Q, WT, EQ4, OT><<<grid, kThreads, 0, st>>>(W, p.delta, p.zu, p.alpha, p.zb, codes, planes, astar,
+    return launch_dependent(export_kernel<Q, WT, EQ4, OT>, grid, kThreads, 0, st, W, p.delta, p.zu, p.alpha, p.zb, codes, planes, astar,
                                                              zstar, sh.out, sh.n_in, sh.g);
-    return cudaGetLastError();
 }
 
 template <int Q, typename OT>

@@ -27,6 +27,8 @@ fwd_kernel(const void* __restrict__ W, const float* __restrict__ S, const float*
            const float* __restrict__ DELTA, const float* __restrict__ ZU, const float* __restrict__ ALPHA,
            const float* __restrict__ ZB, uint8_t* __restrict__ CODES, float* __restrict__ WHAT, int64_t out,
            int n_in, int g, int R, int mode) {
+    dependents_may_start();
+    inputs_ready();
     constexpr int L = 1 << Q;
     constexpr int NG = 32 / LPG;
     __shared__ MapTab<Q, NG> tabs[kWarps];
@@ -141,9 +143,8 @@ static cudaError_t run_fwd(const Shape& sh, const void* W, uq_params p, uint8_t*
     const int Gr = sh.n_in / sh.g;
     const int R = rows_per_block((Gr + NG - 1) / NG);
     const int64_t blocks = (sh.out + R - 1) / R;
-    fwd_kernel<Q, WT, LPG><<<dim3((unsigned)blocks), kThreads, 0, st>>>(
+    return launch_dependent(fwd_kernel<Q, WT, LPG>, dim3((unsigned)blocks), kThreads, 0, st, 
         W, p.s, p.sr, p.delta, p.zu, p.alpha, p.zb, codes, what, sh.out, sh.n_in, sh.g, R, mode);
-    return cudaGetLastError();
 }
 
 template <int Q>

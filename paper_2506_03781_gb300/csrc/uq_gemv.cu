@@ -109,7 +109,8 @@ bcq_gemv_partial_kernel(const uint32_t* __restrict__ PLANES, const float* __rest
     float* xs = nib + kNibFloats;                     // [32][17]: lane l's columns at 17 l
     uint32_t* stages = reinterpret_cast<uint32_t*>(xs + kXsFloats);
     // the tile sum (a programmatic dependent) may be scheduled now; it waits for this grid's results
-    asm volatile("griddepcontrol.launch_dependents;");
+    dependents_may_start();
+    inputs_ready();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int t = (int)(blockIdx.x % n_tiles);
     const int64_t r0 = (int64_t)(blockIdx.x / n_tiles) * rows_per_block;
@@ -317,7 +318,7 @@ bcq_gemv_tma_kernel(const __grid_constant__ CUtensorMap tm_planes, const __grid_
     unsigned char* stages = reinterpret_cast<unsigned char*>(xs + kXsFloats);
     unsigned long long* bars = reinterpret_cast<unsigned long long*>(stages + (size_t)kGemvWarps * NS * SB);
     // the tile sum (a programmatic dependent) may be scheduled now; it waits for this grid's results
-    asm volatile("griddepcontrol.launch_dependents;");
+    dependents_may_start();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int t = (int)(blockIdx.x % n_tiles);
     const int64_t r0 = (int64_t)(blockIdx.x / n_tiles) * rows_per_block;
@@ -337,6 +338,7 @@ bcq_gemv_tma_kernel(const __grid_constant__ CUtensorMap tm_planes, const __grid_
     }
     __syncwarp();
 
+    inputs_ready();
     // items: token-major, this warp's batches k = 0 .. my_nb - 1 per token
     const long long total = (long long)batch * my_nb;
     long long issued = 0, waited = 0;
@@ -543,7 +545,7 @@ bcq_gemv_wide_kernel(const __grid_constant__ CUtensorMap tm_planes, const __grid
     static_assert(NGT >= 4 && (NGT * Q * 4) % 16 == 0, "alpha* and z* boxes must span a multiple of 16 bytes");
     extern __shared__ __align__(128) unsigned char wsm[];
     // the tile sum (a programmatic dependent) may be scheduled now; it waits for this grid's results
-    asm volatile("griddepcontrol.launch_dependents;");
+    dependents_may_start();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int t = (int)(blockIdx.x % n_tiles);
     const int64_t r0 = (int64_t)(blockIdx.x / n_tiles) * rows_per_block;
@@ -588,7 +590,7 @@ bcq_gemv_wide_kernel(const __grid_constant__ CUtensorMap tm_planes, const __grid
     // overwrites, or whatever produced the inputs): nothing global is read or
     // written before that grid has completed.  Only the launch and the set-up
     // above overlap it.
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    inputs_ready();
 
     const int total = batch * my_nb;                           // items: token-major, this warp's batches
     int issued = 0, waited = 0, ik = 0;
@@ -697,8 +699,8 @@ bcq_gemv_reduce_kernel(const float* __restrict__ PART, float* __restrict__ Y, in
     // while that kernel still runs, and waits here until the product grid has
     // completed and its partials are visible.  The next product kernel on the
     // stream may be scheduled once every block of this grid has started.
-    asm volatile("griddepcontrol.launch_dependents;");
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    dependents_may_start();
+    inputs_ready();
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         float acc = 0.f;
         for (int t = 0; t < n_tiles; ++t) acc += __ldg(PART + (int64_t)t * n + i);
@@ -919,17 +921,7 @@ cudaError_t gemv_reduce(const float* work, float* y, int64_t n, int n_tiles, cud
     int64_t blocks = (n + 255) / 256;
     const int64_t cap = (int64_t)sm_count() * 8;
     if (blocks > cap) blocks = cap;
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.gridDim = dim3((unsigned)blocks);
-    cfg.blockDim = dim3(256);
-    cfg.dynamicSmemBytes = 0;
-    cfg.stream = st;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, bcq_gemv_reduce_kernel, work, y, n, n_tiles);
+    return launch_dependent(bcq_gemv_reduce_kernel, (unsigned)blocks, 256, 0, st, work, y, n, n_tiles);
 }
 
 template <int Q, typename XT, int NGT>
@@ -963,9 +955,8 @@ static cudaError_t run_gemv(const uint32_t* planes, const float* astar, const fl
             if (e != cudaSuccess) return e;
             int64_t n_rb = 0, rpb = 0;
             gemv_row_blocks(out, n_tiles, per_sm, n_rb, rpb);
-            kern<<<(unsigned)(n_rb * n_tiles), kGemvThreads, smem_tma, st>>>(mp, ma, mz, x, work, out, n_in, batch,
-                                                                           n_tiles, rpb);
-            e = cudaGetLastError();
+            e = launch_dependent(kern, (unsigned)(n_rb * n_tiles), kGemvThreads, smem_tma, st, mp, ma, mz, x, work, out,
+                                 n_in, batch, n_tiles, rpb);
             if (e != cudaSuccess) return e;
             return gemv_reduce(work, y, (int64_t)batch * out, n_tiles, st);
         }
@@ -976,9 +967,8 @@ static cudaError_t run_gemv(const uint32_t* planes, const float* astar, const fl
     if (e != cudaSuccess) return e;
     int64_t n_rb = 0, rpb = 0;
     gemv_row_blocks(out, n_tiles, per_sm, n_rb, rpb);
-    kern<<<(unsigned)(n_rb * n_tiles), kGemvThreads, smem, st>>>(planes, astar, zstar, x, work, out, n_in, g, batch,
-                                                                 n_tiles, rpb, pwide);
-    e = cudaGetLastError();
+    e = launch_dependent(kern, (unsigned)(n_rb * n_tiles), kGemvThreads, smem, st, planes, astar, zstar, x, work, out, n_in,
+                         g, batch, n_tiles, rpb, pwide);
     if (e != cudaSuccess) return e;
     return gemv_reduce(work, y, (int64_t)batch * out, n_tiles, st);
 }
@@ -1008,17 +998,8 @@ static cudaError_t run_gemv_wide(const uint32_t* planes, const float* astar, con
         const int n_tiles = n_in / kWideCols;
         int64_t n_rb = 0, rpb = 0;
         gemv_row_blocks(out, n_tiles, per_sm, n_rb, rpb, (double)kWideLutRows);
-        cudaLaunchConfig_t cfg = {};
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[0].val.programmaticStreamSerializationAllowed = 1;
-        cfg.gridDim = dim3((unsigned)(n_rb * n_tiles));
-        cfg.blockDim = dim3(NW * 32);
-        cfg.dynamicSmemBytes = DYN;
-        cfg.stream = st;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        e = cudaLaunchKernelEx(&cfg, kern, mp, ma, mz, x, work, out, n_in, batch, n_tiles, rpb);
+        e = launch_dependent(kern, (unsigned)(n_rb * n_tiles), NW * 32, DYN, st, mp, ma, mz, x, work, out, n_in, batch, n_tiles,
+                             rpb);
         if (e != cudaSuccess) return e;
         return gemv_reduce(work, y, (int64_t)batch * out, n_tiles, st);
     } else {

@@ -105,6 +105,23 @@ int sm_count();
 // bounded wait runs out.
 cudaError_t stream_error(bool clear, unsigned int* flag);
 
+// Launches a kernel as a programmatic dependent of the work ahead of it on the
+// stream (see inputs_ready in uq_common.cuh).
+template <typename... P, typename... A>
+cudaError_t launch_dependent(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
+
 // Forward modes (see uq_api.h): full mapping, local remap step, keep codes.
 enum { FWD_FULL = 0, FWD_REMAP = 1, FWD_KEEP = 2 };
 

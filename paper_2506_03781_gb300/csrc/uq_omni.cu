@@ -56,6 +56,8 @@ omni_fwd_kernel(const void* __restrict__ W, const float* __restrict__ BETA, cons
                 const float* __restrict__ ALPHA, const float* __restrict__ ZB, uint8_t* __restrict__ CODES,
                 float* __restrict__ WHAT, float* __restrict__ DOUT, float* __restrict__ ZOUT, int64_t out, int n_in,
                 int g, int R) {
+    dependents_may_start();
+    inputs_ready();
     constexpr int L = 1 << Q;
     constexpr int NG = 32 / LPG;
     __shared__ MapTab<Q, NG> tabs[kWarps];
@@ -154,6 +156,8 @@ omni_bwd_kernel(const void* __restrict__ W, const float* __restrict__ BETA, cons
                 const float* __restrict__ ALPHA, const float* __restrict__ ZB, const uint8_t* __restrict__ CODES,
                 const float* __restrict__ GUP, float* __restrict__ DBETA, float* __restrict__ DGAMMA,
                 float* __restrict__ DALPHA, float* __restrict__ DZB, int64_t out, int n_in, int g, int R) {
+    dependents_may_start();
+    inputs_ready();
     constexpr int L = 1 << Q;
     constexpr int NG = 32 / LPG;
     using SR8 = SegReduce<LPG>;
@@ -295,6 +299,7 @@ __global__ void __launch_bounds__(kThreads, 3)
 omni_stream_fwd_kernel(const void* __restrict__ W, const float* __restrict__ BETA, const float* __restrict__ GAMMA,
                        const float* __restrict__ ALPHA, const float* __restrict__ ZB, uint8_t* __restrict__ CODES,
                        float* __restrict__ WHAT, int64_t out, int n_in, int R, int n_rb) {
+    dependents_may_start();
     using St = OmniFwdStage<Q, WT, G_, MODE>;
     constexpr int L = 1 << Q, LPG = St::LPG, NG = St::NG, NV = St::NV, UE = St::UE, NST = St::NST;
     extern __shared__ __align__(128) unsigned char smem[];
@@ -315,6 +320,7 @@ omni_stream_fwd_kernel(const void* __restrict__ W, const float* __restrict__ BET
         tma::bar_init_fence();
     }
     __syncwarp();
+    inputs_ready();
     auto issue = [&](const Cursor& c, int s) {          // lane 0 only
         omni_issue<Q, St>(it, c, s, tma::smem_addr(&bars[warp][s]), wsm, W, nullptr, CODES, BETA, GAMMA, ZB, ALPHA,
                           out, n_in, Gr);
@@ -409,6 +415,7 @@ omni_stream_bwd_kernel(const void* __restrict__ W, const float* __restrict__ BET
                        const float* __restrict__ ALPHA, const float* __restrict__ ZB, const uint8_t* __restrict__ CODES,
                        const float* __restrict__ GUP, float* __restrict__ DBETA, float* __restrict__ DGAMMA,
                        float* __restrict__ DALPHA, float* __restrict__ DZB, int64_t out, int n_in, int R, int n_rb) {
+    dependents_may_start();
     using St = OmniBwdStage<Q, WT, G_>;
     constexpr int L = 1 << Q, LPG = St::LPG, NG = St::NG, NV = St::NV, UE = St::UE, NST = St::NST;
     using SR8 = SegReduce<LPG>;
@@ -427,6 +434,7 @@ omni_stream_bwd_kernel(const void* __restrict__ W, const float* __restrict__ BET
         tma::bar_init_fence();
     }
     __syncwarp();
+    inputs_ready();
     auto issue = [&](const Cursor& c, int s) {          // lane 0 only
         omni_issue<Q, St>(it, c, s, tma::smem_addr(&bars[warp][s]), wsm, W, GUP, CODES, BETA, GAMMA, ZB, ALPHA, out,
                           n_in, Gr);
@@ -540,8 +548,7 @@ static cudaError_t run_omni_stream_fwd(const Shape& sh, const void* W, uq_params
     int grid = 0;
     cudaError_t e = grid_for<OmniTag<St, MODE>>(kern, dyn, n_rb, grid);
     if (e != cudaSuccess) return e;
-    kern<<<grid, kThreads, dyn, st>>>(W, p.beta, p.gamma, p.alpha, p.zb, codes, what, sh.out, sh.n_in, R, n_rb);
-    return cudaGetLastError();
+    return launch_dependent(kern, grid, kThreads, dyn, st, W, p.beta, p.gamma, p.alpha, p.zb, codes, what, sh.out, sh.n_in, R, n_rb);
 }
 
 template <int Q, typename WT, int G_>
@@ -556,9 +563,8 @@ static cudaError_t run_omni_stream_bwd(const Shape& sh, const void* W, uq_params
     int grid = 0;
     cudaError_t e = grid_for<OmniTag<St, 9>>(kern, dyn, n_rb, grid);
     if (e != cudaSuccess) return e;
-    kern<<<grid, kThreads, dyn, st>>>(W, p.beta, p.gamma, p.alpha, p.zb, codes, gup, gr.dbeta, gr.dgamma, gr.dalpha,
+    return launch_dependent(kern, grid, kThreads, dyn, st, W, p.beta, p.gamma, p.alpha, p.zb, codes, gup, gr.dbeta, gr.dgamma, gr.dalpha,
                                       gr.dzb, sh.out, sh.n_in, R, n_rb);
-    return cudaGetLastError();
 }
 
 template <int Q, typename WT, int G_>
@@ -616,9 +622,8 @@ static cudaError_t run_omni_fwd(const Shape& sh, const void* W, uq_params_omni p
     const int Gr = sh.n_in / sh.g;
     const int R = rows_per_block((Gr + NG - 1) / NG);
     const int64_t blocks = (sh.out + R - 1) / R;
-    omni_fwd_kernel<Q, WT, LPG, MODE><<<dim3((unsigned)blocks), kThreads, 0, st>>>(
+    return launch_dependent(omni_fwd_kernel<Q, WT, LPG, MODE>, dim3((unsigned)blocks), kThreads, 0, st, 
         W, p.beta, p.gamma, p.alpha, p.zb, codes, what, dout, zout, sh.out, sh.n_in, sh.g, R);
-    return cudaGetLastError();
 }
 
 template <int Q, typename WT, int LPG>
@@ -628,10 +633,9 @@ static cudaError_t run_omni_bwd(const Shape& sh, const void* W, uq_params_omni p
     const int Gr = sh.n_in / sh.g;
     const int R = rows_per_block((Gr + NG - 1) / NG);
     const int64_t blocks = (sh.out + R - 1) / R;
-    omni_bwd_kernel<Q, WT, LPG><<<dim3((unsigned)blocks), kThreads, 0, st>>>(
+    return launch_dependent(omni_bwd_kernel<Q, WT, LPG>, dim3((unsigned)blocks), kThreads, 0, st, 
         W, p.beta, p.gamma, p.alpha, p.zb, codes, gup, gr.dbeta, gr.dgamma, gr.dalpha, gr.dzb, sh.out, sh.n_in,
         sh.g, R);
-    return cudaGetLastError();
 }
 
 // kind: 0 forward (mode), 1 backward, 2 scales only

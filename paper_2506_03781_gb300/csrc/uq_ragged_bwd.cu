@@ -71,6 +71,7 @@ __global__ void __launch_bounds__(kThreads, 2)
 ragged_bwd_kernel(const RaggedSrc src, const float* __restrict__ SR, float* __restrict__ DS, float* __restrict__ DSR,
                   float* __restrict__ DDELTA, float* __restrict__ DZU, float* __restrict__ DZB,
                   float* __restrict__ DALPHA, int64_t out, int n_in, int R, int n_rb) {
+    dependents_may_start();
     using St = RaggedBwdStage<Q, WT, G_>;
     constexpr int L = 1 << Q, LPG = St::LPG, NG = St::NG, NV = St::NV, UE = St::UE, NST = St::NST;
     using SR8 = SegReduce<LPG>;
@@ -93,6 +94,7 @@ ragged_bwd_kernel(const RaggedSrc src, const float* __restrict__ SR, float* __re
     ragged_copies<Q, St>(cps, src);
     __syncthreads();
     const int64_t whole = ragged_whole<Q>(out * Gr);
+    inputs_ready();
     auto issue = [&](const Cursor& c, int s) {           // the whole warp
         const uint32_t bar = tma::smem_addr(&bars[warp][s]);
         const int64_t row = it.row(c.k);
@@ -241,9 +243,8 @@ static cudaError_t run_ragged_bwd(const Shape& sh, const void* W, uq_params p, c
     if (e != cudaSuccess) return e;
     const RaggedSrc src{static_cast<const unsigned char*>(W), reinterpret_cast<const unsigned char*>(p.s),
                         reinterpret_cast<const unsigned char*>(gup), codes, p.delta, p.zu, p.zb, p.alpha};
-    kern<<<grid, kThreads, dyn, st>>>(src, p.sr, gr.ds, gr.dsr, gr.ddelta, gr.dzu, gr.dzb, gr.dalpha, sh.out, sh.n_in,
+    return launch_dependent(kern, grid, kThreads, dyn, st, src, p.sr, gr.ds, gr.dsr, gr.ddelta, gr.dzu, gr.dzb, gr.dalpha, sh.out, sh.n_in,
                                       R, n_rb);
-    return cudaGetLastError();
 }
 
 template <int Q, int G_>

@@ -24,6 +24,7 @@ template <int Q, typename WT, int G_, int MODE>
 __global__ void __launch_bounds__(kThreads, MODE == FWD_KEEP ? 4 : 3)
 ragged_fwd_kernel(const RaggedSrc src, const float* __restrict__ SR, uint8_t* __restrict__ CODES,
                   float* __restrict__ WHAT, int64_t out, int n_in, int R, int n_rb) {
+    dependents_may_start();
     using St = RaggedFwdStage<Q, WT, G_, MODE>;
     constexpr int L = 1 << Q, LPG = St::LPG, NG = St::NG, NV = St::NV, UE = St::UE, NST = St::NST;
     extern __shared__ __align__(128) unsigned char smem[];
@@ -46,6 +47,7 @@ ragged_fwd_kernel(const RaggedSrc src, const float* __restrict__ SR, uint8_t* __
     ragged_copies<Q, St>(cps, src);
     __syncthreads();
     const int64_t whole = ragged_whole<Q>(out * Gr);
+    inputs_ready();
     auto issue = [&](const Cursor& c, int s) {           // the whole warp
         const uint32_t bar = tma::smem_addr(&bars[warp][s]);
         const int64_t row = it.row(c.k);
@@ -159,8 +161,7 @@ static cudaError_t run_ragged_fwd(const Shape& sh, const void* W, uq_params p, u
     if (e != cudaSuccess) return e;
     const RaggedSrc src{static_cast<const unsigned char*>(W), reinterpret_cast<const unsigned char*>(p.s), nullptr,
                         codes, p.delta, p.zu, p.zb, p.alpha};
-    kern<<<grid, kThreads, dyn, st>>>(src, p.sr, codes, what, sh.out, sh.n_in, R, n_rb);
-    return cudaGetLastError();
+    return launch_dependent(kern, grid, kThreads, dyn, st, src, p.sr, codes, what, sh.out, sh.n_in, R, n_rb);
 }
 
 template <int Q, int G_>

@@ -65,6 +65,7 @@ bwd_stream_kernel(const void* __restrict__ W, const float* __restrict__ S, const
                   float* __restrict__ DS, float* __restrict__ DSR, float* __restrict__ DDELTA,
                   float* __restrict__ DZU, float* __restrict__ DZB, float* __restrict__ DALPHA, int64_t out,
                   int n_in, int R, int n_rb, int branchy) {
+    dependents_may_start();
     using St = Stage<Q, WT, G_, true, true, true, UQ_BWD_STAGE_BYTES>;
     constexpr int L = 1 << Q, LPG = St::LPG, NG = St::NG, NV = St::NV, UE = St::UE, NST = St::NST;
     constexpr uint32_t TX = St::TX;
@@ -105,6 +106,7 @@ bwd_stream_kernel(const void* __restrict__ W, const float* __restrict__ S, const
         cps[i] = CopySpec{b[i], per[i], size[i], off[i], i >= 4 ? 1u : 0u};
     }
     __syncthreads();
+    inputs_ready();
     // issued by the whole warp: lane 0 arms the stage's mbarrier with the
     // unit's bytes, then lanes 0..7 each start one copy
     auto issue = [&](const Cursor& c, int s) {
@@ -276,6 +278,7 @@ fwd_stream_kernel(const void* __restrict__ W, const float* __restrict__ S, const
                   const float* __restrict__ DELTA, const float* __restrict__ ZU, const float* __restrict__ ALPHA,
                   const float* __restrict__ ZB, uint8_t* __restrict__ CODES, float* __restrict__ WHAT,
                   int64_t out, int n_in, int R, int n_rb) {
+    dependents_may_start();
     static_assert(MODE != FWD_KEEP, "the keep step runs keep_stream_kernel");
     constexpr int mode = MODE;
     constexpr bool need_c = MODE != FWD_FULL;
@@ -299,6 +302,7 @@ fwd_stream_kernel(const void* __restrict__ W, const float* __restrict__ S, const
         tma::bar_init_fence();
     }
     __syncwarp();
+    inputs_ready();
 
     auto issue = [&](const Cursor& c, int s) {           // lane 0 only
         const uint32_t bar = tma::smem_addr(&bars[warp][s]);
@@ -409,6 +413,7 @@ __global__ void __launch_bounds__(kThreads, UQ_STREAM_FWD_MIN_BLOCKS)
 keep_stream_kernel(const float* __restrict__ DELTA, const float* __restrict__ ZU, const float* __restrict__ ALPHA,
                    const float* __restrict__ ZB, const uint8_t* __restrict__ CODES, float* __restrict__ WHAT,
                    int64_t out, int n_in, int R, int n_rb) {
+    dependents_may_start();
     using St = KeepStage<Q, G_, KU>;
     constexpr int L = 1 << Q, LPG = St::LPG, NG = St::NG, NGK = St::NGK, NV = St::NV, UE = St::UE, NST = St::NST;
     extern __shared__ __align__(128) unsigned char smem[];
@@ -426,6 +431,7 @@ keep_stream_kernel(const float* __restrict__ DELTA, const float* __restrict__ ZU
         tma::bar_init_fence();
     }
     __syncwarp();
+    inputs_ready();
 
     auto issue = [&](const Cursor& c, int s) {           // lane 0 only
         const uint32_t bar = tma::smem_addr(&bars[warp][s]);
@@ -522,10 +528,9 @@ static cudaError_t run_bwd_stream(const Shape& sh, const void* W, uq_params p, c
     // one occupancy cache (and shared-memory opt-in) per kernel variant
     cudaError_t e = grid_for<BwdTag<St, ELEM>>(kern, dyn, n_rb, grid);
     if (e != cudaSuccess) return e;
-    kern<<<grid, kThreads, dyn, st>>>(W, p.s, p.sr, p.delta, p.zu, p.alpha, p.zb, codes, gup, gr.ds, gr.dsr,
+    return launch_dependent(kern, grid, kThreads, dyn, st, W, p.s, p.sr, p.delta, p.zu, p.alpha, p.zb, codes, gup, gr.ds, gr.dsr,
                                       gr.ddelta, gr.dzu, gr.dzb, gr.dalpha, sh.out, sh.n_in, R, n_rb,
                                       U >= kBranchyUnits ? 1 : 0);
-    return cudaGetLastError();
 }
 
 template <int Q, typename WT, int G_, int MODE>
@@ -540,9 +545,8 @@ static cudaError_t run_fwd_stream_mode(const Shape& sh, const void* W, uq_params
     int grid = 0;
     cudaError_t e = grid_for<St>(kern, dyn, n_rb, grid);
     if (e != cudaSuccess) return e;
-    kern<<<grid, kThreads, dyn, st>>>(W, p.s, p.sr, p.delta, p.zu, p.alpha, p.zb, codes, what, sh.out, sh.n_in, R,
+    return launch_dependent(kern, grid, kThreads, dyn, st, W, p.s, p.sr, p.delta, p.zu, p.alpha, p.zb, codes, what, sh.out, sh.n_in, R,
                                       n_rb);
-    return cudaGetLastError();
 }
 
 template <int Q, int G_, int KU>
@@ -556,8 +560,7 @@ static cudaError_t run_keep_stream(const Shape& sh, uq_params p, const uint8_t* 
     int grid = 0;
     cudaError_t e = grid_for<St>(kern, dyn, n_rb, grid);
     if (e != cudaSuccess) return e;
-    kern<<<grid, kThreads, dyn, st>>>(p.delta, p.zu, p.alpha, p.zb, codes, what, sh.out, sh.n_in, R, n_rb);
-    return cudaGetLastError();
+    return launch_dependent(kern, grid, kThreads, dyn, st, p.delta, p.zu, p.alpha, p.zb, codes, what, sh.out, sh.n_in, R, n_rb);
 }
 
 // Units per keep item: as many adjacent units (up to 4 and kKeepMaxGroups
