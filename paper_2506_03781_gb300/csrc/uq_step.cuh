@@ -30,8 +30,13 @@
 // W, s and the codes therefore cross HBM once per step.  Rows of up to 8
 // units belong to one thread block (R rows per block when a row has fewer
 // units than the block has warps); longer rows are split over a thread
-// block cluster of csize <= 8 blocks, whose ds_r partials are read through
-// distributed shared memory after a cluster barrier.  Each warp keeps two
+// block cluster of csize <= 8 blocks: every warp sends its ds_r partial to each
+// of them with asynchronous stores that complete on that block's mbarrier, so
+// no cluster barrier (whose release waits for the s' stores to reach memory)
+// stands between the phases; the tables of phase B are built while the
+// partials travel.  A buffer of partials is written again two row blocks
+// later: by then every warp has sent its partial of the row block between,
+// after it read this one.  Each warp keeps two
 // stages: the row block in use and the next one, whose copies are in flight
 // meanwhile.  Every mbarrier wait is bounded; a wait that runs out sets
 // g_step_err (reported by uq_check_device), and the warp stops computing
@@ -71,9 +76,16 @@ union StepTab {
     MapTab<Q, NG> b;               // phase B: levels, sorted order, local-mapping neighbours
 };
 
-__device__ __forceinline__ void step_sync(int csize) {
-    if (csize > 1) cg::this_cluster().sync();
-    else __syncthreads();
+// 4 bytes to shared memory of block `rank` of the cluster (addresses as in the
+// own block), completing on that block's mbarrier.
+__device__ __forceinline__ void send_f32(uint32_t dst, uint32_t bar, uint32_t rank, float v) {
+    asm volatile(
+        "{\n\t.reg .u32 d, b;\n\t"
+        "mapa.shared::cluster.u32 d, %0, %2;\n\t"
+        "mapa.shared::cluster.u32 b, %1, %2;\n\t"
+        "st.async.shared::cluster.mbarrier::complete_tx::bytes.b32 [d], %3, [b];\n\t}" ::"r"(dst),
+        "r"(bar), "r"(rank), "r"(__float_as_uint(v))
+        : "memory");
 }
 
 // BIO: dL/dW^ is read as bf16 and W^ written as bf16 (round to nearest
@@ -91,7 +103,8 @@ step_kernel(const void* __restrict__ W, float* S, float* SR, float* DELTA, float
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ __align__(8) unsigned long long bars[kWarps][2];
     __shared__ StepTab<Q, NG> tabs[kWarps];
-    __shared__ float red[2][kWarps];              // ds_r partials (Delta S3 sums) of row blocks k, k + 1
+    __shared__ float red[2][kMaxCluster * kWarps];   // ds_r partials (Delta S3 sums) of row blocks k, k + 1: [rank][warp]
+    __shared__ __align__(8) unsigned long long rbar[2];   // their arrival, when the row is spread over a cluster
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int sub = lane / LPG, li = lane % LPG;
@@ -114,9 +127,14 @@ step_kernel(const void* __restrict__ W, float* S, float* SR, float* DELTA, float
     if (lane == 0) {
         tma::bar_init(tma::smem_addr(&bars[warp][0]), 1);
         tma::bar_init(tma::smem_addr(&bars[warp][1]), 1);
+        if (warp == 0) {
+            tma::bar_init(tma::smem_addr(&rbar[0]), 1);
+            tma::bar_init(tma::smem_addr(&rbar[1]), 1);
+        }
         tma::bar_init_fence();
     }
-    __syncthreads();
+    if (csize > 1) cg::this_cluster().sync();     // no partial arrives before the barriers exist
+    else __syncthreads();
 
     // The eight copies of a unit, one per lane 0..7: source base, bytes per
     // element (per group for the parameters), size and stage offset, from a
@@ -158,7 +176,7 @@ step_kernel(const void* __restrict__ W, float* S, float* SR, float* DELTA, float
     int64_t next_issue = 0, next_wait = 0;        // items issued / waited for (every lane)
     while (next_issue < 2 && next_issue < n_items) issue(next_issue++);
 
-    bool alive = true;
+    bool alive = true, joined = true;
     for (int64_t k = 0; k < n_blocks; ++k) {
         const int64_t row = row_of(k);
         const bool mine = k < n_items;
@@ -168,6 +186,8 @@ step_kernel(const void* __restrict__ W, float* S, float* SR, float* DELTA, float
         float* pb = reinterpret_cast<float*>(st + St::OFF_B);
         float* pa = reinterpret_cast<float*>(st + St::OFF_A);
         float sr = 1.f, prow = 0.f;
+        if (csize > 1 && threadIdx.x == 0)
+            tma::bar_arrive_tx(tma::smem_addr(&rbar[k & 1]), (uint32_t)(csize * kWarps * sizeof(float)));
         if (mine && alive) {
             // one verdict for the whole warp (lanes poll the mbarrier separately)
             if (__all_sync(kFull, tma::bar_wait(tma::smem_addr(&bars[warp][k & 1]), (uint32_t)((k >> 1) & 1)))) {
@@ -179,7 +199,7 @@ step_kernel(const void* __restrict__ W, float* S, float* SR, float* DELTA, float
         }
         if (mine && alive) {
             // ---- phase A: backward of step t and the update of s and the group parameters ----
-            sr = SR[row];                          // this row's s_r is rewritten only after the barrier below
+            sr = SR[row];                          // rewritten only once every partial of the row has been sent
 #pragma unroll
             for (int e = lane; e < NG * L; e += 32) {
                 const int kk = e / L, c = e % L;
@@ -255,26 +275,14 @@ step_kernel(const void* __restrict__ W, float* S, float* SR, float* DELTA, float
             }
         }
         prow = warp_sum(prow);
-        if (lane == 0) red[k & 1][warp] = prow;
-        step_sync(csize);                          // every ds_r partial of row block k is in shared memory
+        if (csize == 1) {
+            if (lane == 0) red[k & 1][warp] = prow;
+        } else if (lane < csize) {
+            send_f32(tma::smem_addr(&red[k & 1][crank * kWarps + warp]), tma::smem_addr(&rbar[k & 1]), (uint32_t)lane, prow);
+        }
+        __syncwarp();                              // the updated parameters of the unit are in the stage
         if (mine && alive) {
-            // ---- s_r' of the row: partials summed in (block rank, warp) order, the same in every block ----
-            float tot = 0.f;
-            if (csize > 1) {
-                cg::cluster_group cl = cg::this_cluster();
-                for (int c = 0; c < csize; ++c) {
-                    const float* rr = cl.map_shared_rank(&red[k & 1][0], c);
-#pragma unroll
-                    for (int w = 0; w < kWarps; ++w) tot += rr[w];
-                }
-            } else {
-                for (int w = 0; w < WPR; ++w) tot += red[k & 1][row_sub * WPR + w];
-            }
-            const float dsr = -tot / sr;
-            const float sr_new = __fsub_rn(sr, __fmul_rn(lr_f, dsr));
-            if (unit == 0 && lane == 0) SR[row] = sr_new;
-
-            // ---- phase B: forward of step t + 1 from the stage ----
+            // ---- phase B's tables, while the partials are on their way ----
 #pragma unroll
             for (int e = lane; e < NG * L; e += 32) {
                 const int kk = e / L, c = e % L;
@@ -286,6 +294,29 @@ step_kernel(const void* __restrict__ W, float* S, float* SR, float* DELTA, float
             __syncwarp();
             if constexpr (MODEB == FWD_REMAP) unit_sort<Q, NG, true>(t.b, lane);
             else if constexpr (MODEB == FWD_FULL) unit_sort<Q, NG, false>(t.b, lane);
+        }
+        // every ds_r partial of row block k is in shared memory
+        if (csize == 1) {
+            __syncthreads();
+        } else if (joined && !__all_sync(kFull, tma::bar_wait(tma::smem_addr(&rbar[k & 1]), (uint32_t)((k >> 1) & 1)))) {
+            joined = alive = false;                // no later row block is waited for
+            if (lane == 0) atomicOr(&g_step_err, 2u);
+        }
+        if (mine && alive) {
+            // ---- s_r' of the row: partials summed in a fixed order, the same in every block ----
+            float tot = 0.f;
+            if (csize > 1) {
+                const int n = csize * kWarps;          // at most 64, [rank][warp]
+                const float* rr = red[k & 1];
+                tot = warp_sum((lane < n ? rr[lane] : 0.f) + (lane + 32 < n ? rr[lane + 32] : 0.f));
+            } else {
+                for (int w = 0; w < WPR; ++w) tot += red[k & 1][row_sub * WPR + w];
+            }
+            const float dsr = -tot / sr;
+            const float sr_new = __fsub_rn(sr, __fmul_rn(lr_f, dsr));
+            if (unit == 0 && lane == 0) SR[row] = sr_new;
+
+            // ---- phase B: forward of step t + 1 from the stage ----
             const float dl = pd[sub], zu = pz[sub];
             const int64_t ebase = row * n_in + (int64_t)unit * UE;
             float srt[L];
