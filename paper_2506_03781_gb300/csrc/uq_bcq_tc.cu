@@ -7,15 +7,21 @@
 // The +-1 entries are exact in bf16 and so are the activations: a bf16 token
 // is one column of the right-hand matrix, an fp32 token three (its value cut
 // into three bf16 pieces that add up to it exactly), so every product is
-// exact and the sums are taken in fp32 (tcgen05.mma kind::f16, 128 rows by N
-// columns, fp32 accumulators in tensor memory).
+// exact and the sums D_j are taken in fp32 (tcgen05.mma kind::f16, 128 rows by
+// N columns, fp32 accumulators in tensor memory).  With 64 columns, or with
+// several blocks to a pass, the entries are +-1 themselves, made by two
+// operations per pair.  Else, where making them is what takes the time (450 of
+// 900 clocks), they are of four kinds, one operation
+// each wherever the bit lies (see expand16): +-0.5; 2 or 0, against half the
+// activation; 1 or 2^-64; 1 or 2^-32.  With S0 the sum of x over the columns
+// of the first kind, (C_j x)_r = 2 D_j + S0 - S then, but for the 2^-64 and
+// 2^-32 of the clear bits, at most 2^-33 of sum |x|.
 //
 // A warpgroup owns 128 rows, one per thread.  For every plane and 128
-// columns a thread expands the row's four plane words to +-1 values in
-// registers and stores them to tensor memory, which is the left operand;
-// element k = 2 (16 word + p) + h of a row is bit p + 16 h of the word, so a
-// register holds the bits p and p + 16, moved to its two sign positions by
-// one product and one logic operation.  The block keeps the activations of
+// columns a thread expands the row's four plane words in registers and stores
+// them to tensor memory, which is the left operand; element k = 2 (16 word +
+// p) + h of a row is bit p + 16 h of the word, so a register holds the bits p
+// and p + 16.  The block keeps the activations of
 // its column slice in shared memory in the same column order (K-major core
 // matrices of 8 tokens x 16 bytes, no swizzle).  The sums come back one row per thread and are scaled
 // by that row's alpha* in registers.  Operand and sums have two buffers each:
@@ -37,19 +43,18 @@
 // summed in order by a second kernel.  Every wait is bounded.  Deterministic;
 // no atomics on outputs.
 //
-// What bounds it: with 64 columns the tensor cores need 256 clocks for a
-// plane of 128 x 128 (measured 272) and the two warpgroups about 900 each,
-// the expansion (124 operations per thread, half of them on the half-rate
-// logic pipe) and the scaling of 64 sums; with 16 columns the products take
-// 197 clocks and three warpgroups about 550 each.  14336 x 4096, q = 3,
-// g = 128, bf16: 64 tokens 447 -> 39.4 us (per-token lookup tables before),
-// 16 tokens 114 -> 20.3 us, 4 tokens 30.4 -> 19.4 us; 8192 x 28672, 4 fp32
-// tokens: 99.8 -> 76.4 us.  The same product with mma.sync and fragments in
-// registers took 72.5, 28.2, 20.6 and 108 us: a fragment register holds the
-// same expanded pair, but every lane of a quad repeats the loads and the
-// scaling, and 64 columns are bound by that pipe (38 us).  Error against 64
-// bits: 0.8e-7 to 1.3e-7, the lookup tables' 0.7e-7 to 1.7e-7.
+// What bounds it: a plane of 128 x 128 takes the tensor cores 256 clocks with
+// 64 columns (measured 272) and 197 with 16, a warpgroup 1270 (700 to expand,
+// 430 to scale 64 sums) and 750: two or three warpgroups share the logic pipe,
+// which runs at half rate.  14336 x 4096, q = 3, g = 128, bf16: 64 tokens 447
+// -> 37.9 us (per-token lookup tables before), 16 tokens 114 -> 18.8 us, 4
+// tokens 30.4 -> 18.3 us (19.4 with +-1 entries); 8192 x 28672, 4 fp32 tokens:
+// 99.8 -> 68.1 us (76.4).  The same product with mma.sync and fragments in
+// registers took 72.5, 28.2, 20.6 and 108 us: every lane of a quad repeats
+// the loads and the scaling, and 64 columns are bound by that pipe (38 us).
+// Error against 64 bits: 0.6e-7 to 1.3e-7, the lookup tables' 0.7e-7 to 1.7e-7.
 #include <cuda.h>   // CUtensorMap
+#include <cuda_bf16.h>
 
 #include <atomic>
 
@@ -80,7 +85,11 @@ __host__ __device__ constexpr int tc_tmem_cols(int gb, int n) { return 2 * (64 +
 __host__ __device__ constexpr int tc_groups(int gb, int n) {
     return 512 / tc_tmem_cols(gb, n) < kTcMaxGroups ? 512 / tc_tmem_cols(gb, n) : kTcMaxGroups;
 }
-__host__ __device__ constexpr int tc_pass_bytes(int gb, int n) { return kTcCols * n * 2 + kTcCols / gb * n * 4; }
+// Entries of four kinds instead of +-1, and the sums kept per block and column: S, and S0 - S for the kinds.
+__host__ __device__ constexpr bool tc_kinds(int gb, int n) { return gb == 128 && n < 64; }
+__host__ __device__ constexpr int tc_pass_bytes(int gb, int n) {
+    return kTcCols * n * 2 + kTcCols / gb * n * (tc_kinds(gb, n) ? 8 : 4);
+}
 
 namespace tc {
 
@@ -156,19 +165,41 @@ __device__ __forceinline__ uint64_t desc(uint32_t addr, int n) {
 
 }  // namespace tc
 
-// Bits p and p + 16 of w as two bf16 values, +1 where set and -1 where not:
-// moved to the sign positions by a product (the multiply pipe is idle here,
-// the logic pipe is what bounds the expansion) and one three-input logic
-// operation.  The factors 2^(15 - p) and the two masks come from the kernel's
-// arguments, so the compiler keeps the product and needs no second operation
-// for a second immediate.
-struct Pm1 {
-    uint32_t mul[16], mask, one;
+// Bits p and p + 16 of w as two bf16 values.  Shifted left by 12 - 4 (p / 4)
+// the two lie at positions 12 + p % 4 of the halves, where one three-input
+// logic operation turns them into numbers:
+//   15: sign of 0.5                        (t & 8000) ^ bf00: set 0.5, clear -0.5
+//   14: top bit of the exponent            t & 4000: 2 or 0
+//   13: second bit, the rest as in 1.0     (t & 2000) | 1f80: 1 or 2^-64
+//   12: third bit, likewise                (t & 1000) | 2f80: 1 or 2^-32
+// so a word takes 3 shifts and 16 logic operations (15 and 16 with one
+// position for all).  The constants come from the kernel's arguments: a second
+// immediate would cost a second operation.
+struct Expand {
+    uint32_t mask[4], fill[4];                              // positions 12, 13, 14, 15
+    uint32_t mul[16];                                       // 2^(15 - p), for pm1
 };
-__device__ __forceinline__ uint32_t pm1(uint32_t w, int p, const Pm1& c, uint32_t mask, uint32_t one) {
-    uint32_t r;
-    asm("lop3.b32 %0, %1, %2, %3, 0x6a;" : "=r"(r) : "r"(p == 15 ? w : w * c.mul[p]), "r"(mask), "r"(one));
-    return r;
+__device__ __forceinline__ void expand16(uint32_t w, const uint32_t (&mask)[4], const uint32_t (&fill)[4], uint32_t (&a)[16]) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const uint32_t t = i == 3 ? w : w << (12 - 4 * i);
+        asm("lop3.b32 %0, %1, %2, %3, 0xea;" : "=r"(a[4 * i]) : "r"(t), "r"(mask[0]), "r"(fill[0]));
+        asm("lop3.b32 %0, %1, %2, %3, 0xea;" : "=r"(a[4 * i + 1]) : "r"(t), "r"(mask[1]), "r"(fill[1]));
+        a[4 * i + 2] = t & mask[2];
+        asm("lop3.b32 %0, %1, %2, %3, 0x6a;" : "=r"(a[4 * i + 3]) : "r"(t), "r"(mask[3]), "r"(fill[3]));
+    }
+}
+// The same pairs as +-1: moved to the sign positions by a product (it runs
+// beside the logic operations) and one logic operation.
+__device__ __forceinline__ void expand16_pm1(uint32_t w, const uint32_t (&mul)[16], uint32_t mask, uint32_t one, uint32_t (&a)[16]) {
+#pragma unroll
+    for (int p = 0; p < 16; ++p)
+        asm("lop3.b32 %0, %1, %2, %3, 0x6a;" : "=r"(a[p]) : "r"(p == 15 ? w : w * mul[p]), "r"(mask), "r"(one));
+}
+// Half of both bf16 values of a pair (exact but for subnormal results).
+__device__ __forceinline__ uint32_t half_pair(uint32_t v) {
+    const __nv_bfloat162 h = __hmul2(*reinterpret_cast<const __nv_bfloat162*>(&v), __floats2bfloat162_rn(0.5f, 0.5f));
+    return *reinterpret_cast<const uint32_t*>(&h);
 }
 
 // Piece 0, 1 or 2 of an fp32 value: three bf16 numbers that add up to it
@@ -190,9 +221,11 @@ __global__ void __launch_bounds__(tc_groups(GB, N) * 160, 1)
 bcq_tc_kernel(const __grid_constant__ CUtensorMap tm_planes, const uint32_t* __restrict__ PLANES,
               const float* __restrict__ ASTAR, const float* __restrict__ ZSTAR, const void* __restrict__ X, int x_bf16,
               float* __restrict__ DST, int64_t out, int n_in, int g, int batch, int n_ks, int sb_per, int tiles,
-              int tmem_cols, int staged, const __grid_constant__ Pm1 pm) {
+              int tmem_cols, int staged, const __grid_constant__ Expand ex) {
     constexpr int NB = kTcCols / GB;                       // scaling blocks of one pass
     constexpr int SBS = tc_sbs(N), SB = tc_stage_bytes(Q, N);
+    constexpr bool KINDS = tc_kinds(GB, N);
+    constexpr int NSUM = KINDS ? 2 : 1;
     extern __shared__ __align__(128) unsigned char tsm[];
     // per warpgroup and buffer: plane expanded (its four warps), products done; per stage: copies landed
     __shared__ __align__(8) unsigned long long ready[kTcMaxGroups][2], done[kTcMaxGroups][2], full[kTcMaxGroups][kTcStages];
@@ -256,7 +289,7 @@ bcq_tc_kernel(const __grid_constant__ CUtensorMap tm_planes, const uint32_t* __r
         const int tok = x_bf16 ? col : col / 3, piece = x_bf16 ? 0 : col - tok * 3;
         const int word = (sb0 + sb) * 4 + tig;
         uint32_t pr[16];                                   // columns p and p + 16 of the word
-        float sum = 0.f;
+        float sum = 0.f, sum0 = 0.f;                       // S, and its columns of the first kind (bits 3, 7, 11, 15)
         if (tok < toks && word < words) {
             const int64_t x0 = (int64_t)(tok0 + tok) * n_in + (int64_t)word * 32;
             if (x_bf16) {
@@ -267,8 +300,6 @@ bcq_tc_kernel(const __grid_constant__ CUtensorMap tm_planes, const uint32_t* __r
                     const uint4 v = __ldg(p + i);
                     u[4 * i] = v.x; u[4 * i + 1] = v.y; u[4 * i + 2] = v.z; u[4 * i + 3] = v.w;
                 }
-#pragma unroll
-                for (int i = 0; i < 16; ++i) sum += __uint_as_float(u[i] << 16) + __uint_as_float(u[i] & 0xffff0000u);
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
                     pr[2 * i] = __byte_perm(u[i], u[i + 8], 0x5410);
@@ -291,12 +322,13 @@ bcq_tc_kernel(const __grid_constant__ CUtensorMap tm_planes, const uint32_t* __r
 #pragma unroll
                     for (int k = 0; k < 4; ++k) {
                         const uint32_t a = cut(lo[k]), b = cut(hi[k]);
-                        sum += __uint_as_float(a & 0xffff0000u) + __uint_as_float(b & 0xffff0000u);
                         pr[4 * i + k] = __byte_perm(a, b, 0x7632);
                     }
                 }
-                if (!(fabsf(sum) < __int_as_float(0x7f800000))) {      // an infinity or a NaN among them
-                    sum = 0.f;
+                uint32_t top = 0;
+#pragma unroll
+                for (int i = 0; i < 16; ++i) top |= ((pr[i] & 0x7f807f80u) + 0x00800080u) & 0x80008000u;
+                if (top != 0) {                             // an infinity or a NaN among them
 #pragma unroll
                     for (int i = 0; i < 4; ++i) {
                         float lo[4], hi[4];
@@ -305,7 +337,6 @@ bcq_tc_kernel(const __grid_constant__ CUtensorMap tm_planes, const uint32_t* __r
 #pragma unroll
                         for (int k = 0; k < 4; ++k) {
                             const uint32_t a = bf16_piece(lo[k], piece), b = bf16_piece(hi[k], piece);
-                            sum += __uint_as_float(a << 16) + __uint_as_float(b << 16);
                             pr[4 * i + k] = a | (b << 16);
                         }
                     }
@@ -315,9 +346,27 @@ bcq_tc_kernel(const __grid_constant__ CUtensorMap tm_planes, const uint32_t* __r
 #pragma unroll
             for (int i = 0; i < 16; ++i) pr[i] = 0u;
         }
-        if (GB >= 64) sum += __shfl_xor_sync(kFull, sum, 1);
-        if (GB >= 128) sum += __shfl_xor_sync(kFull, sum, 2);
-        if (tig % (4 / NB) == 0) sums[(sb * NB + tig / (4 / NB)) * N + col] = sum;
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            const float v = __uint_as_float(pr[i] << 16) + __uint_as_float(pr[i] & 0xffff0000u);
+            if (i % 4 == 3) sum0 += v;
+            else sum += v;
+            if (KINDS && i % 4 == 2) pr[i] = half_pair(pr[i]);
+        }
+        // sum: the columns of the other kinds, S - S0
+        if (GB >= 64) {
+            sum += __shfl_xor_sync(kFull, sum, 1);
+            sum0 += __shfl_xor_sync(kFull, sum0, 1);
+        }
+        if (GB >= 128) {
+            sum += __shfl_xor_sync(kFull, sum, 2);
+            sum0 += __shfl_xor_sync(kFull, sum0, 2);
+        }
+        if (tig % (4 / NB) == 0) {
+            float* d = sums + ((sb * NB + tig / (4 / NB)) * N + col) * NSUM;
+            d[0] = sum + sum0;
+            if (KINDS) d[NSUM - 1] = -sum;
+        }
 #pragma unroll
         for (int v = 0; v < 4; ++v)
             xs[(sb * 16 + tig * 4 + v) * N + col] = make_uint4(pr[4 * v], pr[4 * v + 1], pr[4 * v + 2], pr[4 * v + 3]);
@@ -373,7 +422,9 @@ bcq_tc_kernel(const __grid_constant__ CUtensorMap tm_planes, const uint32_t* __r
     uint32_t phase = 0;                                    // bit b: parity of buffer b's next completion
     int buf = 0, waited = 0;                               // buffer of the next plane; stages waited for
     bool alive = true;
-    const uint32_t mask = pm.mask, one = pm.one;
+    uint32_t mask[4], fill[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) { mask[i] = ex.mask[i]; fill[i] = ex.fill[i]; }
 
     for (int mt = 0; mt < my_tiles && alive && !issuer; ++mt) {
         const int64_t row_raw = (tile0 + wg + (int64_t)mt * n_wg) * kTcRows + wt;
@@ -436,8 +487,8 @@ bcq_tc_kernel(const __grid_constant__ CUtensorMap tm_planes, const uint32_t* __r
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 uint32_t a[16];
-#pragma unroll
-                for (int p = 0; p < 16; ++p) a[p] = pm1(w[i], p, pm, mask, one);
+                if constexpr (KINDS) expand16(w[i], mask, fill, a);
+                else expand16_pm1(w[i], ex.mul, mask[3], fill[3], a);
                 tc::store(tlane + 64 * b + 16 * i, a);
             }
             tc::wait_store();
@@ -474,7 +525,7 @@ bcq_tc_kernel(const __grid_constant__ CUtensorMap tm_planes, const uint32_t* __r
                 tc::fence_after();
 #pragma unroll
                 for (int h = 0; h < NB; ++h) {
-                    const float* S = sums + (sb * NB + h) * N;
+                    const float* S = sums + (sb * NB + h) * N * NSUM;
 #pragma unroll
                     for (int n0 = 0; n0 < N; n0 += 16) {
                         float d[16];
@@ -482,8 +533,10 @@ bcq_tc_kernel(const __grid_constant__ CUtensorMap tm_planes, const uint32_t* __r
 #pragma unroll
                         for (int n = 0; n < 16; ++n) {
                             // the block's terms first, then the running sum: one rounding per pass at its size
-                            if (j == 0) v[n0 + n] = h == 0 ? __fmul_rn(pz[h], S[n0 + n]) : fmaf(pz[h], S[n0 + n], v[n0 + n]);
-                            v[n0 + n] = fmaf(pa[h][j], d[n], v[n0 + n]);
+                            const float* s2 = S + (n0 + n) * NSUM;
+                            if (j == 0) v[n0 + n] = h == 0 ? __fmul_rn(pz[h], s2[0]) : fmaf(pz[h], s2[0], v[n0 + n]);
+                            const float cx = KINDS ? fmaf(2.f, d[n], s2[NSUM - 1]) : d[n];
+                            v[n0 + n] = fmaf(pa[h][j], cx, v[n0 + n]);
                             if (j == Q - 1 && h == NB - 1) acc[n0 + n] += v[n0 + n];
                         }
                     }
@@ -560,7 +613,7 @@ TcPlan tc_plan(int64_t out, int n_in, int chunks, bool staged) {
     for (int w = 1; w <= tc_groups(GB, N); ++w) {
         const int fit = (kTcSmem - 1024 - (staged ? w * kTcStages * tc_stage_bytes(Q, N) : 0)) / tc_pass_bytes(GB, N);
         const int least = (n_sb + fit - 1) / fit;
-        for (int ks = least; ks <= most_ks && ks < least + 8; ++ks) {
+        for (int ks = least; ks <= most_ks && ks < least + 16; ++ks) {
             const int per = (n_sb + ks - 1) / ks, n_ks = (n_sb + per - 1) / per;
             for (int waves = 1; waves <= 2; ++waves) {
                 int64_t n_rb = (int64_t)sms * waves / ((int64_t)n_ks * chunks);
@@ -591,10 +644,9 @@ cudaError_t run_tc(const uint32_t* planes, const float* astar, const float* zsta
     CUtensorMap map = {};
     const bool staged = n_in % kTcCols == 0 && bcq_planes_map(planes, out, n_in, Q, 4 * tc_sbs(N), kTcRows, &map);
     const TcPlan p = tc_plan<Q, GB, N>(out, n_in, chunks, staged);
-    Pm1 pm;
-    for (int i = 0; i < 16; ++i) pm.mul[i] = 1u << (15 - i);
-    pm.mask = 0x80008000u;
-    pm.one = 0xbf80bf80u;
+    Expand ex{{0x10001000u, 0x20002000u, 0x40004000u, 0x80008000u},
+              {0x2f802f80u, 0x1f801f80u, 0u, tc_kinds(GB, N) ? 0xbf00bf00u : 0xbf80bf80u}, {}};
+    for (int i = 0; i < 16; ++i) ex.mul[i] = 1u << (15 - i);
     auto kern = bcq_tc_kernel<Q, GB, N>;
     static std::atomic<int> ready[kMaxDevices] = {};
     int dev = 0;
@@ -610,7 +662,7 @@ cudaError_t run_tc(const uint32_t* planes, const float* astar, const float* zsta
     int smem = 1024 + p.sb_per * tc_pass_bytes(GB, N) + (staged ? p.groups * kTcStages * tc_stage_bytes(Q, N) : 0);
     if (smem < kTcMinSmem) smem = kTcMinSmem;
     e = launch_dependent(kern, dim3((unsigned)(p.n_ks * p.n_rb), (unsigned)chunks), dim3(p.groups * 160), (size_t)smem, st, map, planes, astar, zstar, x, x_bf16, p.n_ks > 1 ? work : y, out, n_in, g, batch,
-                           p.n_ks, p.sb_per, p.tiles, cols, staged ? 1 : 0, pm);
+                           p.n_ks, p.sb_per, p.tiles, cols, staged ? 1 : 0, ex);
     if (e != cudaSuccess || p.n_ks == 1) return e;
     return gemv_reduce(work, y, (int64_t)batch * out, p.n_ks, st);
 }

@@ -1040,11 +1040,11 @@ cudaError_t launch_gemv(const uint32_t* planes, const float* astar, const float*
                         int g, const void* x, int xdtype, int batch, float* y, float* work, cudaStream_t st) {
     // The lookup tables hold one token, so their kernels build them and read
     // the planes once per token; the tensor-core product reads the planes once
-    // for up to 64 columns.  Three tokens and more: 23.6 vs 19.4 us on
-    // 14336 x 4096 (2 tokens: 16.5 vs 19.3), 77 vs 74 on 8192 x 28672 (53 vs
-    // 74), 9.5 vs 8.9 on 1024 x 4096 q = 4 (7.0 vs 8.9), 7.5 vs 6.2 on 256 x
-    // 512 (5.9 vs 6.2).  Two tokens where the 512-column kernels would run:
-    // 31.6 vs 20.4 us on 4096 x 11008, but 8.4 vs 9.0 on 1024 x 8192 g = 512.
+    // for up to 64 columns.  Three tokens and more: 23.6 vs 18.3 us on
+    // 14336 x 4096 (2 tokens: 16.5 vs 18.2), 77 vs 68 on 8192 x 28672 (53 vs
+    // 68), 9.5 vs 8.9 on 1024 x 4096 q = 4 (7.0 vs 8.8), 7.5 vs 6.4 on 256 x
+    // 512 (5.9 vs 6.4).  Two tokens where the 512-column kernels would run:
+    // 31.6 vs 18.8 us on 4096 x 11008, but 8.4 vs 8.6 on 1024 x 8192 g = 512.
     const bool wide = n_in % kWideCols == 0 && g <= 256;
     if (batch >= 3 || (batch == 2 && !wide && out * n_in >= (int64_t(1) << 24)))
         return launch_bcq_tc(planes, astar, zstar, out, n_in, q, g, x, xdtype, batch, y, work, st);
