@@ -323,41 +323,59 @@ __global__ void init_kernel(const void* __restrict__ W, int64_t n_groups, int n_
 // measured): lane l of a warp owns group 32 w + l whole, so no sum needs a
 // shuffle and each group's normal equations are solved once.  During the T
 // rounds x is fixed and only the code words move, so C^T (x - z_B) and C^T C
-// are formed from per-code-word sums of x and counts; a round touches only
-// the elements whose code moved.  Shared memory per warp, element-major so
-// that the 32 lanes touch consecutive words (init_lane_warp_bytes).
+// are formed from per-code-word sums of x and counts (fp64 path: kept over the
+// rounds, an element whose code moves goes from one sum to the other).  Shared
+// memory per warp, element-major so that the 32 lanes touch consecutive words
+// (init_lane_warp_bytes).
 //
-// Where init_kernel sums in fp64 this kernel takes the same values without
-// fp64, and goes back to fp64 wherever it cannot show that they are the same:
-//  * sums of |r| and x: with all values multiples of 2^-k below 2^30 2^-k
+// The fast path of a candidate works on the group's weights in ascending order
+// (sorted once, kept in the group's part of the output S until the end): x is
+// then ascending too, so the codes of a round are intervals of positions
+// between L - 1 boundaries, a round finds the boundaries by binary search and
+// forms its sums from prefix sums of x, and no element is touched.  Its values
+// are those of the fp64 path:
+//  * sums of |r| and x: with all values multiples of 2^-k below 2^44 2^-k
 //    (k per group and candidate; every value is checked), the fp64 sums are
 //    exact in any order, and so are 64-bit integer sums;
 //  * the normal equations: the exact solution N_j / D from integers (Cramer's
 //    rule), rounded to fp32 only where it lies further from a tie of that
-//    rounding than the fp64 elimination can be off (see below);
-//  * the nearest level: a binary search over the midpoints of the sorted
-//    levels where x is further from each of them than the fp32 distances can
-//    be off, else the scan of nearest_rank;
+//    rounding than the fp64 elimination can be off (see below), else the
+//    elimination;
+//  * the nearest level: with X the largest |x|, M the largest |level| and every
+//    gap of distinct levels above 2^-21 (X + M), the test fl|x - l_{r+1}| <
+//    fl|x - l_r| of neighbouring levels is false below the two, true above
+//    them (the gap survives the rounding) and monotonic between them, since
+//    rounding is; so it is monotonic in x and decides between ranks up to r
+//    and above exactly as the scan does.  Equal levels: the scan takes the
+//    lowest of their ranks, the others get no element;
 //  * the candidate's error: an fp32 sum, and the fp64 sums of the candidate
 //    and the kept one only where the two fp32 sums are within their bound.
-// So every output is bit for bit what fp64 gave.  1024 x 4096, q = 3, g = 128,
-// G = 30, T = 15: 15.8 -> 9.2 ms (fp64 pipe 76 % -> 7 % busy; now bound by
-// issue at 1.7 warps per scheduler, half of the lanes idle in the late rounds).
-constexpr int kLaneInitMaxG = 256;
+// Where a value is no such multiple, levels are too close, or z_B moves (G =
+// 1), the warp takes the fp64 path for the candidate.  So every output is bit
+// for bit what fp64 gives.  1024 x 4096, q = 3, g = 128, G = 30, T = 15:
+// 15.8 -> 3.5 ms, with the same shape at q = 2 2.0, q = 4 10.2 and g = 64 5.6
+// ms.  (Rounds that moved element by element instead of boundaries: 8.8 ms,
+// 5.6, 16.3 and 7.1; without the sort network of lane_sorted_levels and with g
+// at run time 3.9 ms.)  Bound by issue and latency: 7 warps per SM, as many
+// as this matrix has groups for and nearly as many as fit in shared memory.
+constexpr int kLaneInitMaxG = 256, kLaneInitMaxWarps = 12;     // 12: 170 registers a thread
 
-// Shared memory of one warp: the per-code sums of x [L][32] (64 bits), x
-// [g][32], the sorted levels [L][32], W^ of the sorted levels [L][32] and the
-// code words [g][32]; rounded up to 16 bytes.
+// Shared memory of one warp: x [g][32], then the prefix sums of x before every
+// fourth element [g / 4][32] (64 bits) or, on the fp64 path, the per-code sums
+// of x [L][32] (fp64) and the code words [g][32].
+__host__ __device__ constexpr size_t init_lane_aux_bytes(int q, int g) {
+    return (size_t)g * 64 > (size_t)g * 32 + ((size_t)256 << q) ? (size_t)g * 64 : (size_t)g * 32 + ((size_t)256 << q);
+}
 __host__ __device__ constexpr size_t init_lane_warp_bytes(int q, int g) {
-    return (((size_t)(1 << q) * 32 * (8 + 4 + 4) + (size_t)g * 32 * (4 + 1)) + 15) & ~size_t(15);
+    return (size_t)g * 128 + init_lane_aux_bytes(q, g);
 }
 
-// Counts of the L code words of one group, BITS bits per code word packed in
+// Counts of the L code words of one group, 16 bits per code word packed in
 // 64-bit registers; c is a compile-time index wherever get() is used, add()
 // takes any c.
-template <int L, int BITS>
+template <int L>
 struct CodeHist {
-    static constexpr int PER = 64 / BITS, NW = (L + PER - 1) / PER;
+    static constexpr int BITS = 16, PER = 64 / BITS, NW = (L + PER - 1) / PER;
     uint64_t h[NW];
     __device__ __forceinline__ CodeHist() {
 #pragma unroll
@@ -373,92 +391,47 @@ struct CodeHist {
     }
 };
 
-// Levels of (a, zb), sorted ascending (ties by code word) into srt_s and
-// registers; cor holds the code word of rank r in bits 4 r .. 4 r + 3, that of
+// Levels of (a, zb), sorted ascending (ties by code word); cor holds the code word of rank r in bits 4 r .. 4 r + 3, that of
 // the lowest rank among equal levels (the one nearest_rank takes).
 template <int Q>
-__device__ __forceinline__ void lane_sorted_levels(const float a[Q], float zb, float* srt_s, int lane,
-                                                   float srt[1 << Q], uint64_t& cor) {
+__device__ __forceinline__ void lane_sorted_levels(const float a[Q], float zb, float srt[1 << Q], uint64_t& cor) {
     constexpr int L = 1 << Q;
-    float lv[L];
-#pragma unroll
-    for (int c = 0; c < L; ++c) lv[c] = level_of<Q>(c, a, zb);
-    cor = 0;
+    int code[L];
 #pragma unroll
     for (int c = 0; c < L; ++c) {
-        int r = 0, first = 0;
-#pragma unroll
-        for (int c2 = 0; c2 < L; ++c2) {
-            r += (lv[c2] < lv[c]) || (lv[c2] == lv[c] && c2 < c);
-            if (c2 < c && lv[c2] == lv[c] && !(first & 16)) first = 16 | c2;     // lowest equal code word
-        }
-        srt_s[r * 32 + lane] = lv[c];
-        cor |= uint64_t((first & 16) ? (first & 15) : c) << (4 * r);
+        srt[c] = level_of<Q>(c, a, zb);
+        code[c] = c;
     }
+    // Batcher's odd-even merge sort (19 exchanges of eight levels, 63 of sixteen)
 #pragma unroll
-    for (int r = 0; r < L; ++r) srt[r] = srt_s[r * 32 + lane];
+    for (int p = 1; p < L; p *= 2)
+#pragma unroll
+        for (int k = p; k >= 1; k /= 2)
+#pragma unroll
+            for (int i = 0; i < L; ++i)
+                if (i >= k % p && (i - k % p) % (2 * k) < k && i + k < L && i / (2 * p) == (i + k) / (2 * p)) {
+                    const float u = srt[i], v = srt[i + k];
+                    const int cu = code[i], cv = code[i + k];
+                    const bool swap = v < u || (v == u && cv < cu);
+                    srt[i] = swap ? v : u;
+                    srt[i + k] = swap ? u : v;
+                    code[i] = swap ? cv : cu;
+                    code[i + k] = swap ? cu : cv;
+                }
+    cor = (uint64_t)code[0];
+    int first = code[0];
+#pragma unroll
+    for (int r = 1; r < L; ++r) {
+        first = srt[r] == srt[r - 1] ? first : code[r];
+        cor |= (uint64_t)first << (4 * r);
+    }
 }
 
-// The search for the nearest level: thresholds t (midpoints of neighbouring
-// sorted levels) and the margin around them inside which the scan decides.
-//
-// With M the largest |level| and X the largest |x| of the group, x further
-// than m = 2^-21 (X + M) from t_r lies on the same side of the exact midpoint
-// (t_r is off by at most 2^-24 M), and where it lies between the two levels
-// the exact distances differ by more than 2 m - 2^-23 M > 2^-23 M, their
-// roundings by at most 2^-24 of their sum (at most 2^-23 M): the rounded
-// distances keep the order.  Beyond both levels they differ by the gap of the
-// levels, and rounding could make them equal only if the gap is below 2^-23
-// (X + M): then no x is sure (m = infinity).  Equal levels have equal
-// distances, and cor names the lowest of their ranks.
-template <int L>
-struct LevelSearch {
-    float t[L - 1], m;
-    __device__ __forceinline__ void set(const float srt[L], float xmax) {
-        const float M = fmaxf(fabsf(srt[0]), fabsf(srt[L - 1]));
-        m = (xmax + M) * 0x1p-21f;
-        bool ok = M < 0x1p100f && xmax < 0x1p100f;          // false also for NaN
-#pragma unroll
-        for (int r = 0; r + 1 < L; ++r) {
-            t[r] = 0.5f * (srt[r] + srt[r + 1]);
-            const float gap = srt[r + 1] - srt[r];
-            ok &= gap == 0.f || gap > m;
-        }
-        if (!ok) m = __int_as_float(0x7f800000);
-    }
-    // Rank of the nearest level; srt_s: the lane's sorted levels in shared memory (for the scan).
-    __device__ __forceinline__ int rank(float x, const float* srt_s) const {
-        float c[L - 1];
-#pragma unroll
-        for (int i = 0; i < L - 1; ++i) c[i] = t[i];
-        int r = 0;
-        float near = __int_as_float(0x7f800000);
-#pragma unroll
-        for (int n = L / 2; n >= 1; n /= 2) {                // 2 n - 1 candidates left, the middle one c[n - 1]
-            const float d = x - c[n - 1];
-            const bool up = d > 0.f;
-            near = fminf(near, fabsf(d));
-            r = 2 * r + (up ? 1 : 0);
-#pragma unroll
-            for (int i = 0; i < n - 1; ++i) c[i] = up ? c[n + i] : c[i];
-        }
-        if (!(near > m)) {
-            float best = fabsf(__fsub_rn(x, srt_s[0]));
-            r = 0;
-#pragma unroll 1
-            for (int k = 1; k < L; ++k) {
-                const float d = fabsf(__fsub_rn(x, srt_s[k * 32]));
-                if (d < best) { best = d; r = k; }
-            }
-        }
-        return r;
-    }
-};
-
-// Exact solution of C^T C alpha = b as integers: N_j / D (D = det, N = adj b).
-// n[i][j] (|n| <= g <= 128) and D fit 32 bits, N 64 bits for |b| < 2^38.
+// Exact solution of C^T C alpha = b as integers: N_j / D (D = det, N = adj b),
+// N_j rounded to fp64 once.  n[i][j] (|n| <= g <= 128) and D fit 32 bits, adj
+// 24; |b| < 2^53, so N_j is formed from two parts of b.
 template <int Q>
-__device__ __forceinline__ int cramer(const int n[Q][Q], const long long b[Q], long long N[Q]) {
+__device__ __forceinline__ int cramer(const int n[Q][Q], const long long b[Q], double N[Q]) {
     auto det2 = [&](int r0, int r1, int c0, int c1) { return n[r0][c0] * n[r1][c1] - n[r0][c1] * n[r1][c0]; };
     auto det3 = [&](int r0, int r1, int r2, int c0, int c1, int c2) {
         return n[r0][c0] * det2(r1, r2, c1, c2) - n[r0][c1] * det2(r1, r2, c0, c2) + n[r0][c2] * det2(r1, r2, c0, c1);
@@ -487,59 +460,82 @@ __device__ __forceinline__ int cramer(const int n[Q][Q], const long long b[Q], l
     for (int j = 0; j < Q; ++j) D += n[0][j] * adj[0][j];
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
-        N[i] = 0;
+        long long lo = 0, hi = 0;
 #pragma unroll
-        for (int j = 0; j < Q; ++j) N[i] += (long long)adj[i][j] * b[j];
+        for (int j = 0; j < Q; ++j) {
+            lo += (long long)adj[i][j] * (b[j] & 0x3ffffff);
+            hi += (long long)adj[i][j] * (b[j] >> 26);
+        }
+        hi += lo >> 26;                                     // |hi| < 2^53
+        N[i] = fma((double)hi, 0x1p26, (double)(lo & 0x3ffffff));
     }
     return D;
 }
 
 template <int Q, typename WT, int G_>
-__global__ void init_lane_kernel(const void* __restrict__ W, int64_t n_groups, int n_in, int G, int T, int clip,
-                                 float* __restrict__ DELTA, float* __restrict__ ZU, float* __restrict__ S,
-                                 float* __restrict__ SR, float* __restrict__ ALPHA, float* __restrict__ ZB,
-                                 uint8_t* __restrict__ CODES) {
-    constexpr int L = 1 << Q;
-    constexpr size_t WARP_BYTES = init_lane_warp_bytes(Q, G_);
-    constexpr bool CRAMER = G_ <= 128;                      // the 32-bit determinant and the 64-bit N_j hold
-    using Hist = CodeHist<L, G_ <= 128 ? 8 : 16>;
+__global__ void __launch_bounds__(kLaneInitMaxWarps * 32, 1)
+    init_lane_kernel(const void* __restrict__ W, int64_t n_groups, int n_in, int G, int T, int clip,
+                     float* __restrict__ DELTA, float* __restrict__ ZU, float* S, float* __restrict__ SR,
+                     float* __restrict__ ALPHA, float* __restrict__ ZB, uint8_t* __restrict__ CODES) {
+    constexpr int g = G_, L = 1 << Q;
+    constexpr size_t WARP_BYTES = init_lane_warp_bytes(Q, g);
+    constexpr bool CRAMER = g <= 128;                                   // where the 32-bit determinant holds
     extern __shared__ __align__(16) unsigned char smem[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     unsigned char* base = smem + (size_t)warp * WARP_BYTES;
-    double* bx = reinterpret_cast<double*>(base);                       // [L][32]; integers where they are exact
-    long long* bi = reinterpret_cast<long long*>(base);
-    float* xs = reinterpret_cast<float*>(bx + L * 32);                  // [G_][32]
-    float* srt_s = xs + G_ * 32;                                        // [L][32]
-    float* wh_s = srt_s + L * 32;                                       // [L][32]
-    uint8_t* cs = reinterpret_cast<uint8_t*>(wh_s + L * 32);            // [G_][32]
+    float* xs = reinterpret_cast<float*>(base);                         // [g][32]
+    unsigned char* aux = base + (size_t)g * 128;
+    long long* pf = reinterpret_cast<long long*>(aux);                  // [g / 4][32]
+    double* bx = reinterpret_cast<double*>(aux);                        // [L][32]
+    uint8_t* cs = aux + (size_t)L * 256;                                // [g][32]
 
     const int64_t grp0 = ((int64_t)blockIdx.x * (blockDim.x >> 5) + warp) * 32;
     if (grp0 >= n_groups) return;                      // whole warp; no block barrier in this kernel
     const int64_t grp_raw = grp0 + lane;
     const bool live = grp_raw < n_groups;
-    const int64_t grp = live ? grp_raw : n_groups - 1; // absent lanes repeat the last group, store nothing
-    const int Gr = n_in / G_;
+    const int64_t grp = live ? grp_raw : n_groups - 1; // absent lanes repeat the last group, store nothing of their own
+    const int Gr = n_in / g;
     const int64_t row = grp / Gr;
-    const int64_t eoff = row * (int64_t)n_in + (grp % Gr) * (int64_t)G_;
+    const int64_t eoff = row * (int64_t)n_in + (grp % Gr) * (int64_t)g;
+    float* ws = S + eoff;                              // the sorted weights until the end
     auto w4 = [&](int i, float (&w)[4]) { WT::unpack(WT::load(W, eoff + i), w); };
     auto X = [&](int i) -> float& { return xs[i * 32 + lane]; };
     auto C = [&](int i) -> uint8_t& { return cs[i * 32 + lane]; };
     auto BX = [&](int c) -> double& { return bx[c * 32 + lane]; };
-    auto BI = [&](int c) -> long long& { return bi[c * 32 + lane]; };
-    const float inf = __int_as_float(0x7f800000);
+    const float inf = __int_as_float(0x7f800000), rg = 1.f / (float)g;    // exact: g is a power of two
 
     float wmin = INFINITY, wmax = -INFINITY;
-    for (int i = 0; i < G_; i += 4) {
+    bool finite = true;
+    for (int i = 0; i < g; i += 4) {
         float w[4];
         w4(i, w);
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             wmin = fminf(wmin, w[k]);
             wmax = fmaxf(wmax, w[k]);
+            finite &= fabsf(w[k]) < inf;
+            X(i + k) = w[k];
         }
     }
     const float top = (float)(L - 1);
     const float rng = fmaxf(__fsub_rn(wmax, wmin), 1e-12f);
+    // the group's weights in ascending order (bitonic network), into ws
+#pragma unroll 1
+    for (int k = 2; k <= g; k *= 2)
+#pragma unroll 1
+        for (int j = k / 2; j >= 1; j /= 2)
+#pragma unroll 4
+            for (int p = 0; p < g / 2; ++p) {
+                const int i = ((p & ~(j - 1)) << 1) | (p & (j - 1));
+                const float u = X(i), v = X(i + j);
+                const bool swap = (u > v) == ((i & k) == 0);
+                X(i) = swap ? v : u;
+                X(i + j) = swap ? u : v;
+            }
+#pragma unroll 4
+    for (int i = 0; i < g; i += 4)
+        *reinterpret_cast<float4*>(ws + i) = make_float4(X(i), X(i + 1), X(i + 2), X(i + 3));
+    auto ws4 = [&](int i, float (&w)[4]) { f4_to(*reinterpret_cast<const float4*>(ws + i), w); };
 
     // The kept candidate, its fp32 error (ef) and its fp64 error (ed, where
     // have_ed); before the first one ed = infinity.
@@ -551,16 +547,15 @@ __global__ void init_lane_kernel(const void* __restrict__ W, int64_t n_groups, i
     for (int j = 0; j < Q; ++j) ba[j] = 0.f;
     float srt[L];
     uint64_t cor;
-    LevelSearch<L> ls;
 
     // fp64 error of a candidate from its own parameters (the values of init_kernel, in the same order)
     auto error64 = [&](float dc, float zc, const float (&a)[Q], float zb) {
         float sv[L];
         uint64_t unused;
-        lane_sorted_levels<Q>(a, zb, wh_s, lane, sv, unused);
+        lane_sorted_levels<Q>(a, zb, sv, unused);
         double e = 0.0;
 #pragma unroll 1
-        for (int i = 0; i < G_; i += 4) {
+        for (int i = 0; i < g; i += 4) {
             float w[4];
             w4(i, w);
 #pragma unroll
@@ -574,101 +569,314 @@ __global__ void init_lane_kernel(const void* __restrict__ W, int64_t n_groups, i
         return e;
     };
 
-    for (int gi = 1; gi <= G; ++gi) {
-        const float gamma = __fdiv_rn((float)gi, (float)G);
-        const float dc = __fdiv_rn(__fmul_rn(gamma, rng), top);
-        float zc;
-        if (clip == UQ_CLIP_FIXED_MIN) zc = __fdiv_rn(-wmin, dc);
-        else if (clip == UQ_CLIP_FIXED_MAX) zc = __fsub_rn(top, __fdiv_rn(wmax, dc));
-        else zc = __fdiv_rn(-__fmul_rn(gamma, wmin), dc);
-        float a[Q], zb = bzb;
-        float xmax = 0.f;
-        bool nan = false;
+    // The fp64 elimination (alpha stays where C^T C is singular).
+    auto solve64 = [&](const int (&ctc)[Q][Q], const double (&cty)[Q], float (&a)[Q]) {
+        long long n64[Q][Q];
+#pragma unroll
+        for (int j = 0; j < Q; ++j)
+#pragma unroll
+            for (int k = 0; k < Q; ++k) n64[j][k] = ctc[j][k];
+        if (!int_singular<Q>(n64)) {
+            double sol[Q];
+            solve_fp64<Q>(n64, cty, sol);
+#pragma unroll
+            for (int j = 0; j < Q; ++j) a[j] = (float)sol[j];
+        }
+    };
+
+    // A candidate's alpha and fp32 error on the fast path.  Whole warp; false
+    // (for every lane) where some lane's group cannot take it.
+    auto fast = [&](float dc, float zc, float zb, float (&a)[Q], float& err) -> bool {
+        float u;
+        const float x0 = transform_x(wmin, 1.f, dc, 1.f, zc, u), x1 = transform_x(wmax, 1.f, dc, 1.f, zc, u);
+        const float xmax = fmaxf(fabsf(x0), fabsf(x1));
+        // Fixed point: values below 2^e in units of 2^-k, k = 44 - e (sums of 256 stay below 2^53;
+        // with 30 bits groups with outliers fail, and the fp64 path of a few makes the kernel last
+        // 9.6 ms where it takes 3.5).
+        const float bound = xmax + fabsf(zb);
+        const int ebits = (int)((__float_as_uint(bound) >> 23) & 0xffu) - 126;      // bound < 2^ebits
+        const int kfix = 44 - ebits;
+        bool ok = finite && x0 == x0 && x1 == x1 && bound < 0x1p60f && bound > 0x1p-60f;
+        const float up = ok ? __int_as_float((127 + kfix) << 23) : 1.f, down = ok ? __int_as_float((127 - kfix) << 23) : 1.f;
+        // v in units of 2^-k, ok left set only where it is a multiple of it: the
+        // leading 20 bits and the rest, both exact.  (The 64-bit conversions run
+        // at the fp64 rate.)
+        const float up_hi = up * 0x1p-24f, down_hi = down * -0x1p24f;
+        auto to_fixed = [&](float v) -> long long {
+            const int hi = __float2int_rn(v * up_hi);
+            const float rest = fmaf((float)hi, down_hi, v) * up;
+            const int lo = __float2int_rn(rest);
+            ok &= (float)lo == rest && (unsigned)(hi + (1 << 20)) <= 1u << 21;
+            return ((long long)hi << 24) + lo;
+        };
+        const long long zbi = to_fixed(zb);
+        if (!__all_sync(kFull, ok)) return false;
+
+        long long total = 0;
 #pragma unroll 2
-        for (int i = 0; i < G_; i += 4) {
+        for (int i = 0; i < g; i += 4) {
+            float w[4];
+            ws4(i, w);
+            pf[(i >> 2) * 32 + lane] = total;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const float x = transform_x(w[k], 1.f, dc, 1.f, zc, u);
+                X(i + k) = x;
+                total += to_fixed(x);
+            }
+        }
+        // --- Algorithm 3: greedy start (one bit at a time); with the last bit the sums of the first round ---
+        long long b[Q];                                     // C^T (x - z_B) in units of 2^-k
+        int ctc[Q][Q];
+#pragma unroll
+        for (int j = 0; j < Q; ++j) b[j] = 0;
+        uint32_t diff[2] = {0u, 0u};                        // elements whose bits j < k differ: 10 bits per pair
+#pragma unroll
+        for (int j = 0; j < Q; ++j) {
+            long long sum = 0;
+#pragma unroll 4
+            for (int i = 0; i < g; ++i) {
+                const float x = X(i);
+                float r = __fsub_rn(x, zb);
+                int c = 0;
+#pragma unroll
+                for (int jj = 0; jj < j; ++jj) {
+                    const bool s1 = r >= 0.f;
+                    c |= s1 ? 1 << jj : 0;
+                    r = __fsub_rn(r, s1 ? a[jj] : -a[jj]);
+                }
+                sum += to_fixed(fabsf(r));
+                if (j == Q - 1) {
+                    c |= r >= 0.f ? 1 << j : 0;
+                    const long long y = to_fixed(x) - zbi;
+#pragma unroll
+                    for (int jj = 0; jj < Q; ++jj) b[jj] += ((c >> jj) & 1) ? y : -y;
+                    int pair = 0;
+#pragma unroll
+                    for (int jj = 0; jj < Q; ++jj)
+#pragma unroll
+                        for (int kk = jj + 1; kk < Q; ++kk, ++pair)
+                            diff[pair / 3] += (uint32_t)(((c >> jj) ^ (c >> kk)) & 1) << (10 * (pair % 3));
+                }
+            }
+            a[j] = __ll2float_rn(sum) * (down * rg);             // powers of two: exact
+        }
+        {
+            int pair = 0;
+#pragma unroll
+            for (int j = 0; j < Q; ++j) {
+                ctc[j][j] = g;
+#pragma unroll
+                for (int k = j + 1; k < Q; ++k, ++pair)
+                    ctc[j][k] = ctc[k][j] = g - 2 * (int)((diff[pair / 3] >> (10 * (pair % 3))) & 1023u);
+            }
+        }
+        if (!__all_sync(kFull, ok)) return false;
+
+        // Boundaries of the ranks in the sorted x: rank r holds the positions [B[r - 1], B[r]).
+        int B[L];
+        auto boundaries = [&]() {
+            lane_sorted_levels<Q>(a, zb, srt, cor);
+            const float M = fmaxf(fabsf(srt[0]), fabsf(srt[L - 1]));
+            const float m = (xmax + M) * 0x1p-21f;
+            ok &= M < 0x1p100f;                             // false also for NaN
+#pragma unroll
+            for (int r = 0; r + 1 < L; ++r) {
+                const float gap = srt[r + 1] - srt[r];
+                ok &= gap == 0.f || gap > m;
+                B[r] = 0;
+            }
+#pragma unroll
+            for (int step = g / 2; step >= 1; step /= 2)
+#pragma unroll
+                for (int r = 0; r + 1 < L; ++r) {
+                    const float x = X(B[r] + step - 1);
+                    if (!(fabsf(__fsub_rn(x, srt[r + 1])) < fabsf(__fsub_rn(x, srt[r])))) B[r] += step;
+                }
+#pragma unroll
+            for (int r = 0; r + 1 < L; ++r) {
+                const float x = X(B[r]);                    // at most g - 1 here
+                if (!(fabsf(__fsub_rn(x, srt[r + 1])) < fabsf(__fsub_rn(x, srt[r])))) B[r] += 1;
+            }
+            B[L - 1] = g;
+#pragma unroll
+            for (int r = L - 2; r >= 0; --r)
+                if (srt[r + 1] == srt[r]) B[r] = B[r + 1];  // the lower of two equal ranks takes all
+        };
+        // Sum of x before position p.
+        auto before = [&](int p) {
+            if (p == g) return total;
+            long long v = pf[(p >> 2) * 32 + lane];
+#pragma unroll
+            for (int k = 0; k < 3; ++k)
+                if (k < (p & 3)) v += to_fixed(X((p & ~3) + k));
+            return v;
+        };
+
+        // --- T rounds of alpha and C ---
+        bool done = false;
+        uint64_t cor_prev = ~uint64_t(0);
+        for (int it = 0; it < T; ++it) {
+            if (!done) {
+                bool solved = false;
+                if constexpr (CRAMER) {
+                    double N[Q];
+                    const int D = cramer<Q>(ctc, b, N);
+                    if (D == 0) {
+                        solved = true;                      // singular: alpha stays
+                    } else {
+                        // The elimination's forward error is at most 2^11 u kappa max|alpha| (n <= 4,
+                        // growth <= 8; kappa, the condition of the positive definite matrix, from its
+                        // trace Q g and determinant), N_j / D as formed here within 2^-51 of itself.
+                        const double rd = (double)down / (double)D;
+                        double sol[Q];
+                        float amax = 0.f, av[Q];
+#pragma unroll
+                        for (int j = 0; j < Q; ++j) {
+                            sol[j] = N[j] * rd;
+                            av[j] = (float)sol[j];
+                            amax = fmaxf(amax, fabsf(av[j]));
+                        }
+                        float kappa = (float)(Q * g);
+#pragma unroll
+                        for (int j = 1; j < Q; ++j) kappa *= (float)(Q * g) / (float)(Q > 1 ? Q - 1 : 1);
+                        kappa = __fdividef(kappa, fabsf((float)D));
+                        bool sure = amax < 0x1p90f;
+#pragma unroll
+                        for (int j = 0; j < Q; ++j) {
+                            const int off = (int)((uint32_t)__double2loint(sol[j]) & 0x1fffffffu) - (1 << 28);   // from a tie
+                            const float need = 2048.f * kappa * __fdividef(amax, fabsf(av[j])) + 16.f;
+                            sure &= fabsf(av[j]) > 0x1p-90f && (float)(off < 0 ? -off : off) > need;
+                        }
+                        if (sure) {
+#pragma unroll
+                            for (int j = 0; j < Q; ++j) a[j] = av[j];
+                            solved = true;
+                        }
+                    }
+                }
+                if (!solved) {
+                    double cty[Q];
+#pragma unroll
+                    for (int j = 0; j < Q; ++j) cty[j] = (double)b[j] * (double)down;      // exact
+                    solve64(ctc, cty, a);
+                }
+                int P[L];
+#pragma unroll
+                for (int r = 0; r < L; ++r) P[r] = it == 0 ? -1 : B[r];
+                boundaries();
+                // the same intervals and codes as in the round before: a fixed point (every
+                // later round would repeat it); a difference in empty ranks only costs a round
+                done = cor == cor_prev;
+                cor_prev = cor;
+#pragma unroll
+                for (int r = 0; r < L; ++r) done &= P[r] == B[r];
+                if (!done) {
+                    long long lo = 0;
+                    int n_lo = 0;
+#pragma unroll
+                    for (int j = 0; j < Q; ++j) {
+                        b[j] = 0;
+#pragma unroll
+                        for (int k = j + 1; k < Q; ++k) ctc[j][k] = 0;
+                    }
+#pragma unroll
+                    for (int r = 0; r < L; ++r) {
+                        const long long hi = r == L - 1 ? total : before(B[r]);
+                        const int n = B[r] - n_lo, c = (int)((cor >> (4 * r)) & 15u);
+                        const long long y = hi - lo - (long long)n * zbi;
+                        lo = hi;
+                        n_lo = B[r];
+#pragma unroll
+                        for (int j = 0; j < Q; ++j) {
+                            b[j] += ((c >> j) & 1) ? y : -y;
+#pragma unroll
+                            for (int k = j + 1; k < Q; ++k) ctc[j][k] += (((c >> j) ^ (c >> k)) & 1) ? -n : n;
+                        }
+                    }
+#pragma unroll
+                    for (int j = 0; j < Q; ++j)
+#pragma unroll
+                        for (int k = 0; k < j; ++k) ctc[j][k] = ctc[k][j];
+                }
+            }
+            if (!__all_sync(kFull, ok)) return false;
+            if (__all_sync(kFull, done)) break;
+        }
+        if (T == 0) boundaries();
+        if (!__all_sync(kFull, ok)) return false;
+
+        // --- candidate error with the full mapping (Eq. 2), s = s_r = 1: the last round's intervals ---
+        float wh[L];
+#pragma unroll
+        for (int r = 0; r < L; ++r) wh[r] = __fmul_rn(dc, __fsub_rn(srt[r], zc));
+        float e4[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 2
+        for (int i = 0; i < g; i += 4) {
+            float w[4];
+            ws4(i, w);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                float h = wh[0];
+#pragma unroll
+                for (int r = 0; r + 1 < L; ++r) h = i + k >= B[r] ? wh[r + 1] : h;
+                const float df = w[k] - h;
+                e4[k] = fmaf(df, df, e4[k]);
+            }
+        }
+        err = (e4[0] + e4[1]) + (e4[2] + e4[3]);
+        return true;
+    };
+
+    // A candidate's alpha and z_B with fp64 sums, element by element in the order of W.
+    auto slow = [&](float dc, float zc, float (&a)[Q], float& zb) {
+#pragma unroll 1
+        for (int i = 0; i < g; i += 4) {
             float w[4];
             w4(i, w);
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 float u;
-                const float x = transform_x(w[k], 1.f, dc, 1.f, zc, u);
-                X(i + k) = x;
+                X(i + k) = transform_x(w[k], 1.f, dc, 1.f, zc, u);
                 C(i + k) = 0;
-                xmax = fmaxf(xmax, fabsf(x));
-                nan |= x != x;
             }
         }
-        // Fixed point: values below 2^e in units of 2^-k, k = 30 - e.
-        const float bound = xmax + fabsf(zb);
-        const int ebits = (int)((__float_as_uint(bound) >> 23) & 0xffu) - 126;      // bound < 2^ebits
-        const int kfix = 30 - ebits;
-        bool fixed = !nan && bound < 0x1p60f && bound > 0x1p-60f;
-        const float up = fixed ? __int_as_float((127 + kfix) << 23) : 1.f, down = fixed ? __int_as_float((127 - kfix) << 23) : 1.f;
-        auto to_fixed = [&](float v) { return __float2int_rn(v * up); };
-        auto is_fixed = [&](float v, int n) { return (float)n == v * up; };
-
         // --- Algorithm 3: greedy start (one bit at a time) ---
 #pragma unroll
         for (int j = 0; j < Q; ++j) {
-            auto residual = [&](int i, int c) {
+            double sabs = 0.0;
+#pragma unroll 1
+            for (int i = 0; i < g; ++i) {
                 float r = __fsub_rn(X(i), zb);
+                const int c = C(i);
 #pragma unroll
                 for (int jj = 0; jj < j; ++jj) r = __fsub_rn(r, ((c >> jj) & 1) ? a[jj] : -a[jj]);
-                return r;
-            };
-            long long sum = 0;
-            bool exact = fixed;
-#pragma unroll 4
-            for (int i = 0; i < G_; ++i) {
-                const int c = C(i);
-                const float r = residual(i, c);
-                const int n = to_fixed(fabsf(r));
-                exact &= is_fixed(fabsf(r), n);
-                sum += n;
+                sabs += (double)fabsf(r);
                 if (r >= 0.f) C(i) = (uint8_t)(c | (1 << j));
             }
-            if (exact) {
-                a[j] = __ll2float_rn(sum) * (down * (1.f / (float)G_));     // powers of two: exact
-            } else {
-                double sabs = 0.0;
-#pragma unroll 1
-                for (int i = 0; i < G_; ++i) sabs += (double)fabsf(residual(i, C(i) & ((1 << j) - 1)));
-                a[j] = (float)(sabs / (double)G_);
-            }
+            a[j] = (float)(sabs / (double)g);
         }
         // Per code word c: the sum of x over the group's elements with code c
         // and their count (hist).  Then C^T (x - z_B) = sum_c s(c) (bx_c - n_c
         // z_B) and C^T C = sum_c n_c s(c) s(c)^T, where s(c) is the sign vector
         // of c; a round only moves the elements whose code changed from one sum
         // to the other.
-        Hist hist;
+        CodeHist<L> hist;
 #pragma unroll
-        for (int c = 0; c < L; ++c) BI(c) = 0;
-        const int zbi = to_fixed(zb);
-        fixed &= is_fixed(zb, zbi) && G > 1;               // z_B moves when G == 1
-#pragma unroll 2
-        for (int i = 0; i < G_; ++i) {
+        for (int c = 0; c < L; ++c) BX(c) = 0.0;
+#pragma unroll 1
+        for (int i = 0; i < g; ++i) {
             const int c = C(i);
-            const float x = X(i);
-            const int n = to_fixed(x);
-            fixed &= is_fixed(x, n);
-            BI(c) += n;
+            BX(c) += (double)X(i);
             hist.add(c, 1);
         }
-        fixed = __all_sync(kFull, fixed);                   // one form of the sums for the warp
-        if (!fixed) {
-#pragma unroll
-            for (int c = 0; c < L; ++c) BX(c) = 0.0;
-#pragma unroll 1
-            for (int i = 0; i < G_; ++i) BX(C(i)) += (double)X(i);
-        }
-
         // --- T rounds of alpha, C (and z_B when G == 1) ---
-        bool more = true;
         for (int it = 0; it < T; ++it) {
             int ctc[Q][Q];
+            double cty[Q];
 #pragma unroll
-            for (int j = 0; j < Q; ++j)
+            for (int j = 0; j < Q; ++j) {
+                cty[j] = 0.0;
 #pragma unroll
                 for (int k = j; k < Q; ++k) {
                     int v = 0;
@@ -676,97 +884,28 @@ __global__ void init_lane_kernel(const void* __restrict__ W, int64_t n_groups, i
                     for (int c = 0; c < L; ++c) v += (((c >> j) ^ (c >> k)) & 1) ? -hist.get(c) : hist.get(c);
                     ctc[j][k] = ctc[k][j] = v;
                 }
-            bool solved = false;
-            if (CRAMER && fixed) {
-                long long b[Q], N[Q];
-#pragma unroll
-                for (int j = 0; j < Q; ++j) b[j] = 0;
-#pragma unroll
-                for (int c = 0; c < L; ++c) {
-                    const long long y = BI(c) - (long long)hist.get(c) * zbi;
-#pragma unroll
-                    for (int j = 0; j < Q; ++j) b[j] += ((c >> j) & 1) ? y : -y;
-                }
-                const int D = cramer<Q>(ctc, b, N);
-                if (D == 0) {
-                    solved = true;                          // singular: alpha stays
-                } else {
-                    // The elimination's forward error is at most 2^11 u kappa max|alpha| (n <= 4,
-                    // growth <= 8; kappa, the condition of the positive definite matrix, from its
-                    // trace Q G_ and determinant), N_j / D as formed here within 2^-51 of itself.
-                    const double rd = (double)down / (double)D;
-                    double sol[Q];
-                    float amax = 0.f, av[Q];
-#pragma unroll
-                    for (int j = 0; j < Q; ++j) {
-                        sol[j] = (double)N[j] * rd;
-                        av[j] = (float)sol[j];
-                        amax = fmaxf(amax, fabsf(av[j]));
-                    }
-                    float kappa = (float)(Q * G_);
-#pragma unroll
-                    for (int j = 1; j < Q; ++j) kappa *= (float)(Q * G_) / (float)(Q > 1 ? Q - 1 : 1);
-                    kappa = __fdividef(kappa, fabsf((float)D));
-                    bool sure = amax < 0x1p90f;
-#pragma unroll
-                    for (int j = 0; j < Q; ++j) {
-                        const int off = (int)((uint32_t)__double2loint(sol[j]) & 0x1fffffffu) - (1 << 28);   // from a tie
-                        const float need = 2048.f * kappa * __fdividef(amax, fabsf(av[j])) + 16.f;
-                        sure &= fabsf(av[j]) > 0x1p-90f && (float)(off < 0 ? -off : off) > need;
-                    }
-                    if (sure) {
-#pragma unroll
-                        for (int j = 0; j < Q; ++j) a[j] = av[j];
-                        solved = true;
-                    }
-                }
             }
-            if (!solved) {
-                double cty[Q];
-                long long n64[Q][Q];
 #pragma unroll
-                for (int j = 0; j < Q; ++j) {
-                    cty[j] = 0.0;
+            for (int c = 0; c < L; ++c) {
+                const double yc = BX(c) - (double)hist.get(c) * (double)zb;
 #pragma unroll
-                    for (int k = 0; k < Q; ++k) n64[j][k] = ctc[j][k];
-                }
-#pragma unroll 1
-                for (int c = 0; c < L; ++c) {
-                    int n = 0;
-#pragma unroll
-                    for (int c2 = 0; c2 < L; ++c2) n = c2 == c ? hist.get(c2) : n;
-                    const double sx = fixed ? (double)BI(c) * (double)down : BX(c);
-                    const double yc = sx - (double)n * (double)zb;
-#pragma unroll
-                    for (int j = 0; j < Q; ++j) cty[j] += ((c >> j) & 1) ? yc : -yc;
-                }
-                if (!int_singular<Q>(n64)) {
-                    double sol[Q];
-                    solve_fp64<Q>(n64, cty, sol);
-#pragma unroll
-                    for (int j = 0; j < Q; ++j) a[j] = (float)sol[j];
-                }
+                for (int j = 0; j < Q; ++j) cty[j] += ((c >> j) & 1) ? yc : -yc;
             }
-            lane_sorted_levels<Q>(a, zb, srt_s, lane, srt, cor);
-            ls.set(srt, xmax);
+            solve64(ctc, cty, a);
+            lane_sorted_levels<Q>(a, zb, srt, cor);
             bool moved = false;
-#pragma unroll 4
-            for (int i = 0; i < G_; ++i) {
+#pragma unroll 1
+            for (int i = 0; i < g; ++i) {
+                float m;
                 const float x = X(i);
-                const int r = ls.rank(x, srt_s + lane);
+                const int r = nearest_rank<L>(x, srt, m);
                 const int c = (int)((cor >> (4 * r)) & 15u);
                 const int old = C(i);
                 if (c != old) {
                     moved = true;
-                    if (fixed) {
-                        const int n = to_fixed(x);
-                        BI(old) -= n;
-                        BI(c) += n;
-                    } else {
-                        const double xd = (double)x;
-                        BX(old) -= xd;
-                        BX(c) += xd;
-                    }
+                    const double xd = (double)x;
+                    BX(old) -= xd;
+                    BX(c) += xd;
                     hist.add(old, -1);
                     hist.add(c, 1);
                     C(i) = (uint8_t)c;
@@ -774,7 +913,7 @@ __global__ void init_lane_kernel(const void* __restrict__ W, int64_t n_groups, i
             }
             const float zb_prev = zb;
             if (G == 1) {
-                // z_B = mean of x - C alpha = sum_c (bx_c - n_c (s(c) . alpha)) / g (fp64 sums: not fixed)
+                // z_B = mean of x - C alpha = sum_c (bx_c - n_c (s(c) . alpha)) / g
                 double sres = 0.0;
 #pragma unroll
                 for (int c = 0; c < L; ++c) {
@@ -783,35 +922,33 @@ __global__ void init_lane_kernel(const void* __restrict__ W, int64_t n_groups, i
                     for (int j = 0; j < Q; ++j) ca += ((c >> j) & 1) ? (double)a[j] : -(double)a[j];
                     sres += BX(c) - (double)hist.get(c) * ca;
                 }
-                zb = (float)(sres / (double)G_);
+                zb = (float)(sres / (double)g);
             }
             // No code moved (and z_B did not either): the next round would
             // solve the same system, get the same alpha and the same codes, so
             // every remaining round repeats this state bit for bit.
-            more = moved || __float_as_uint(zb) != __float_as_uint(zb_prev);
-            if (!more) break;
+            if (!moved && __float_as_uint(zb) == __float_as_uint(zb_prev)) break;
         }
+    };
 
-        // --- candidate error with the full mapping (Eq. 2), s = s_r = 1 ---
-        lane_sorted_levels<Q>(a, zb, srt_s, lane, srt, cor);
-        ls.set(srt, xmax);
-#pragma unroll
-        for (int r = 0; r < L; ++r) wh_s[r * 32 + lane] = __fmul_rn(dc, __fsub_rn(srt[r], zc));
-        float e4[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll 2
-        for (int i = 0; i < G_; i += 4) {
-            float w[4];
-            w4(i, w);
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const float df = w[k] - wh_s[ls.rank(X(i + k), srt_s + lane) * 32 + lane];
-                e4[k] = fmaf(df, df, e4[k]);
-            }
+    for (int gi = 1; gi <= G; ++gi) {
+        const float gamma = __fdiv_rn((float)gi, (float)G);
+        const float dc = __fdiv_rn(__fmul_rn(gamma, rng), top);
+        float zc;
+        if (clip == UQ_CLIP_FIXED_MIN) zc = __fdiv_rn(-wmin, dc);
+        else if (clip == UQ_CLIP_FIXED_MAX) zc = __fsub_rn(top, __fdiv_rn(wmax, dc));
+        else zc = __fdiv_rn(-__fmul_rn(gamma, wmin), dc);
+        float a[Q], zb = bzb, e = inf;
+        __syncwarp();
+        const bool found = G > 1 && fast(dc, zc, zb, a, e);
+        __syncwarp();
+        if (!found) {
+            e = inf;
+            slow(dc, zc, a, zb);                       // (its code words share the prefix sums' memory)
         }
-        // Within 2^-23 per square and 2^-24 per addition of the exact sum (at
-        // most 66 of them): 5e-6; a square below 2^-126 may be lost, so the sum
-        // has to be well above 256 of those.
-        const float e = (e4[0] + e4[1]) + (e4[2] + e4[3]);
+        // The fp32 error is within 2^-23 per square and 2^-24 per addition of
+        // the exact sum (at most 66 of them): 5e-6; a square below 2^-126 may be
+        // lost, so the sum has to be well above 256 of those.
         const bool usable = e > 0x1p-90f && e < inf;
         bool take;
         if (usable && (e * 1.00001f < ef * 0.99999f) && (ef < inf || !(ed < INFINITY))) {
@@ -838,7 +975,8 @@ __global__ void init_lane_kernel(const void* __restrict__ W, int64_t n_groups, i
         }
     }
 
-    lane_sorted_levels<Q>(ba, bzb, srt_s, lane, srt, cor);
+    lane_sorted_levels<Q>(ba, bzb, srt, cor);
+    __syncwarp();                                      // absent lanes read the last group's sorted weights until here
     if (!live) return;                                 // no warp-wide operation follows
     DELTA[grp] = bd;
     ZU[grp] = bz;
@@ -847,7 +985,7 @@ __global__ void init_lane_kernel(const void* __restrict__ W, int64_t n_groups, i
     for (int j = 0; j < Q; ++j) ALPHA[grp * Q + j] = ba[j];
     if (grp % Gr == 0) SR[row] = 1.f;
 #pragma unroll 2
-    for (int i = 0; i < G_; i += 4) {
+    for (int i = 0; i < g; i += 4) {
         float w[4];
         w4(i, w);
         uint32_t c4 = 0;
@@ -866,9 +1004,10 @@ template <int Q, typename WT, int G_>
 static cudaError_t run_init_lane(const Shape& sh, const void* W, int G, int T, int clip, uq_params p,
                                  uint8_t* codes, cudaStream_t st) {
     constexpr size_t warp_bytes = init_lane_warp_bytes(Q, G_);
-    // as many warps as fit in the 227 KB a block may opt in to, at most 16
-    constexpr int most = (int)((227 * 1024) / warp_bytes) > 16 ? 16 : (int)((227 * 1024) / warp_bytes);
-    static_assert(most >= 1, "one warp's tables must fit");
+    // as many warps as fit in the 227 KB a block may opt in to, at most 12
+    constexpr int fit = (int)((227 * 1024) / warp_bytes);
+    static_assert(fit >= 1, "one warp's tables must fit");
+    constexpr int most = fit > kLaneInitMaxWarps ? kLaneInitMaxWarps : fit;
     const int64_t n_groups = sh.out * (int64_t)(sh.n_in / G_);
     // ... but no more than spreads a small matrix over every SM
     const int64_t spread = ((n_groups + 31) / 32 + sm_count() - 1) / sm_count();
@@ -879,8 +1018,8 @@ static cudaError_t run_init_lane(const Shape& sh, const void* W, int G, int T, i
     if (e != cudaSuccess) return e;
     const int64_t per_block = (int64_t)wpb * 32;
     const int64_t blocks = (n_groups + per_block - 1) / per_block;
-    kern<<<dim3((unsigned)blocks), wpb * 32, dyn, st>>>(W, n_groups, sh.n_in, G, T, clip, p.delta, p.zu, p.s, p.sr,
-                                                       p.alpha, p.zb, codes);
+    kern<<<dim3((unsigned)blocks), wpb * 32, dyn, st>>>(W, n_groups, sh.n_in, G, T, clip, p.delta, p.zu, p.s,
+                                                       p.sr, p.alpha, p.zb, codes);
     return cudaGetLastError();
 }
 
@@ -890,7 +1029,7 @@ static cudaError_t run_init(const Shape& sh, const void* W, int G, int T, int cl
     if (sh.g == 32) return run_init_lane<Q, WT, 32>(sh, W, G, T, clip, p, codes, st);
     if (sh.g == 64) return run_init_lane<Q, WT, 64>(sh, W, G, T, clip, p, codes, st);
     if (sh.g == 128) return run_init_lane<Q, WT, 128>(sh, W, G, T, clip, p, codes, st);
-    if (sh.g == kLaneInitMaxG) return run_init_lane<Q, WT, 256>(sh, W, G, T, clip, p, codes, st);
+    if (sh.g == 256) return run_init_lane<Q, WT, 256>(sh, W, G, T, clip, p, codes, st);
     const int64_t n_groups = sh.out * (int64_t)(sh.n_in / sh.g);
     const size_t per_warp = (size_t)sh.g * (sizeof(float) + 1);
     int wpc = (int)((96 * 1024) / per_warp);
