@@ -499,6 +499,15 @@ __device__ __forceinline__ void unit_full_iv(const SortTab<Q, NS>& t, float4 (*i
     __syncwarp();
 }
 
+// Where the full mapping of whole units searches; else it scans the levels
+// (full_scan4).  The interval tables cost a unit about what the scan of a few
+// levels does: 8192 x 4096, bf16, scan vs search: q = 4 g = 32, 64, 128: 233
+// vs 204, 185 vs 166, 165 vs 102 us; q = 3 g = 128: 92 vs 79, but g = 64: 100
+// vs 104, g = 32: 119 vs 127; q = 2 g = 64: 63 vs 72, q = 1 g = 32: 69 vs 81.
+// (14336 x 4096, q = 3, g = 128: 168 -> 133 us, q = 4: 294 -> 172 us.)
+template <int Q, int G_>
+constexpr bool kFullSearch = Q == 4 || (Q == 3 && G_ >= 128);
+
 // Every fourth midpoint of a group (none for L <= 4).
 template <int L>
 struct FullKeys {
@@ -553,6 +562,21 @@ __device__ __forceinline__ uint32_t full_vec4(const float w[4], const float s4[4
             code = t.cor[sub][br];
         }
         nc |= code << (8 * kq);
+    }
+    return nc;
+}
+
+// The same by the scan: IEEE x, nearest of the group's sorted levels srt (in registers).
+template <int Q, int NS>
+__device__ __forceinline__ uint32_t full_scan4(const float w[4], const float s4[4], const SortTab<Q, NS>& t,
+                                               const float srt[1 << Q], int sub, float dl, float sr, float zu, float o[4]) {
+    uint32_t nc = 0;
+#pragma unroll
+    for (int kq = 0; kq < 4; ++kq) {
+        float u, m;
+        const int r = nearest_rank<(1 << Q)>(transform_x(w[kq], s4[kq], dl, sr, zu, u), srt, m);
+        o[kq] = __fmul_rn(dl, __fsub_rn(m, zu));
+        nc |= (uint32_t)t.cor[sub][r] << (8 * kq);
     }
     return nc;
 }

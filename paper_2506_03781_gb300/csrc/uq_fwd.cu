@@ -1,8 +1,10 @@
 // Forward quantizer: Q*_IF (Eq. 3, local and periodic mapping of
 // Algorithm 4) and Q_IF (Eq. 2, full mapping).
 //
-// The kernel here takes the groups of more than 512 elements and of 384; the
-// pipelined kernels of uq_stream.cu and uq_ragged_fwd.cu take every other g.
+// The kernel here takes the groups of more than 512 elements and of 384, and
+// the full mapping of rows that are no whole number of work units where it is
+// the faster one (ragged_full_ok); the pipelined kernels of uq_stream.cu and
+// uq_ragged_fwd.cu take everything else.
 //
 // Per warp and work unit (NG whole groups, see uq_common.cuh): the lanes
 // issue their vector loads (W, s, codes) first, then build the unit's group
@@ -147,17 +149,28 @@ static cudaError_t run_fwd(const Shape& sh, const void* W, uq_params p, uint8_t*
         W, p.s, p.sr, p.delta, p.zu, p.alpha, p.zb, codes, what, sh.out, sh.n_in, sh.g, R, mode);
 }
 
+template <int Q, typename WT>
+static cudaError_t fwd_g(const Shape& sh, const void* W, uq_params p, uint8_t* codes, int mode, float* what,
+                         cudaStream_t st) {
+    switch (lanes_per_group(sh.g)) {
+        case 4: return run_fwd<Q, WT, 4>(sh, W, p, codes, mode, what, st);
+        case 8: return run_fwd<Q, WT, 8>(sh, W, p, codes, mode, what, st);
+        default: return run_fwd<Q, WT, 32>(sh, W, p, codes, mode, what, st);
+    }
+}
+
 template <int Q>
 static cudaError_t fwd_w(const Shape& sh, const void* W, uq_params p, uint8_t* codes, int mode, float* what,
                          cudaStream_t st) {
-    if (sh.wdtype == UQ_W_BF16) return run_fwd<Q, WBF16, 32>(sh, W, p, codes, mode, what, st);
-    return run_fwd<Q, WF32, 32>(sh, W, p, codes, mode, what, st);
+    if (sh.wdtype == UQ_W_BF16) return fwd_g<Q, WBF16>(sh, W, p, codes, mode, what, st);
+    return fwd_g<Q, WF32>(sh, W, p, codes, mode, what, st);
 }
 
 cudaError_t launch_fwd(const Shape& sh, const void* W, uq_params p, uint8_t* codes, int mode, float* what,
                        cudaStream_t st) {
     if (stream_path_ok(sh)) return launch_fwd_stream(sh, W, p, codes, mode, what, st);
-    if (ragged_path_ok(sh)) return launch_fwd_ragged(sh, W, p, codes, mode, what, st);
+    if (ragged_path_ok(sh) && (mode != FWD_FULL || ragged_full_ok(sh.q, sh.g)))
+        return launch_fwd_ragged(sh, W, p, codes, mode, what, st);
     switch (sh.q) {
         case 1: return fwd_w<1>(sh, W, p, codes, mode, what, st);
         case 2: return fwd_w<2>(sh, W, p, codes, mode, what, st);

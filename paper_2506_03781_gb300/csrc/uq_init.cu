@@ -1029,7 +1029,7 @@ static cudaError_t run_init(const Shape& sh, const void* W, int G, int T, int cl
     if (sh.g == 32) return run_init_lane<Q, WT, 32>(sh, W, G, T, clip, p, codes, st);
     if (sh.g == 64) return run_init_lane<Q, WT, 64>(sh, W, G, T, clip, p, codes, st);
     if (sh.g == 128) return run_init_lane<Q, WT, 128>(sh, W, G, T, clip, p, codes, st);
-    if (sh.g == 256) return run_init_lane<Q, WT, 256>(sh, W, G, T, clip, p, codes, st);
+    if (sh.g == kLaneInitMaxG) return run_init_lane<Q, WT, kLaneInitMaxG>(sh, W, G, T, clip, p, codes, st);
     const int64_t n_groups = sh.out * (int64_t)(sh.n_in / sh.g);
     const size_t per_warp = (size_t)sh.g * (sizeof(float) + 1);
     int wpc = (int)((96 * 1024) / per_warp);

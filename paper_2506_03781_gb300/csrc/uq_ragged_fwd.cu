@@ -168,11 +168,14 @@ template <int Q, int G_>
 static cudaError_t ragged_fwd_g(const Shape& sh, const void* W, uq_params p, uint8_t* codes, int mode, float* what,
                                 cudaStream_t st) {
     if (mode == FWD_KEEP) return run_ragged_fwd<Q, WBF16, G_, FWD_KEEP>(sh, W, p, codes, what, st);
-    if (sh.wdtype == UQ_W_BF16)
-        return mode == FWD_REMAP ? run_ragged_fwd<Q, WBF16, G_, FWD_REMAP>(sh, W, p, codes, what, st)
-                                 : run_ragged_fwd<Q, WBF16, G_, FWD_FULL>(sh, W, p, codes, what, st);
-    return mode == FWD_REMAP ? run_ragged_fwd<Q, WF32, G_, FWD_REMAP>(sh, W, p, codes, what, st)
-                             : run_ragged_fwd<Q, WF32, G_, FWD_FULL>(sh, W, p, codes, what, st);
+    const bool bf16 = sh.wdtype == UQ_W_BF16;
+    if (mode == FWD_REMAP)
+        return bf16 ? run_ragged_fwd<Q, WBF16, G_, FWD_REMAP>(sh, W, p, codes, what, st)
+                    : run_ragged_fwd<Q, WF32, G_, FWD_REMAP>(sh, W, p, codes, what, st);
+    if constexpr (ragged_full_ok(Q, G_))
+        return bf16 ? run_ragged_fwd<Q, WBF16, G_, FWD_FULL>(sh, W, p, codes, what, st)
+                    : run_ragged_fwd<Q, WF32, G_, FWD_FULL>(sh, W, p, codes, what, st);
+    return cudaErrorInvalidValue;                        // launch_fwd sends the rest to its own kernel
 }
 
 template <int Q>

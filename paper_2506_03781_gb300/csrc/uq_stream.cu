@@ -287,8 +287,9 @@ fwd_stream_kernel(const void* __restrict__ W, const float* __restrict__ S, const
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ __align__(8) unsigned long long bars[kWarps][NST];
     __shared__ SortTab<Q, NG> tabs[kWarps];
-    __shared__ float4 ivs[kWarps][NG][L];                        // intervals of the remap or of the full mapping
-    __shared__ __align__(16) float ths[kWarps][mode == FWD_FULL ? NG : 1][L];      // midpoints of the full mapping
+    constexpr bool search = mode == FWD_FULL && kFullSearch<Q, G_>;
+    __shared__ float4 ivs[kWarps][mode != FWD_FULL || search ? NG : 1][L];         // intervals of the remap or of the search
+    __shared__ __align__(16) float ths[kWarps][search ? NG : 1][L];                // midpoints of the search
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int sub = lane / LPG, li = lane % LPG;
     const int U = n_in / UE, Gr = n_in / G_;
@@ -345,13 +346,18 @@ fwd_stream_kernel(const void* __restrict__ W, const float* __restrict__ S, const
                 unit_remap_iv<Q, NG>(t, ivs[warp], lane, pd, pz);
             } else if constexpr (mode == FWD_FULL) {
                 unit_sort<Q, NG, false>(t, lane);
-                unit_full_iv<Q, NG>(t, ivs[warp], ths[warp], lane, pd, pz, NG);
+                if constexpr (search) unit_full_iv<Q, NG>(t, ivs[warp], ths[warp], lane, pd, pz, NG);
             }
             const float dl = pd[sub], zu = pz[sub];
             const float sr = __ldg(SR + row);
             const int64_t ebase = row * n_in + (int64_t)it.unit(cc.j) * UE;
             FullKeys<L> keys;
-            if constexpr (mode == FWD_FULL) keys.load(ths[warp][sub]);
+            if constexpr (search) keys.load(ths[warp][sub]);
+            float srt[L];
+            if constexpr (mode == FWD_FULL && !search) {
+#pragma unroll
+                for (int r = 0; r < L; ++r) srt[r] = t.srt[sub][r];
+            }
 #pragma unroll
             for (int v = 0; v < NV; ++v) {
                 const int el = sub * G_ + 4 * li + 4 * LPG * v;
@@ -365,6 +371,8 @@ fwd_stream_kernel(const void* __restrict__ W, const float* __restrict__ S, const
                     f4_to(*reinterpret_cast<const float4*>(st + St::OFF_S + el * 4), s4);
                     if constexpr (mode == FWD_REMAP) {
                         nc = remap_vec4<Q, NG>(w, s4, cv, t, ivs[warp], sub, dl, sr, zu, o);
+                    } else if constexpr (!search) {
+                        nc = full_scan4<Q, NG>(w, s4, t, srt, sub, dl, sr, zu, o);
                     } else {
                         nc = full_vec4<Q, NG>(w, s4, t, ivs[warp], ths[warp], keys, sub, dl, sr, zu, o);
                     }
