@@ -49,7 +49,7 @@
 // which runs at half rate.  14336 x 4096, q = 3, g = 128, bf16: 64 tokens 447
 // -> 37.9 us (per-token lookup tables before), 16 tokens 114 -> 18.8 us, 4
 // tokens 30.4 -> 18.3 us (19.4 with +-1 entries); 8192 x 28672, 4 fp32 tokens:
-// 99.8 -> 68.1 us (76.4).  The same product with mma.sync and fragments in
+// 99.8 -> 70.2 us (76.4).  The same product with mma.sync and fragments in
 // registers took 72.5, 28.2, 20.6 and 108 us: every lane of a quad repeats
 // the loads and the scaling, and 64 columns are bound by that pipe (38 us).
 // Error against 64 bits: 0.6e-7 to 1.3e-7, the lookup tables' 0.7e-7 to 1.7e-7.
@@ -419,6 +419,7 @@ bcq_tc_kernel(const __grid_constant__ CUtensorMap tm_planes, const uint32_t* __r
     const int64_t pstride = out * words;
     const int gdiv = g > kTcCols ? g / kTcCols : 1;        // passes per group
     const bool vec = g <= kTcCols && (Gr & 3) == 0;        // four groups of a row are 16-byte aligned
+    const bool vec2 = gdiv == 2 && (Gr & 1) == 0;          // two groups of two passes each, 8-byte aligned
     uint32_t phase = 0;                                    // bit b: parity of buffer b's next completion
     int buf = 0, waited = 0;                               // buffer of the next plane; stages waited for
     bool alive = true;
@@ -447,6 +448,25 @@ bcq_tc_kernel(const __grid_constant__ CUtensorMap tm_planes, const uint32_t* __r
 #pragma unroll
                         for (int j = 0; j < Q; ++j) pa[k][j] = f[k * Q + j];
                     f4_to(__ldg(reinterpret_cast<const float4*>(ZSTAR + row * Gr + b0)), pz);
+                }
+            } else if (vec2) {                             // (value by value: 8192 x 8192, 4 tokens 32.5 vs 23.7 us)
+                const int grp = b0 >> 1;
+                if (grp < Gr) {
+                    const float2* a2 = reinterpret_cast<const float2*>(ASTAR + (row * Gr + grp) * Q);
+                    float f[2 * Q];
+#pragma unroll
+                    for (int i = 0; i < Q; ++i) {
+                        const float2 t2 = __ldg(a2 + i);
+                        f[2 * i] = t2.x;
+                        f[2 * i + 1] = t2.y;
+                    }
+                    const float2 z2 = __ldg(reinterpret_cast<const float2*>(ZSTAR + row * Gr + grp));
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        pz[k] = k < 2 ? z2.x : z2.y;
+#pragma unroll
+                        for (int j = 0; j < Q; ++j) pa[k][j] = f[(k >> 1) * Q + j];
+                    }
                 }
             } else {
 #pragma unroll

@@ -1040,13 +1040,17 @@ cudaError_t launch_gemv(const uint32_t* planes, const float* astar, const float*
                         int g, const void* x, int xdtype, int batch, float* y, float* work, cudaStream_t st) {
     // The lookup tables hold one token, so their kernels build them and read
     // the planes once per token; the tensor-core product reads the planes once
-    // for up to 64 columns.  Three tokens and more: 23.6 vs 18.3 us on
-    // 14336 x 4096 (2 tokens: 16.5 vs 18.2), 77 vs 68 on 8192 x 28672 (53 vs
-    // 68), 9.5 vs 8.9 on 1024 x 4096 q = 4 (7.0 vs 8.8), 7.5 vs 6.4 on 256 x
-    // 512 (5.9 vs 6.4).  Two tokens where the 512-column kernels would run:
-    // 31.6 vs 18.8 us on 4096 x 11008, but 8.4 vs 8.6 on 1024 x 8192 g = 512.
-    const bool wide = n_in % kWideCols == 0 && g <= 256;
-    if (batch >= 3 || (batch == 2 && !wide && out * n_in >= (int64_t(1) << 24)))
+    // for up to 64 columns.  Four tokens and more: 30.3 vs 18.3 us on 14336 x
+    // 4096, 32 vs 24 on 8192 x 8192, 12.0 vs 11.8 on 1024 x 4096 g = 32 q = 4.
+    // Three: 23.5 vs 18.2 us on 14336 x 4096 (2 tokens: 16.4 vs 18.2), 77 vs 68
+    // on 8192 x 28672 (53 vs 68), 7.2 vs 5.8 on 256 x 512; but with the blocks
+    // of smaller groups 27.1 vs 29.7 on 8192 x 8192 g = 64, 9.6 vs 10.8 on 1024
+    // x 4096 g = 32 q = 4, and 9.7 vs 10.4 on 100 x 8192 g = 512 q = 4.
+    // Two tokens where the 512-column kernels would run: 35.1 vs 20.2 us on
+    // 4096 x 11008 g = 64, but 8.4 vs 8.6 on 1024 x 8192 g = 512.
+    const bool wide = n_in % kWideCols == 0 && g <= 256, large = out * n_in >= (int64_t(1) << 24);
+    const bool three = wide ? g >= 128 : large || q < 4 || g <= 256;
+    if (batch >= 4 || (batch == 3 && three) || (batch == 2 && !wide && large))
         return launch_bcq_tc(planes, astar, zstar, out, n_in, q, g, x, xdtype, batch, y, work, st);
     switch (q) {
         case 1: return gemv_x<1>(planes, astar, zstar, out, n_in, g, x, xdtype, batch, y, work, st);
