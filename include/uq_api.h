@@ -399,7 +399,7 @@ uq_status uq_export_bcq_half(const void* W, uq_wdtype wdtype, int64_t out, int64
  * One or two tokens: the columns are split into tiles, 1024 columns (32 per
  * lane) when in is a multiple of 1024 and g <= 256, else 512; each tile's
  * contribution is formed from per-8-column partial sums of x (one table
- * lookup per plane byte).  Three tokens and more (and two of a large matrix
+ * lookup per plane byte).  Four tokens and more (and fewer of a large matrix
  * that the 1024-column tiles do not take): a +-1 matrix product per plane on
  * the tensor cores, the activations as bf16 values (an fp32 one as the exact
  * sum of three), fp32 sums scaled by alpha* per group.  Partial sums of tiles

@@ -1029,9 +1029,10 @@ static cudaError_t run_init(const Shape& sh, const void* W, int G, int T, int cl
     if (sh.g == 32) return run_init_lane<Q, WT, 32>(sh, W, G, T, clip, p, codes, st);
     if (sh.g == 64) return run_init_lane<Q, WT, 64>(sh, W, G, T, clip, p, codes, st);
     if (sh.g == 128) return run_init_lane<Q, WT, 128>(sh, W, G, T, clip, p, codes, st);
-    // 256 elements and q = 4 on so few groups that a warp each is one wave: 7.9
-    // vs 9.2 ms on 16 x 4096 (at 16384 groups and q = 3 54 vs 5.7 ms)
-    const bool few = Q == 4 && sh.g == kLaneInitMaxG && sh.out * (int64_t)(sh.n_in / sh.g) <= 1024;
+    // A warp each for so few groups of 256 that they are one wave of blocks, of
+    // as long a chain as a lane's from q = 3 on: 256 to 1152 groups 4.5 vs 4.7
+    // to 5.2 ms at q = 3, 7.9 vs 9.2 to 10.0 ms at q = 4 (16384: 54 vs 5.7 ms).
+    const bool few = Q >= 3 && sh.g == kLaneInitMaxG && sh.out * (int64_t)(sh.n_in / sh.g) <= 8 * sm_count();
     if (sh.g == kLaneInitMaxG && !few) return run_init_lane<Q, WT, kLaneInitMaxG>(sh, W, G, T, clip, p, codes, st);
     const int64_t n_groups = sh.out * (int64_t)(sh.n_in / sh.g);
     const size_t per_warp = (size_t)sh.g * (sizeof(float) + 1);

@@ -171,6 +171,22 @@ def test_init_groups_outside_the_fast_paths(q, g):
     C.check_init(W, q, g, 9, api.CLIP_FIXED_MIN, got, C.host(codes), ref, errs, chosen, f"outside q={q} g={g}")
 
 
+@pytest.mark.parametrize("q", [3, 4])
+def test_init_groups_of_256_with_a_lane_each(q):
+    """More groups of 256 than one wave of a warp each (which few groups take)."""
+    g, out, Gr = 256, 25, 50
+    groups = out * Gr
+    assert groups > 8 * torch.cuda.get_device_properties(0).multi_processor_count
+    rng = np.random.default_rng(q)
+    raw, W = synth.bf16_round((rng.standard_t(4, (out, Gr * g)) * 0.014).astype(np.float32))
+    p = api.empty_params(out, Gr * g, q, g, C.dev())
+    codes = torch.empty(out, Gr * g, dtype=torch.uint8, device=C.dev())
+    api.uq_init_params(api.weights_tensor(raw, C.dev()), q, g, p, codes, G=4, T=3)
+    ref, errs, chosen = O.unified_init(W, q, g, G=4, T=3, return_errors=True)
+    got = {k: C.host(v) for k, v in p.items()}
+    assert C.check_init(W, q, g, 4, api.CLIP_FIXED_MIN, got, C.host(codes), ref, errs, chosen, f"lanes q={q}") == 1.0
+
+
 def test_edge_level_ties_negative_alpha_and_high_code_bits():
     """alpha_1 == alpha_2 makes two code words share a level (ties in the sort
     and in the mapping); a negative alpha reverses part of the order; code
