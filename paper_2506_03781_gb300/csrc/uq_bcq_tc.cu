@@ -40,8 +40,11 @@
 // Split: block (slice, row block) keeps one column slice of all tokens of its
 // chunk and walks its 128-row tiles.  With one slice the result is y itself,
 // else the slices go to the caller's workspace [slice][token][row] and are
-// summed in order by a second kernel.  Every wait is bounded.  Deterministic;
-// no atomics on outputs.
+// summed in order by a second kernel.  Every wait on a barrier is bounded; the
+// wait for the work ahead on the stream and the allocation of tensor memory are
+// the hardware's, and the order of the two (see the kernel) lets no block hold
+// tensor memory that a kernel it waits for needs.  Deterministic; no atomics on
+// outputs.
 //
 // What bounds it: a plane of 128 x 128 takes the tensor cores 256 clocks with
 // 64 columns (measured 272) and 197 with 16, a warpgroup 1270 (700 to expand,
@@ -248,9 +251,6 @@ bcq_tc_kernel(const __grid_constant__ CUtensorMap tm_planes, const uint32_t* __r
     uint4* xs = reinterpret_cast<uint4*>(base + (staged ? (size_t)n_wg * kTcStages * SB : 0));      // [sb][16][N]
     float* sums = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(xs) + (size_t)sb_per * kTcCols * N * 2);
 
-    // the slice sum (a programmatic dependent) may be scheduled now; it waits for this grid's results
-    dependents_may_start();
-    if (warp == 0) tc::alloc(tma::smem_addr(&tm_addr), (uint32_t)tmem_cols);
     if (threadIdx.x < kTcMaxGroups) {
         const int i = threadIdx.x;
         for (int k = 0; k < 2; ++k) {
@@ -261,9 +261,15 @@ bcq_tc_kernel(const __grid_constant__ CUtensorMap tm_planes, const uint32_t* __r
         dead = 0;
         tma::bar_init_fence();
     }
-    __syncthreads();
-    // launched as a programmatic dependent itself: nothing global is touched before the work ahead has completed
+    // Launched as a programmatic dependent: nothing global is touched before the work ahead has
+    // completed, and no tensor memory is taken.  A block of the kernel ahead may need what is left of
+    // it on this SM, and a block that held some while it waited for that kernel would never end.
     inputs_ready();
+    if (warp == 0) tc::alloc(tma::smem_addr(&tm_addr), (uint32_t)tmem_cols);
+    __syncthreads();
+    // The next kernel (the slice sum first of all) may be scheduled only now, for the same reason: one
+    // that takes tensor memory before it waits for this grid finds that every block here has its own.
+    dependents_may_start();
 
     // stages of a warpgroup: tile-major, spt per tile
     const int spt = (sbn + SBS - 1) / SBS;
