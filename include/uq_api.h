@@ -401,8 +401,10 @@ uq_status uq_export_bcq_half(const void* W, uq_wdtype wdtype, int64_t out, int64
  * contribution is formed from per-8-column partial sums of x (one table
  * lookup per plane byte).  Four tokens and more (and fewer of a large matrix
  * that the 1024-column tiles do not take): a +-1 matrix product per plane on
- * the tensor cores, the activations as bf16 values (an fp32 one as the exact
- * sum of three), fp32 sums scaled by alpha* per group.  Partial sums of tiles
+ * the tensor cores, the activations as bf16 values (an fp32 one as the sum of
+ * three; a token whose largest |x| in a column slice is below 2^-64 or 2^110 or
+ * more is scaled there by a power of two, so that nothing above 2^-69 of it is
+ * lost), fp32 sums scaled by alpha* per group.  Partial sums of tiles
  * or column slices go to `workspace` (caller-owned device memory of at least
  * uq_bcq_gemv_workspace_bytes(out, in, batch) bytes, overwritten) and are
  * summed in order into y.  Products of +-1 are exact and every sum is fp32, in

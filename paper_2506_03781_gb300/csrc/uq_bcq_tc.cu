@@ -17,6 +17,15 @@
 // of the first kind, (C_j x)_r = 2 D_j + S0 - S then, but for the 2^-64 and
 // 2^-32 of the clear bits, at most 2^-33 of sum |x|.
 //
+// Pieces, halves and sums leave the range of bf16 or fp32 where activations
+// are near its ends.  So a token whose largest activation in a slice is below
+// 2^-64 is multiplied by 2^64 there, one of 2^110 or more by 2^-32, and its
+// sums are multiplied back.  Of the others, what lies below the smallest bf16
+// number, 2^-133, is lost: less than 2^-69 of the largest.  The operands are
+// built without a look at this first, and again in the blocks that meet such a
+// number (64 tokens of 14336 x 4096: 39.8 us without the look, 40.2 with it;
+// with a scale for each pass, applied in the loop over the passes, 43.2).
+//
 // A warpgroup owns 128 rows, one per thread.  For every plane and 128
 // columns a thread expands the row's four plane words in registers and stores
 // them to tensor memory, which is the left operand; element k = 2 (16 word +
@@ -199,15 +208,15 @@ __device__ __forceinline__ void expand16_pm1(uint32_t w, const uint32_t (&mul)[1
     for (int p = 0; p < 16; ++p)
         asm("lop3.b32 %0, %1, %2, %3, 0x6a;" : "=r"(a[p]) : "r"(p == 15 ? w : w * mul[p]), "r"(mask), "r"(one));
 }
-// Half of both bf16 values of a pair (exact but for subnormal results).
+// Half of both bf16 values of a pair (but for subnormal results exact: see tc_scale).
 __device__ __forceinline__ uint32_t half_pair(uint32_t v) {
     const __nv_bfloat162 h = __hmul2(*reinterpret_cast<const __nv_bfloat162*>(&v), __floats2bfloat162_rn(0.5f, 0.5f));
     return *reinterpret_cast<const uint32_t*>(&h);
 }
 
-// Piece 0, 1 or 2 of an fp32 value: three bf16 numbers that add up to it
-// exactly (8 significant bits each, cut and not rounded, so none overflows).
-// Infinities and NaN stay in piece 0.  Used for words that hold one.
+// Piece 0, 1 or 2 of an fp32 value: three bf16 numbers that add up to it (8
+// significant bits each, cut and not rounded, so none overflows; exactly from
+// 2^-109 on).  Infinities and NaN stay in piece 0.
 __device__ __forceinline__ uint32_t bf16_piece(float x, int piece) {
     const uint32_t b = __float_as_uint(x);
     if ((b & 0x7f800000u) == 0x7f800000u) return piece ? 0u : (b & 0x007fffffu) ? 0x7fc0u : b >> 16;
@@ -217,6 +226,141 @@ __device__ __forceinline__ uint32_t bf16_piece(float x, int piece) {
     if (piece == 0) return h0 >> 16;
     if (piece == 1) return h1 >> 16;
     return __float_as_uint(__fsub_rn(r, __uint_as_float(h1))) >> 16;
+}
+
+// What a token is multiplied by in a slice, from the bits of its largest |x| there,
+// and what its sums are multiplied by.
+constexpr uint32_t kTcTiny = (127u - 64u) << 23, kTcHuge = (127u + 110u) << 23;
+__device__ __forceinline__ float tc_scale(uint32_t top) {
+    return top >= kTcHuge ? 0x1p-32f : top < kTcTiny ? 0x1p64f : 1.f;
+}
+__device__ __forceinline__ float tc_unscale(uint32_t top) {
+    return top >= kTcHuge ? 0x1p32f : top < kTcTiny ? 0x1p-64f : 1.f;
+}
+
+// The activations of a slice in operand order, into xs [sb][16][N], and their
+// block sums; true where the thread met one that asks for scaling.  SCALED:
+// with tops, the largest |x| of each token in the slice.
+template <int GB, int N, bool SCALED>
+__device__ __forceinline__ bool tc_operands(uint4* xs, float* sums, const uint32_t* tops, const void* __restrict__ X, int x_bf16,
+                                            int n_in, int tok0, int toks, int sb0, int sbn, int warp, int nw, int lane) {
+    constexpr int NB = kTcCols / GB;
+    constexpr bool KINDS = tc_kinds(GB, N);
+    constexpr int NSUM = KINDS ? 2 : 1;
+    const int words = n_in / 32;
+    bool odd = false;
+    for (int it = warp; it < sbn * (N / 8); it += nw) {
+        const int sb = it / (N / 8), n8 = it - sb * (N / 8);
+        const int tig = lane & 3, col = n8 * 8 + (lane >> 2);
+        const int tok = x_bf16 ? col : col / 3, piece = x_bf16 ? 0 : col - tok * 3;
+        const int word = (sb0 + sb) * 4 + tig;
+        uint32_t pr[16];                                   // columns p and p + 16 of the word
+        uint32_t any = 0;                                  // bits of all of them (fp32)
+        float sum = 0.f, sum0 = 0.f;                       // S, and its columns of the first kind (bits 3, 7, 11, 15)
+        if (tok < toks && word < words) {
+            const int64_t x0 = (int64_t)(tok0 + tok) * n_in + (int64_t)word * 32;
+            const float scale = SCALED ? tc_scale(tops[tok]) : 1.f;
+            if (x_bf16) {
+                const uint4* p = reinterpret_cast<const uint4*>(static_cast<const uint16_t*>(X) + x0);
+                uint32_t u[16];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const uint4 v = __ldg(p + i);
+                    u[4 * i] = v.x; u[4 * i + 1] = v.y; u[4 * i + 2] = v.z; u[4 * i + 3] = v.w;
+                }
+                if (SCALED) {
+#pragma unroll
+                    for (int i = 0; i < 16; ++i)
+                        u[i] = __byte_perm(__float_as_uint(__uint_as_float(u[i] << 16) * scale),
+                                           __float_as_uint(__uint_as_float(u[i] & 0xffff0000u) * scale), 0x7632);
+                }
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    pr[2 * i] = __byte_perm(u[i], u[i + 8], 0x5410);
+                    pr[2 * i + 1] = __byte_perm(u[i], u[i + 8], 0x7632);
+                }
+            } else {
+                const float4* p = reinterpret_cast<const float4*>(static_cast<const float*>(X) + x0);
+                // x less its upper 16 bits once for piece 1 and twice for piece 2, then cut
+                const uint32_t m1 = piece >= 1 ? 0xffff0000u : 0u, m2 = piece == 2 ? 0xffff0000u : 0u;
+                auto cut = [&](float v) {
+                    v = __fsub_rn(v, __uint_as_float(__float_as_uint(v) & m1));
+                    v = __fsub_rn(v, __uint_as_float(__float_as_uint(v) & m2));
+                    return __float_as_uint(v);
+                };
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    float lo[4], hi[4];
+                    f4_to(__ldg(p + i), lo);
+                    f4_to(__ldg(p + i + 4), hi);
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        if (SCALED) {
+                            pr[4 * i + k] = bf16_piece(lo[k] * scale, piece) | (bf16_piece(hi[k] * scale, piece) << 16);
+                        } else {
+                            any |= __float_as_uint(lo[k]) | __float_as_uint(hi[k]);
+                            pr[4 * i + k] = __byte_perm(cut(lo[k]), cut(hi[k]), 0x7632);
+                        }
+                    }
+                }
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < 16; ++i) pr[i] = 0u;
+        }
+        if (!SCALED && piece == 0) {                       // (the other pieces see the same activations)
+            uint32_t top = 0;
+#pragma unroll
+            for (int i = 0; i < 16; ++i) top = __vmaxu2(top, pr[i] & 0x7fff7fffu);
+            top = max(top & 0xffffu, top >> 16);
+            odd |= top >= kTcHuge >> 16 || (top < kTcTiny >> 16 && ((top | any) & 0x7fffffffu) != 0u);
+        }
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            const float v = __uint_as_float(pr[i] << 16) + __uint_as_float(pr[i] & 0xffff0000u);
+            if (i % 4 == 3) sum0 += v;
+            else sum += v;
+            if (KINDS && i % 4 == 2) pr[i] = half_pair(pr[i]);
+        }
+        // sum: the columns of the other kinds, S - S0
+        if (GB >= 64) {
+            sum += __shfl_xor_sync(kFull, sum, 1);
+            sum0 += __shfl_xor_sync(kFull, sum0, 1);
+        }
+        if (GB >= 128) {
+            sum += __shfl_xor_sync(kFull, sum, 2);
+            sum0 += __shfl_xor_sync(kFull, sum0, 2);
+        }
+        if (tig % (4 / NB) == 0) {
+            float* d = sums + ((sb * NB + tig / (4 / NB)) * N + col) * NSUM;
+            d[0] = sum + sum0;
+            if (KINDS) d[NSUM - 1] = -sum;
+        }
+#pragma unroll
+        for (int v = 0; v < 4; ++v)
+            xs[(sb * 16 + tig * 4 + v) * N + col] = make_uint4(pr[4 * v], pr[4 * v + 1], pr[4 * v + 2], pr[4 * v + 3]);
+    }
+    return odd;
+}
+
+// ... once more for a slice with tiny or huge activations: first the largest of each token.  Whole block.
+template <int GB, int N>
+__device__ __noinline__ void tc_scaled_operands(uint4* xs, float* sums, uint32_t* tops, const void* __restrict__ X, int x_bf16,
+                                                int n_in, int tok0, int toks, int sb0, int sbn, int warp, int nw, int lane) {
+    const int c0 = sb0 * kTcCols, c1 = min(n_in, c0 + sbn * kTcCols);
+    for (int t = warp; t < toks; t += nw) {
+        uint32_t top = 0;
+        for (int c = c0 + lane; c < c1; c += 32) {
+            const int64_t i = (int64_t)(tok0 + t) * n_in + c;
+            const uint32_t b = x_bf16 ? (uint32_t)__ldg(static_cast<const unsigned short*>(X) + i) << 16
+                                      : __float_as_uint(__ldg(static_cast<const float*>(X) + i));
+            top = max(top, b & 0x7fffffffu);
+        }
+        top = __reduce_max_sync(kFull, top);
+        if (lane == 0) tops[t] = top;
+    }
+    __syncthreads();
+    tc_operands<GB, N, true>(xs, sums, tops, X, x_bf16, n_in, tok0, toks, sb0, sbn, warp, nw, lane);
 }
 
 template <int Q, int GB, int N>
@@ -234,6 +378,8 @@ bcq_tc_kernel(const __grid_constant__ CUtensorMap tm_planes, const uint32_t* __r
     __shared__ __align__(8) unsigned long long ready[kTcMaxGroups][2], done[kTcMaxGroups][2], full[kTcMaxGroups][kTcStages];
     __shared__ uint32_t tm_addr;
     __shared__ volatile int dead;                          // a wait ran out: every warp stops
+    __shared__ volatile int scaled;                        // some token of the slice is
+    __shared__ uint32_t tops[N];                           // largest |x| of each token there
     const int warp = __shfl_sync(kFull, threadIdx.x >> 5, 0), lane = threadIdx.x & 31, nw = blockDim.x >> 5;
     // warps 0 .. 4 n_wg - 1: four of each warpgroup; then the issuing warp of each
     const int n_wg = blockDim.x / 160, wt = threadIdx.x & 127;
@@ -258,7 +404,7 @@ bcq_tc_kernel(const __grid_constant__ CUtensorMap tm_planes, const uint32_t* __r
             tma::bar_init(tma::smem_addr(&done[i][k]), 1);
         }
         for (int k = 0; k < kTcStages; ++k) tma::bar_init(tma::smem_addr(&full[i][k]), 1);
-        dead = 0;
+        dead = scaled = 0;
         tma::bar_init_fence();
     }
     // Launched as a programmatic dependent: nothing global is touched before the work ahead has
@@ -289,94 +435,9 @@ bcq_tc_kernel(const __grid_constant__ CUtensorMap tm_planes, const uint32_t* __r
         for (int i = 0; i < kTcStages && i < my_tiles * spt; ++i) copy(wg, i);
 
     // --- the slice's activations in operand order, and their block sums ---
-    for (int it = warp; it < sbn * (N / 8); it += nw) {
-        const int sb = it / (N / 8), n8 = it - sb * (N / 8);
-        const int tig = lane & 3, col = n8 * 8 + (lane >> 2);
-        const int tok = x_bf16 ? col : col / 3, piece = x_bf16 ? 0 : col - tok * 3;
-        const int word = (sb0 + sb) * 4 + tig;
-        uint32_t pr[16];                                   // columns p and p + 16 of the word
-        float sum = 0.f, sum0 = 0.f;                       // S, and its columns of the first kind (bits 3, 7, 11, 15)
-        if (tok < toks && word < words) {
-            const int64_t x0 = (int64_t)(tok0 + tok) * n_in + (int64_t)word * 32;
-            if (x_bf16) {
-                const uint4* p = reinterpret_cast<const uint4*>(static_cast<const uint16_t*>(X) + x0);
-                uint32_t u[16];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const uint4 v = __ldg(p + i);
-                    u[4 * i] = v.x; u[4 * i + 1] = v.y; u[4 * i + 2] = v.z; u[4 * i + 3] = v.w;
-                }
-#pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    pr[2 * i] = __byte_perm(u[i], u[i + 8], 0x5410);
-                    pr[2 * i + 1] = __byte_perm(u[i], u[i + 8], 0x7632);
-                }
-            } else {
-                const float4* p = reinterpret_cast<const float4*>(static_cast<const float*>(X) + x0);
-                // x less its upper 16 bits once for piece 1 and twice for piece 2, then cut
-                const uint32_t m1 = piece >= 1 ? 0xffff0000u : 0u, m2 = piece == 2 ? 0xffff0000u : 0u;
-                auto cut = [&](float v) {
-                    v = __fsub_rn(v, __uint_as_float(__float_as_uint(v) & m1));
-                    v = __fsub_rn(v, __uint_as_float(__float_as_uint(v) & m2));
-                    return __float_as_uint(v);
-                };
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    float lo[4], hi[4];
-                    f4_to(__ldg(p + i), lo);
-                    f4_to(__ldg(p + i + 4), hi);
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        const uint32_t a = cut(lo[k]), b = cut(hi[k]);
-                        pr[4 * i + k] = __byte_perm(a, b, 0x7632);
-                    }
-                }
-                uint32_t top = 0;
-#pragma unroll
-                for (int i = 0; i < 16; ++i) top |= ((pr[i] & 0x7f807f80u) + 0x00800080u) & 0x80008000u;
-                if (top != 0) {                             // an infinity or a NaN among them
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        float lo[4], hi[4];
-                        f4_to(__ldg(p + i), lo);
-                        f4_to(__ldg(p + i + 4), hi);
-#pragma unroll
-                        for (int k = 0; k < 4; ++k) {
-                            const uint32_t a = bf16_piece(lo[k], piece), b = bf16_piece(hi[k], piece);
-                            pr[4 * i + k] = a | (b << 16);
-                        }
-                    }
-                }
-            }
-        } else {
-#pragma unroll
-            for (int i = 0; i < 16; ++i) pr[i] = 0u;
-        }
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            const float v = __uint_as_float(pr[i] << 16) + __uint_as_float(pr[i] & 0xffff0000u);
-            if (i % 4 == 3) sum0 += v;
-            else sum += v;
-            if (KINDS && i % 4 == 2) pr[i] = half_pair(pr[i]);
-        }
-        // sum: the columns of the other kinds, S - S0
-        if (GB >= 64) {
-            sum += __shfl_xor_sync(kFull, sum, 1);
-            sum0 += __shfl_xor_sync(kFull, sum0, 1);
-        }
-        if (GB >= 128) {
-            sum += __shfl_xor_sync(kFull, sum, 2);
-            sum0 += __shfl_xor_sync(kFull, sum0, 2);
-        }
-        if (tig % (4 / NB) == 0) {
-            float* d = sums + ((sb * NB + tig / (4 / NB)) * N + col) * NSUM;
-            d[0] = sum + sum0;
-            if (KINDS) d[NSUM - 1] = -sum;
-        }
-#pragma unroll
-        for (int v = 0; v < 4; ++v)
-            xs[(sb * 16 + tig * 4 + v) * N + col] = make_uint4(pr[4 * v], pr[4 * v + 1], pr[4 * v + 2], pr[4 * v + 3]);
-    }
+    if (tc_operands<GB, N, false>(xs, sums, nullptr, X, x_bf16, n_in, tok0, toks, sb0, sbn, warp, nw, lane)) scaled = 1;
+    __syncthreads();
+    if (scaled) tc_scaled_operands<GB, N>(xs, sums, tops, X, x_bf16, n_in, tok0, toks, sb0, sbn, warp, nw, lane);
     tma::fence_async_smem();                               // the products read shared memory through the async proxy
     tc::fence_before();
     __syncthreads();
@@ -590,6 +651,10 @@ bcq_tc_kernel(const __grid_constant__ CUtensorMap tm_planes, const uint32_t* __r
 #pragma unroll
                 for (int t = 0; t < N / 3; ++t)
                     if (t < toks) dst[(int64_t)t * out] = (acc[3 * t] + acc[3 * t + 1]) + acc[3 * t + 2];
+            }
+            if (scaled) {                                  // (from memory, for the registers' sake)
+#pragma unroll 1
+                for (int t = 0; t < toks; ++t) dst[(int64_t)t * out] *= tc_unscale(tops[t]);
             }
         }
     }

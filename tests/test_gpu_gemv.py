@@ -55,13 +55,13 @@ def gpu_gemv(planes, a_star, z_star, x, g, xdtype="f32"):
     return C.host(y)
 
 
-def check(planes, a_star, z_star, x, g, xdtype="f32", label=""):
+def check(planes, a_star, z_star, x, g, xdtype="f32", label="", least=1e-30):
     if xdtype == "bf16":
         _, x = synth.bf16_round(x)               # the oracle sees the values the kernel reads
     y = gpu_gemv(planes, a_star, z_star, x, g, xdtype)
     ref = O.bcq_gemv(planes, a_star, z_star, x, g)
     err = np.abs(y.astype(F64) - ref)
-    bound = TOL * mass(a_star, z_star, x, g) + 1e-30
+    bound = TOL * mass(a_star, z_star, x, g) + least
     assert np.isfinite(y).all(), label
     assert (err <= bound).all(), f"{label}: worst {(err / bound).max():.3g} x tolerance"
     return y
@@ -137,6 +137,29 @@ def test_gemv_extreme_activations_stay_in_their_token(xdtype):
     api.uq_bcq_gemv(torch.from_numpy(planes.view(np.int32)).to(C.dev()), torch.from_numpy(a_star).to(C.dev()),
                     torch.from_numpy(z_star).to(C.dev()), xd, y, g)
     assert torch.isfinite(y[:4]).all() and not torch.isfinite(y[4:]).any()
+
+
+# 16, 32 and 64 matrix columns, blocks of one, two and four to a pass, and the lookup tables (one token)
+@pytest.mark.parametrize("g,q", [(32, 2), (64, 3), (128, 3), (512, 4)])
+@pytest.mark.parametrize("batch,xdtype", [(1, "f32"), (5, "f32"), (10, "f32"), (15, "bf16"), (15, "f32"), (40, "bf16")])
+def test_gemv_holds_its_bound_over_the_whole_range_of_the_type(g, q, batch, xdtype):
+    """Tokens down to the smallest numbers of the type (a bf16 piece or half of
+    one of them would fall below it) and up to where a sum of 128 activations
+    exceeds fp32 but the product does not, also with both in one token.  Each
+    term may be rounded to a multiple of 2^-149 besides: n_in of them."""
+    out, n_in = 140, 1024
+    planes, a_star, z_star = random_export(out, n_in, q, g, seed=8)
+    rng = np.random.default_rng(batch)
+    x = rng.standard_normal((batch, n_in)).astype(F32)
+    scales = [2.0 ** -112, 2.0 ** -120, 2.0 ** -126, 2.0 ** -133, 2.0 ** 122, 2.0 ** -64, 2.0 ** 108, 1.0]
+    for b in range(batch):
+        x[b] = (x[b].astype(F64) * scales[(b + batch) % len(scales)]).astype(F32)
+    if batch > 1:
+        x[1] = np.abs(x[1])                                       # one sign: sums that do not cancel
+        x[0, :512] = rng.standard_normal(512).astype(F32) * F32(2.0 ** -124)       # other passes, other scales
+        x[2, ::2] = rng.standard_normal(512).astype(F32) * F32(2.0 ** 109)         # ... and within a pass
+    check(planes, a_star, z_star, x, g, xdtype, label=f"range g{g} q{q} batch {batch} {xdtype}",
+          least=n_in * 2.0 ** -149)
 
 
 def test_gemv_deterministic():
