@@ -363,6 +363,15 @@ __device__ __noinline__ void tc_scaled_operands(uint4* xs, float* sums, uint32_t
     tc_operands<GB, N, true>(xs, sums, tops, X, x_bf16, n_in, tok0, toks, sb0, sbn, warp, nw, lane);
 }
 
+// Waits (bounded) for a warpgroup's last stages of the ring, of `copies` in all,
+// and for the last product of each buffer: ph has the parities of the next ones,
+// so of a phase before the first where there was none.
+__device__ __noinline__ void tc_drain(unsigned long long (&full)[kTcStages], int copies, unsigned long long (&done)[2], uint32_t ph) {
+    bool landed = drain(full, copies > kTcStages ? copies - kTcStages : 0, copies);
+    for (int k = 0; k < 2; ++k) landed &= tma::bar_wait(tma::smem_addr(&done[k]), ((ph >> k) & 1u) ^ 1u);
+    if (!landed) atomicOr(&g_tc_err, kDrainTimeoutBit);
+}
+
 template <int Q, int GB, int N>
 __global__ void __launch_bounds__(tc_groups(GB, N) * 160, 1)
 bcq_tc_kernel(const __grid_constant__ CUtensorMap tm_planes, const uint32_t* __restrict__ PLANES,
@@ -378,6 +387,7 @@ bcq_tc_kernel(const __grid_constant__ CUtensorMap tm_planes, const uint32_t* __r
     __shared__ __align__(8) unsigned long long ready[kTcMaxGroups][2], done[kTcMaxGroups][2], full[kTcMaxGroups][kTcStages];
     __shared__ uint32_t tm_addr;
     __shared__ volatile int dead;                          // a wait ran out: every warp stops
+    __shared__ int started[kTcMaxGroups][2];               // by a warpgroup's issuing warp: stages, products (parities)
     __shared__ volatile int scaled;                        // some token of the slice is
     __shared__ uint32_t tops[N];                           // largest |x| of each token there
     const int warp = __shfl_sync(kFull, threadIdx.x >> 5, 0), lane = threadIdx.x & 31, nw = blockDim.x >> 5;
@@ -479,6 +489,13 @@ bcq_tc_kernel(const __grid_constant__ CUtensorMap tm_planes, const uint32_t* __r
                     ++stage;
                 }
             }
+        // what this warp has started, for the wait at the end (kept in shared memory, and waited for by one
+        // warp: in this branch it cost the whole kernel registers and 2.4 of 40.2 us)
+        const int total = staged ? my_tiles * spt : 0, copies = stage + kTcStages < total ? stage + kTcStages : total;
+        if (lane == 0) {
+            started[wg][0] = copies;
+            started[wg][1] = (int)ph;
+        }
     }
     const uint32_t tmem = tm_addr + (uint32_t)(wg * tc_tmem_cols(GB, N));
     const uint32_t tlane = tmem + ((uint32_t)((warp & 3) * 32) << 16);         // this warp's 32 rows
@@ -658,13 +675,9 @@ bcq_tc_kernel(const __grid_constant__ CUtensorMap tm_planes, const uint32_t* __r
             }
         }
     }
-    // after a wait ran out: bounded waits for copies and products in flight before the block leaves
+    // where a wait ran out, products and copies may still be in flight: they land before the block leaves
     __syncthreads();
-    if (dead && wt == 0 && !issuer) {
-        const bool gone = tma::bar_wait(tma::smem_addr(&full[wg][waited & (kTcStages - 1)]), (uint32_t)(waited / kTcStages) & 1u, 1ll << 24) &
-                          tma::bar_wait(tma::smem_addr(&done[wg][buf]), (phase >> buf) & 1u, 1ll << 24);
-        if (!gone) atomicOr(&g_tc_err, kDrainTimeoutBit);
-    }
+    if (dead && warp == 0 && lane < n_wg) tc_drain(full[lane], started[lane][0], done[lane], (uint32_t)started[lane][1]);
     tc::fence_before();
     __syncthreads();
     if (warp == 0) tc::dealloc(tm_addr, (uint32_t)tmem_cols);
