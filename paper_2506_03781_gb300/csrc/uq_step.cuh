@@ -78,6 +78,20 @@ union StepTab {
     MapTab<Q, NG> b;               // phase B: levels, sorted order, local-mapping neighbours
 };
 
+// The ds_r partials of a row block are 32 bytes per rank.  They lie behind the
+// data of the stages where those leave that much (the copies end before it):
+// the 512 bytes would else cost fp32 weights, q = 3, g = 128 the second block
+// per SM (4096 x 4096: keep step 60.5 -> 79.2 us, remap step 71.8 -> 98.7).
+template <typename St>
+constexpr bool kStepRedInPad = St::BYTES - (St::OFF_A + St::SZ_A) >= kWarps * (int)sizeof(float);
+// Shared memory of a block (stages, tables, barriers, copy table) without the
+// partials, the partials, and what an SM has per block when two are resident.
+template <int Q, typename St>
+constexpr int kStepSmem = kWarps * (2 * St::BYTES + (int)sizeof(StepTab<Q, St::NG>) + 2 * 8) + 2 * 8 + 8 * 24;
+template <typename St>
+constexpr int kStepRedSmem = kStepRedInPad<St> ? 8 : 2 * kMaxCluster * kWarps * 4;
+constexpr int kStepTwoBlocks = 228 * 1024 / 2 - 1024;
+
 // 4 bytes to shared memory of block `rank` of the cluster (addresses as in the
 // own block), completing on that block's mbarrier.
 __device__ __forceinline__ void send_f32(uint32_t dst, uint32_t bar, uint32_t rank, float v) {
@@ -105,7 +119,8 @@ step_kernel(const void* __restrict__ W, float* S, float* SR, float* DELTA, float
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ __align__(8) unsigned long long bars[kWarps][2];
     __shared__ StepTab<Q, NG> tabs[kWarps];
-    __shared__ float red[2][kMaxCluster * kWarps];   // ds_r partials (Delta S3 sums) of row blocks k, k + 1: [rank][warp]
+    // ds_r partials (Delta S3 sums) of row blocks k, k + 1, eight warps of each rank
+    __shared__ float red_s[kStepRedInPad<St> ? 1 : 2 * kMaxCluster * kWarps];
     __shared__ __align__(8) unsigned long long rbar[2];   // their arrival, when the row is spread over a cluster
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -125,6 +140,10 @@ step_kernel(const void* __restrict__ W, float* S, float* SR, float* DELTA, float
     const int64_t n_items = (has_unit && n_rb_sub > cid) ? (n_rb_sub - cid + ncl - 1) / ncl : 0;
     unsigned char* wsm = smem + (size_t)warp * 2 * St::BYTES;
     StepTab<Q, NG>& t = tabs[warp];
+    auto red = [&](int64_t k, int rank) -> float* {
+        const int i = 2 * rank + (int)(k & 1);
+        return kStepRedInPad<St> ? reinterpret_cast<float*>(smem + (size_t)(i + 1) * St::BYTES) - kWarps : red_s + i * kWarps;
+    };
 
     if (lane == 0) {
         tma::bar_init(tma::smem_addr(&bars[warp][0]), 1);
@@ -278,9 +297,9 @@ step_kernel(const void* __restrict__ W, float* S, float* SR, float* DELTA, float
         }
         prow = warp_sum(prow);
         if (csize == 1) {
-            if (lane == 0) red[k & 1][warp] = prow;
+            if (lane == 0) red(k, 0)[warp] = prow;
         } else if (lane < csize) {
-            send_f32(tma::smem_addr(&red[k & 1][crank * kWarps + warp]), tma::smem_addr(&rbar[k & 1]), (uint32_t)lane, prow);
+            send_f32(tma::smem_addr(red(k, crank) + warp), tma::smem_addr(&rbar[k & 1]), (uint32_t)lane, prow);
         }
         __syncwarp();                              // the updated parameters of the unit are in the stage
         if (mine && alive) {
@@ -309,10 +328,10 @@ step_kernel(const void* __restrict__ W, float* S, float* SR, float* DELTA, float
             float tot = 0.f;
             if (csize > 1) {
                 const int n = csize * kWarps;          // at most 64, [rank][warp]
-                const float* rr = red[k & 1];
-                tot = warp_sum((lane < n ? rr[lane] : 0.f) + (lane + 32 < n ? rr[lane + 32] : 0.f));
+                tot = warp_sum((lane < n ? red(k, lane / kWarps)[lane % kWarps] : 0.f) +
+                               (lane + 32 < n ? red(k, lane / kWarps + 4)[lane % kWarps] : 0.f));
             } else {
-                for (int w = 0; w < WPR; ++w) tot += red[k & 1][row_sub * WPR + w];
+                for (int w = 0; w < WPR; ++w) tot += red(k, 0)[row_sub * WPR + w];
             }
             const float dsr = -tot / sr;
             const float sr_new = __fsub_rn(sr, __fmul_rn(lr_f, dsr));
@@ -411,6 +430,8 @@ static cudaError_t run_step(const Shape& sh, const void* W, uq_params p, uint8_t
     const int R = csize == 1 ? rows_per_block(U) : 1;
     const int64_t n_rb = (sh.out + R - 1) / R;
     const size_t dyn = (size_t)kWarps * 2 * St::BYTES;
+    static_assert(kStepSmem<Q, St> > kStepTwoBlocks || kStepSmem<Q, St> + kStepRedSmem<St> <= kStepTwoBlocks,
+                  "the partials must not cost the second block per SM");
     auto kern = step_kernel<Q, WT, G_, MODEB, BIO>;
     // occupancy per device and cluster size (blocks per SM for csize == 1, clusters on the GPU otherwise)
     static std::atomic<int> cache[kMaxDevicesStep][kMaxCluster + 1] = {};
