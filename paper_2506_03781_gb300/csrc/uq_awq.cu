@@ -35,7 +35,6 @@ awq_fwd_kernel(const void* __restrict__ W, const float* __restrict__ SA, const f
                const float* __restrict__ ZA, const float* __restrict__ ALPHA, const float* __restrict__ ZB,
                uint8_t* __restrict__ CODES, float* __restrict__ WHAT, int64_t out, int n_in, int g,
                int64_t rows_per_range) {
-    dependents_may_start();
     inputs_ready();
     constexpr int L = 1 << Q;
     constexpr int NG = 32 / LPG;
@@ -127,7 +126,6 @@ awq_bwd_kernel(const void* __restrict__ W, const float* __restrict__ SA, const f
                const uint8_t* __restrict__ CODES, const float* __restrict__ GUP, float* __restrict__ DDELTA,
                float* __restrict__ DZA, float* __restrict__ DALPHA, float* __restrict__ DZB,
                float* __restrict__ PART, int64_t out, int n_in, int g, int64_t rows_per_range) {
-    dependents_may_start();
     inputs_ready();
     constexpr int L = 1 << Q;
     constexpr int NG = 32 / LPG;
@@ -287,9 +285,9 @@ __global__ void __launch_bounds__(kThreads, 3)
 awq_stream_fwd_kernel(const void* __restrict__ W, const float* __restrict__ SA, const float* __restrict__ DELTA,
                       const float* __restrict__ ZA, const float* __restrict__ ALPHA, const float* __restrict__ ZB,
                       uint8_t* __restrict__ CODES, float* __restrict__ WHAT, int64_t out, int n_in, int R, int n_rb) {
-    dependents_may_start();
     using St = AwqFwdStage<Q, WT, G_, MODE>;
     constexpr int L = 1 << Q, LPG = St::LPG, NG = St::NG, NV = St::NV, UE = St::UE, NST = St::NST;
+    let_next_start(n_in / UE, R, n_rb, 0);
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ __align__(8) unsigned long long bars[kWarps][NST];
     __shared__ SortTab<Q, NG> tabs[kWarps];
@@ -485,9 +483,9 @@ awq_stream_bwd_kernel(const void* __restrict__ W, const float* __restrict__ SA, 
                       const uint8_t* __restrict__ CODES, const float* __restrict__ GUP, float* __restrict__ DDELTA,
                       float* __restrict__ DZA, float* __restrict__ DALPHA, float* __restrict__ DZB,
                       float* __restrict__ PART, int64_t out, int n_in, int R, int n_rb) {
-    dependents_may_start();
     using St = AwqBwdStage<Q, WT, G_>;
     constexpr int L = 1 << Q, LPG = St::LPG, NG = St::NG, NV = St::NV, UE = St::UE, NST = St::NST;
+    let_next_start(n_in / UE, R, n_rb, 0);
     using SR8 = SegReduce<LPG>;
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ __align__(8) unsigned long long bars[kWarps][NST];
@@ -642,7 +640,6 @@ cudaError_t awq_error(bool clear, unsigned int* flag) {
 constexpr int kColsumSlices = 8;
 __global__ void __launch_bounds__(32 * kColsumSlices)
 awq_colsum_kernel(const float* __restrict__ PART, float* __restrict__ DSA, int n_in, int ranges) {
-    dependents_may_start();
     inputs_ready();
     __shared__ float part[kColsumSlices][32];
     const int lane = threadIdx.x & 31, slice = threadIdx.x >> 5;

@@ -36,7 +36,6 @@ bwd_kernel(const void* __restrict__ W, const float* __restrict__ S, const float*
            const float* __restrict__ ZB, const uint8_t* __restrict__ CODES, const float* __restrict__ GUP,
            float* __restrict__ DS, float* __restrict__ DSR, float* __restrict__ DDELTA, float* __restrict__ DZU,
            float* __restrict__ DZB, float* __restrict__ DALPHA, int64_t out, int n_in, int g, int R) {
-    dependents_may_start();
     inputs_ready();
     constexpr int L = 1 << Q;
     constexpr int NG = 32 / LPG;                 // groups per unit

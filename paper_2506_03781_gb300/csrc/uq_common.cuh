@@ -26,16 +26,35 @@ constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
 constexpr unsigned kFull = 0xffffffffu;
 
-// Programmatic dependent launch: a kernel lets the next one on the stream
-// be scheduled while it runs (dependents_may_start, first thing) and itself
-// waits for the work ahead of it before its first access to global memory
-// (inputs_ready; returns at once when it was not launched as a dependent).
-// What overlaps is the launch and the set-up of shared memory.  Four kernels of
-// a 1024 x 1024 matrix: 30.5 -> 19.0 us queued, of 14336 x 4096: 441 -> 427 us.
+// Programmatic dependent launch: a kernel waits for the work ahead of it on the
+// stream before its first access to global memory (inputs_ready; returns at once
+// when it was not launched as a dependent), so its launch and the set-up of
+// shared memory overlap the end of that work.  It may also let the next kernel
+// be scheduled while it runs (dependents_may_start) and not only when its blocks
+// have ended.  Blocks that are scheduled early go where there is room, two or
+// three of a grid to one SM, and what was one even round then takes up to twice
+// as long.  So the pipelined per-step kernels do so where they are few blocks of
+// one round (the fused step: up to two rounds), or, but for AWQ's, many rounds,
+// which even out; no other per-step kernel does.
+// Captured steps (two forwards and backwards) against plain launches, with no
+// early start / with one always: 64 x 512 1.12 / 1.33 times as fast, 1024 x 1024
+// 1.07 / 1.13 (g = 1024: 1.04 / 0.79), 300 x 11008 1.02 / 0.99 (full mapping 1.02 /
+// 0.82), 128 x 14336 1.04 / 0.83, 1024 x 8192 1.01 / 0.96, 4096 x 4096 1.01 /
+// 1.03.  Queued from the host (plain launches / now): a step of 1024 x 1024 30.6 /
+// 20.1 us, of 14336 x 4096 441 / 427 (432 without an early start).
 // Not for the initialization (one long launch) and the clusters of the fused
 // step (slower: see its launch).
 __device__ __forceinline__ void dependents_may_start() { asm volatile("griddepcontrol.launch_dependents;"); }
 __device__ __forceinline__ void inputs_ready() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// First thing in a pipelined per-step kernel of n_rb row blocks, of R rows of U
+// units each; many: the rounds from which on the grid evens out (0: never).
+// After a backward comes a forward, which has half its rounds (2048 x 5632: 6.7
+// and 4.5; 1.01 against 0.98 times a plain launch).
+constexpr int kFewBlocks = 64, kManyRounds = 6, kManyRoundsBwd = 8;
+__device__ __forceinline__ void let_next_start(int U, int R, int n_rb, int many) {
+    const int blocks = (int)gridDim.x;
+    if ((many > 0 && n_rb >= many * blocks) || (blocks <= kFewBlocks && n_rb <= blocks && U * R <= kWarps)) dependents_may_start();
+}
 
 // Weight-storage adaptors: 4 consecutive weights per lane.
 struct WF32 {

@@ -38,7 +38,6 @@ export_kernel(const void* __restrict__ W, const float* __restrict__ DELTA, const
               const float* __restrict__ ALPHA, const float* __restrict__ ZB, const uint8_t* __restrict__ CODES,
               uint32_t* __restrict__ PLANES, typename OT::T* __restrict__ ASTAR, typename OT::T* __restrict__ ZSTAR,
               int64_t out, int n_in, int g) {
-    dependents_may_start();
     inputs_ready();
     constexpr int L = 1 << Q;
     constexpr uint32_t kMask = uint32_t(L - 1) * 0x01010101u;

@@ -29,7 +29,6 @@ fwd_kernel(const void* __restrict__ W, const float* __restrict__ S, const float*
            const float* __restrict__ DELTA, const float* __restrict__ ZU, const float* __restrict__ ALPHA,
            const float* __restrict__ ZB, uint8_t* __restrict__ CODES, float* __restrict__ WHAT, int64_t out,
            int n_in, int g, int R, int mode) {
-    dependents_may_start();
     inputs_ready();
     constexpr int L = 1 << Q;
     constexpr int NG = 32 / LPG;

@@ -56,7 +56,6 @@ omni_fwd_kernel(const void* __restrict__ W, const float* __restrict__ BETA, cons
                 const float* __restrict__ ALPHA, const float* __restrict__ ZB, uint8_t* __restrict__ CODES,
                 float* __restrict__ WHAT, float* __restrict__ DOUT, float* __restrict__ ZOUT, int64_t out, int n_in,
                 int g, int R) {
-    dependents_may_start();
     inputs_ready();
     constexpr int L = 1 << Q;
     constexpr int NG = 32 / LPG;
@@ -156,7 +155,6 @@ omni_bwd_kernel(const void* __restrict__ W, const float* __restrict__ BETA, cons
                 const float* __restrict__ ALPHA, const float* __restrict__ ZB, const uint8_t* __restrict__ CODES,
                 const float* __restrict__ GUP, float* __restrict__ DBETA, float* __restrict__ DGAMMA,
                 float* __restrict__ DALPHA, float* __restrict__ DZB, int64_t out, int n_in, int g, int R) {
-    dependents_may_start();
     inputs_ready();
     constexpr int L = 1 << Q;
     constexpr int NG = 32 / LPG;
@@ -299,9 +297,9 @@ __global__ void __launch_bounds__(kThreads, 3)
 omni_stream_fwd_kernel(const void* __restrict__ W, const float* __restrict__ BETA, const float* __restrict__ GAMMA,
                        const float* __restrict__ ALPHA, const float* __restrict__ ZB, uint8_t* __restrict__ CODES,
                        float* __restrict__ WHAT, int64_t out, int n_in, int R, int n_rb) {
-    dependents_may_start();
     using St = OmniFwdStage<Q, WT, G_, MODE>;
     constexpr int L = 1 << Q, LPG = St::LPG, NG = St::NG, NV = St::NV, UE = St::UE, NST = St::NST;
+    let_next_start(n_in / UE, R, n_rb, kManyRounds);
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ __align__(8) unsigned long long bars[kWarps][NST];
     __shared__ SortTab<Q, NG> tabs[kWarps];
@@ -415,9 +413,9 @@ omni_stream_bwd_kernel(const void* __restrict__ W, const float* __restrict__ BET
                        const float* __restrict__ ALPHA, const float* __restrict__ ZB, const uint8_t* __restrict__ CODES,
                        const float* __restrict__ GUP, float* __restrict__ DBETA, float* __restrict__ DGAMMA,
                        float* __restrict__ DALPHA, float* __restrict__ DZB, int64_t out, int n_in, int R, int n_rb) {
-    dependents_may_start();
     using St = OmniBwdStage<Q, WT, G_>;
     constexpr int L = 1 << Q, LPG = St::LPG, NG = St::NG, NV = St::NV, UE = St::UE, NST = St::NST;
+    let_next_start(n_in / UE, R, n_rb, kManyRoundsBwd);
     using SR8 = SegReduce<LPG>;
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ __align__(8) unsigned long long bars[kWarps][NST];

@@ -71,9 +71,9 @@ __global__ void __launch_bounds__(kThreads, 2)
 ragged_bwd_kernel(const RaggedSrc src, const float* __restrict__ SR, float* __restrict__ DS, float* __restrict__ DSR,
                   float* __restrict__ DDELTA, float* __restrict__ DZU, float* __restrict__ DZB,
                   float* __restrict__ DALPHA, int64_t out, int n_in, int R, int n_rb) {
-    dependents_may_start();
     using St = RaggedBwdStage<Q, WT, G_>;
     constexpr int L = 1 << Q, LPG = St::LPG, NG = St::NG, NV = St::NV, UE = St::UE, NST = St::NST;
+    let_next_start((n_in / G_ + NG - 1) / NG, R, n_rb, kManyRoundsBwd);
     using SR8 = SegReduce<LPG>;
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ __align__(8) unsigned long long bars[kWarps][NST];

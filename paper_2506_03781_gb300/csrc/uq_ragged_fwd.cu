@@ -24,9 +24,9 @@ template <int Q, typename WT, int G_, int MODE>
 __global__ void __launch_bounds__(kThreads, MODE == FWD_KEEP ? 4 : 3)
 ragged_fwd_kernel(const RaggedSrc src, const float* __restrict__ SR, uint8_t* __restrict__ CODES,
                   float* __restrict__ WHAT, int64_t out, int n_in, int R, int n_rb) {
-    dependents_may_start();
     using St = RaggedFwdStage<Q, WT, G_, MODE>;
     constexpr int L = 1 << Q, LPG = St::LPG, NG = St::NG, NV = St::NV, UE = St::UE, NST = St::NST;
+    let_next_start((n_in / G_ + NG - 1) / NG, R, n_rb, kManyRounds);
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ __align__(8) unsigned long long bars[kWarps][NST];
     __shared__ SortTab<Q, NG> tabs[kWarps];

@@ -65,9 +65,9 @@ bwd_stream_kernel(const void* __restrict__ W, const float* __restrict__ S, const
                   float* __restrict__ DS, float* __restrict__ DSR, float* __restrict__ DDELTA,
                   float* __restrict__ DZU, float* __restrict__ DZB, float* __restrict__ DALPHA, int64_t out,
                   int n_in, int R, int n_rb, int branchy) {
-    dependents_may_start();
     using St = Stage<Q, WT, G_, true, true, true, UQ_BWD_STAGE_BYTES>;
     constexpr int L = 1 << Q, LPG = St::LPG, NG = St::NG, NV = St::NV, UE = St::UE, NST = St::NST;
+    let_next_start(n_in / UE, R, n_rb, kManyRoundsBwd);
     constexpr uint32_t TX = St::TX;
     using SR8 = SegReduce<LPG>;
     extern __shared__ __align__(128) unsigned char smem[];
@@ -278,12 +278,12 @@ fwd_stream_kernel(const void* __restrict__ W, const float* __restrict__ S, const
                   const float* __restrict__ DELTA, const float* __restrict__ ZU, const float* __restrict__ ALPHA,
                   const float* __restrict__ ZB, uint8_t* __restrict__ CODES, float* __restrict__ WHAT,
                   int64_t out, int n_in, int R, int n_rb) {
-    dependents_may_start();
     static_assert(MODE != FWD_KEEP, "the keep step runs keep_stream_kernel");
     constexpr int mode = MODE;
     constexpr bool need_c = MODE != FWD_FULL;
     using St = Stage<Q, WT, G_, true, false, need_c, UQ_FWD_STAGE_BYTES>;
     constexpr int L = 1 << Q, LPG = St::LPG, NG = St::NG, NV = St::NV, UE = St::UE, NST = St::NST;
+    let_next_start(n_in / UE, R, n_rb, kManyRounds);
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ __align__(8) unsigned long long bars[kWarps][NST];
     __shared__ SortTab<Q, NG> tabs[kWarps];
@@ -421,9 +421,9 @@ __global__ void __launch_bounds__(kThreads, UQ_STREAM_FWD_MIN_BLOCKS)
 keep_stream_kernel(const float* __restrict__ DELTA, const float* __restrict__ ZU, const float* __restrict__ ALPHA,
                    const float* __restrict__ ZB, const uint8_t* __restrict__ CODES, float* __restrict__ WHAT,
                    int64_t out, int n_in, int R, int n_rb) {
-    dependents_may_start();
     using St = KeepStage<Q, G_, KU>;
     constexpr int L = 1 << Q, LPG = St::LPG, NG = St::NG, NGK = St::NGK, NV = St::NV, UE = St::UE, NST = St::NST;
+    let_next_start(n_in / (KU * UE), R, n_rb, kManyRounds);
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ __align__(8) unsigned long long bars[kWarps][NST];
     __shared__ float lvs[kWarps][NGK][L];               // levels of the item's groups
