@@ -526,6 +526,13 @@ __device__ __forceinline__ void unit_full_iv(const SortTab<Q, NS>& t, float4 (*i
 // (14336 x 4096, q = 3, g = 128: 168 -> 133 us, q = 4: 294 -> 172 us.)
 template <int Q, int G_>
 constexpr bool kFullSearch = Q == 4 || (Q == 3 && G_ >= 128);
+// ... from so many row blocks per SM on: with fewer the tables are what takes
+// the time.  Scan over search: q = 4, g = 128 0.94 to 0.98 up to 100 row blocks,
+// 1.05 to 1.6 beyond; g = 64 0.74 to 1.07 up to 1000, 0.94 to 1.12 from 2000 on; g
+// = 32 0.76 to 1.0 up to 500, 0.99 to 1.22 from 1000 on; q = 3, g = 128 0.73 to 1.0
+// up to 500, 0.97 to 1.17 from 1000 on.
+template <int Q, int G_>
+constexpr int kFullSearchBlocks = Q == 4 && G_ == 128 ? 0 : G_ == 64 ? 12 : 6;
 
 // Every fourth midpoint of a group (none for L <= 4).
 template <int L>

@@ -2,8 +2,8 @@
 // Algorithm 4) and Q_IF (Eq. 2, full mapping).
 //
 // The kernel here takes the groups of more than 512 elements and of 384, and
-// the full mapping of rows that are no whole number of work units where it is
-// the faster one (ragged_full_ok); the pipelined kernels of uq_stream.cu and
+// rows that are no whole number of work units (and g = 256, 512) where it is the
+// faster one (ragged_fwd_ok); the pipelined kernels of uq_stream.cu and
 // uq_ragged_fwd.cu take everything else.
 //
 // Per warp and work unit (NG whole groups, see uq_common.cuh): the lanes
@@ -154,6 +154,7 @@ static cudaError_t fwd_g(const Shape& sh, const void* W, uq_params p, uint8_t* c
     switch (lanes_per_group(sh.g)) {
         case 4: return run_fwd<Q, WT, 4>(sh, W, p, codes, mode, what, st);
         case 8: return run_fwd<Q, WT, 8>(sh, W, p, codes, mode, what, st);
+        case 16: return run_fwd<Q, WT, 16>(sh, W, p, codes, mode, what, st);
         default: return run_fwd<Q, WT, 32>(sh, W, p, codes, mode, what, st);
     }
 }
@@ -165,11 +166,38 @@ static cudaError_t fwd_w(const Shape& sh, const void* W, uq_params p, uint8_t* c
     return fwd_g<Q, WF32>(sh, W, p, codes, mode, what, st);
 }
 
+// The pipelined kernel has its tables and copies to set up and a persistent
+// grid of 3 (keep: 4) blocks per SM, the last round of which may be nearly
+// empty; with few row blocks the kernel here is faster.  Row blocks here, and
+// the time of this kernel over the pipelined one's, bf16, 64 to 8192 rows of 640
+// to 14336 columns:
+//   keep, remap  q >= 3 with g <= 64, q = 4 with g = 128 (this kernel's tables
+//                cost most): 0.94 to 2.2 everywhere
+//   keep         the rest: up to 1000 0.75 to 1.1, from 2000 on 0.95 to 1.9
+//   remap        the rest: up to 500 0.8 to 1.05, 1000 0.9 to 1.1, then 1.0 to
+//                1.25; but q <= 2, g >= 256, 4096 x 14336 0.88 to 0.96 (memory)
+//   full         g >= 256, q = 4: up to 128 0.83 to 1.0, then 1.05 to 1.7; q = 3:
+//                up to 500 0.73 to 1.0, 1000 0.85 to 1.05, then 1.0 to 1.24; q <=
+//                2: up to 1000 0.7 to 0.95, 2000 0.95 to 1.08, then 0.98 to 1.16;
+//                g = 128, q = 4: 0.86 to 1.6
+bool ragged_fwd_ok(const Shape& sh, int mode) {
+    const int NG = 32 / lanes_per_group(sh.g), U = (sh.n_in / sh.g + NG - 1) / NG;
+    const int64_t R = rows_per_block(U), n_rb = (sh.out + R - 1) / R, sms = sm_count();
+    if (mode == FWD_FULL) {
+        if (!ragged_full_has(sh.q, sh.g)) return false;
+        if (sh.g == 128) return true;
+        return n_rb >= (sh.q == 4 ? sms : sh.q == 3 ? 6 * sms : 24 * sms);
+    }
+    if ((sh.q >= 3 && sh.g <= 64) || (sh.q == 4 && sh.g == 128)) return true;
+    if (mode == FWD_KEEP) return n_rb >= 12 * sms;
+    if (sh.q <= 2 && sh.g >= 256 && U > 22 && n_rb >= 24 * sms) return false;
+    return n_rb >= 6 * sms;
+}
+
 cudaError_t launch_fwd(const Shape& sh, const void* W, uq_params p, uint8_t* codes, int mode, float* what,
                        cudaStream_t st) {
     if (stream_path_ok(sh)) return launch_fwd_stream(sh, W, p, codes, mode, what, st);
-    if (ragged_path_ok(sh) && (mode != FWD_FULL || ragged_full_ok(sh.q, sh.g)))
-        return launch_fwd_ragged(sh, W, p, codes, mode, what, st);
+    if (ragged_path_ok(sh) && ragged_fwd_ok(sh, mode)) return launch_fwd_ragged(sh, W, p, codes, mode, what, st);
     switch (sh.q) {
         case 1: return fwd_w<1>(sh, W, p, codes, mode, what, st);
         case 2: return fwd_w<2>(sh, W, p, codes, mode, what, st);

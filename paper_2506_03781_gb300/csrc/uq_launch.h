@@ -42,12 +42,11 @@ cudaError_t launch_bwd_stream(const Shape& sh, const void* W, uq_params p, const
 inline bool ragged_path_ok(const Shape& sh) {
     return sh.g == 32 || sh.g == 64 || sh.g == 128 || sh.g == 256 || sh.g == 512;
 }
-// ... and whether the full mapping takes them too.  Its scan of the levels is
-// as fast or faster in the kernel of uq_fwd.cu for the rest, which loads to
-// registers: 8192 x 4224, g = 128, q = 3: 126 us there vs 130 (fp32: 129 vs
-// 170), q = 2: 107 vs 110; g = 64, q = 4: 255 vs 270; but g = 128, q = 4: 214
-// vs 157, and g = 256, q = 1: 76 vs 63, q = 4: 153 vs 89 on 8192 x 4096.
-constexpr bool ragged_full_ok(int q, int g) { return g >= 256 || (g == 128 && q == 4); }
+// Whether the pipelined forward takes such rows, or the kernel of uq_fwd.cu,
+// which loads to registers and starts sooner (uq_fwd.cu).
+bool ragged_fwd_ok(const Shape& sh, int mode);
+// The combinations of bit-width and group size whose full mapping it has.
+constexpr bool ragged_full_has(int q, int g) { return g >= 256 || (g == 128 && q == 4); }
 cudaError_t launch_fwd_ragged(const Shape& sh, const void* W, uq_params p, uint8_t* codes, int mode, float* what,
                               cudaStream_t st);
 cudaError_t launch_bwd_ragged(const Shape& sh, const void* W, uq_params p, const uint8_t* codes, const float* gup,

@@ -172,10 +172,10 @@ static cudaError_t ragged_fwd_g(const Shape& sh, const void* W, uq_params p, uin
     if (mode == FWD_REMAP)
         return bf16 ? run_ragged_fwd<Q, WBF16, G_, FWD_REMAP>(sh, W, p, codes, what, st)
                     : run_ragged_fwd<Q, WF32, G_, FWD_REMAP>(sh, W, p, codes, what, st);
-    if constexpr (ragged_full_ok(Q, G_))
+    if constexpr (ragged_full_has(Q, G_))
         return bf16 ? run_ragged_fwd<Q, WBF16, G_, FWD_FULL>(sh, W, p, codes, what, st)
                     : run_ragged_fwd<Q, WF32, G_, FWD_FULL>(sh, W, p, codes, what, st);
-    return cudaErrorInvalidValue;                        // launch_fwd sends the rest to its own kernel
+    return cudaErrorInvalidValue;                        // ragged_fwd_ok refuses the rest
 }
 
 template <int Q>

@@ -272,7 +272,7 @@ bwd_stream_kernel(const void* __restrict__ W, const float* __restrict__ S, const
 // Forward
 // ---------------------------------------------------------------------------
 
-template <int Q, typename WT, int G_, int MODE>
+template <int Q, typename WT, int G_, int MODE, bool SEARCH>
 __global__ void __launch_bounds__(kThreads, UQ_STREAM_FWD_MIN_BLOCKS)
 fwd_stream_kernel(const void* __restrict__ W, const float* __restrict__ S, const float* __restrict__ SR,
                   const float* __restrict__ DELTA, const float* __restrict__ ZU, const float* __restrict__ ALPHA,
@@ -287,7 +287,7 @@ fwd_stream_kernel(const void* __restrict__ W, const float* __restrict__ S, const
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ __align__(8) unsigned long long bars[kWarps][NST];
     __shared__ SortTab<Q, NG> tabs[kWarps];
-    constexpr bool search = mode == FWD_FULL && kFullSearch<Q, G_>;
+    constexpr bool search = mode == FWD_FULL && SEARCH;
     __shared__ float4 ivs[kWarps][mode != FWD_FULL || search ? NG : 1][L];         // intervals of the remap or of the search
     __shared__ __align__(16) float ths[kWarps][search ? NG : 1][L];                // midpoints of the search
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -541,7 +541,10 @@ static cudaError_t run_bwd_stream(const Shape& sh, const void* W, uq_params p, c
                                       U >= kBranchyUnits ? 1 : 0);
 }
 
-template <int Q, typename WT, int G_, int MODE>
+template <typename St, bool SEARCH>
+struct FwdTag {};
+
+template <int Q, typename WT, int G_, int MODE, bool SEARCH = false>
 static cudaError_t run_fwd_stream_mode(const Shape& sh, const void* W, uq_params p, uint8_t* codes, float* what,
                                        cudaStream_t st) {
     using St = Stage<Q, WT, G_, true, false, MODE != FWD_FULL, UQ_FWD_STAGE_BYTES>;
@@ -549,9 +552,9 @@ static cudaError_t run_fwd_stream_mode(const Shape& sh, const void* W, uq_params
     const int R = rows_per_block(U);
     const int n_rb = (int)((sh.out + R - 1) / R);
     const size_t dyn = (size_t)kWarps * St::WARP_BYTES;
-    auto kern = fwd_stream_kernel<Q, WT, G_, MODE>;
+    auto kern = fwd_stream_kernel<Q, WT, G_, MODE, SEARCH>;
     int grid = 0;
-    cudaError_t e = grid_for<St>(kern, dyn, n_rb, grid);
+    cudaError_t e = grid_for<FwdTag<St, SEARCH>>(kern, dyn, n_rb, grid);
     if (e != cudaSuccess) return e;
     return launch_dependent(kern, grid, kThreads, dyn, st, W, p.s, p.sr, p.delta, p.zu, p.alpha, p.zb, codes, what, sh.out, sh.n_in, R,
                                       n_rb);
@@ -588,7 +591,15 @@ static cudaError_t run_fwd_stream(const Shape& sh, const void* W, uq_params p, u
                                   float* what, cudaStream_t st) {
     if (mode == FWD_KEEP) return keep_stream<Q, G_>(sh, p, codes, what, st);
     if (mode == FWD_REMAP) return run_fwd_stream_mode<Q, WT, G_, FWD_REMAP>(sh, W, p, codes, what, st);
-    return run_fwd_stream_mode<Q, WT, G_, FWD_FULL>(sh, W, p, codes, what, st);
+    if constexpr (kFullSearch<Q, G_>) {
+        const int U = sh.n_in / Stage<Q, WT, G_, true, false, false, UQ_FWD_STAGE_BYTES>::UE;
+        const int64_t R = rows_per_block(U), n_rb = (sh.out + R - 1) / R;
+        if (n_rb >= (int64_t)kFullSearchBlocks<Q, G_> * sm_count())
+            return run_fwd_stream_mode<Q, WT, G_, FWD_FULL, true>(sh, W, p, codes, what, st);
+    }
+    if constexpr (!kFullSearch<Q, G_> || kFullSearchBlocks<Q, G_> > 0)
+        return run_fwd_stream_mode<Q, WT, G_, FWD_FULL>(sh, W, p, codes, what, st);
+    return cudaErrorInvalidValue;                        // not reached
 }
 
 template <int Q, typename WT, bool ELEM>

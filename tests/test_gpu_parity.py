@@ -302,6 +302,36 @@ def test_rows_of_partial_units(out, n_in, g, q, wd):
     api.uq_check_device()
 
 
+# The forward's kernel depends on the row blocks per SM (8 rows each here): both sides of every such line, for
+# rows of partial units, g = 256 and 512, and for the search of the full mapping in whole units
+@pytest.mark.parametrize("q,g,n_in,mode,step,line", [
+    (1, 32, 96, api.MAP_LOCAL_PERIODIC, 0, 6), (2, 64, 192, api.MAP_LOCAL_PERIODIC, 1, 12),
+    (3, 128, 128, api.MAP_LOCAL_PERIODIC, 0, 6), (3, 128, 128, api.MAP_LOCAL_PERIODIC, 1, 12),
+    (2, 256, 256, api.MAP_LOCAL_PERIODIC, 0, 6), (4, 256, 256, api.MAP_LOCAL_PERIODIC, 1, 12),
+    (3, 512, 512, api.MAP_LOCAL_PERIODIC, 0, 6), (2, 512, 512, api.MAP_LOCAL_PERIODIC, 1, 12),
+    (4, 256, 256, api.MAP_FULL, 0, 1), (3, 512, 512, api.MAP_FULL, 0, 6), (2, 256, 256, api.MAP_FULL, 0, 24),
+    (3, 128, 512, api.MAP_FULL, 0, 6), (4, 64, 512, api.MAP_FULL, 0, 12), (4, 32, 256, api.MAP_FULL, 0, 6)])
+@pytest.mark.parametrize("wd", ["bf16", "f32"])
+def test_forward_on_both_sides_of_a_row_block_line(q, g, n_in, mode, step, line, wd):
+    """Some rows' inputs repeated over as many rows as it takes; every copy gives the oracle's rows."""
+    few = 40
+    raw, W, P, codes0, _ = C.make_inputs(few, n_in, q, g, seed=q + g + n_in, wdtype=wd, init_G=3, init_T=2)
+    r_what, r_codes = O.quantize_fwd(W, P["s"], P["sr"], P["delta"], P["zu"], P["alpha"], P["zb"],
+                                     None if mode == api.MAP_FULL else codes0, g, mode, step, 2)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    d = C.dev()
+    Wd = api.weights_tensor(raw, d) if wd == "bf16" else torch.from_numpy(W).to(d)
+    Pd, cd = C.to_dev(P), torch.from_numpy(codes0).to(d)
+    for out in (8 * line * sms - 8, 8 * line * sms - 7):           # one row block less, and the line's
+        rows = torch.arange(out, device=d) % few
+        p = {k: v[rows].contiguous() for k, v in Pd.items()}
+        codes, what = cd[rows].contiguous(), torch.full((out, n_in), float("nan"), device=d)
+        api.uq_quantize_fwd(Wd[rows].contiguous(), q, g, p, codes, what, mode, step, 2)
+        assert torch.equal(what, torch.from_numpy(r_what).to(d)[rows])
+        assert torch.equal(codes, torch.from_numpy(np.asarray(r_codes, np.uint8)).to(d)[rows])
+    api.uq_check_device()
+
+
 def test_deterministic_and_in_bounds():
     """Two identical calls give identical bits; outputs written into the middle
     of larger buffers leave the sentinel margins untouched."""
