@@ -187,6 +187,26 @@ def test_init_groups_of_256_with_a_lane_each(q):
     assert C.check_init(W, q, g, 4, api.CLIP_FIXED_MIN, got, C.host(codes), ref, errs, chosen, f"lanes q={q}") == 1.0
 
 
+@pytest.mark.parametrize("q,G,waves", [(1, 3, 4), (2, 3, 1), (2, 1, 3), (3, 1, 2), (4, 1, 3)])
+def test_init_groups_of_256_on_both_sides_of_a_wave_line(q, G, waves):
+    """Groups of 256: a warp each up to so many waves of eight per SM, a lane each beyond."""
+    g, line = 256, waves * 8 * torch.cuda.get_device_properties(0).multi_processor_count
+    rng = np.random.default_rng(q + G)
+    few = 32
+    raw, W = synth.bf16_round((rng.standard_t(4, (few, g)) * 0.014).astype(np.float32))
+    ref, errs, chosen = O.unified_init(W, q, g, G=G, T=3, return_errors=True)
+    for out in (line, line + 1):                              # one group to a row, some rows repeated
+        rows = np.arange(out) % few
+        p = api.empty_params(out, g, q, g, C.dev())
+        codes = torch.empty(out, g, dtype=torch.uint8, device=C.dev())
+        api.uq_init_params(api.weights_tensor(raw[rows], C.dev()), q, g, p, codes, G=G, T=3)
+        got, gc = {k: C.host(v) for k, v in p.items()}, C.host(codes)
+        C.check_init(W, q, g, G, api.CLIP_FIXED_MIN, {k: v[:few] for k, v in got.items()}, gc[:few], ref, errs, chosen,
+                     f"q={q} G={G} {out} groups")
+        for v in (*got.values(), gc):
+            assert np.array_equal(v, v[:few][rows])           # every copy has the same bits
+
+
 def test_edge_level_ties_negative_alpha_and_high_code_bits():
     """alpha_1 == alpha_2 makes two code words share a level (ties in the sort
     and in the mapping); a negative alpha reverses part of the order; code
