@@ -1041,17 +1041,37 @@ cudaError_t launch_gemv(const uint32_t* planes, const float* astar, const float*
     // The lookup tables hold one token, so their kernels build them and read
     // the planes once per token; the tensor-core product reads the planes once
     // for up to 64 columns.  Four tokens and more: 30.3 vs 18.3 us on 14336 x
-    // 4096, 32 vs 24 on 8192 x 8192, 12.0 vs 11.8 on 1024 x 4096 g = 32 q = 4.
-    // Three: 23.5 vs 18.2 us on 14336 x 4096 (2 tokens: 16.4 vs 18.2), 77 vs 68
-    // on 8192 x 28672 (53 vs 68), 7.2 vs 5.8 on 256 x 512; but with the blocks
-    // of smaller groups 27.1 vs 29.7 on 8192 x 8192 g = 64, 9.6 vs 10.8 on 1024
-    // x 4096 g = 32 q = 4, and 9.7 vs 10.4 on 100 x 8192 g = 512 q = 4.
-    // Two tokens where the 512-column kernels would run: 35.1 vs 20.2 us on
-    // 4096 x 11008 g = 64, but 8.4 vs 8.6 on 1024 x 8192 g = 512.
-    const bool wide = n_in % kWideCols == 0 && g <= 256, large = out * n_in >= (int64_t(1) << 24);
-    const bool three = wide ? g >= 128 : large || q < 4 || g <= 256;
-    if (batch >= 4 || (batch == 3 && three) || (batch == 2 && !wide && large))
-        return launch_bcq_tc(planes, astar, zstar, out, n_in, q, g, x, xdtype, batch, y, work, st);
+    // 4096, 32 vs 24 on 8192 x 8192, 12.0 vs 11.8 on 1024 x 4096 g = 32 q = 4; but four
+    // of a small matrix with q = 4 9.6 vs 10.8 on 512 x 1536 g = 32, 9.6 vs 10.0 on 300 x
+    // 2560 g = 64.
+    // Three, 1024-column tiles: 23.5 vs 18.2 us on 14336 x 4096 (2 tokens: 16.4 vs
+    // 18.2), 77 vs 68 on 8192 x 28672 (53 vs 68); but with the blocks of smaller
+    // groups 27.1 vs 29.7 on 8192 x 8192 g = 64, 9.6 vs 10.8 on 1024 x 4096 g = 32 q
+    // = 4.  Three, else: expanding q planes into small blocks takes a large enough
+    // matrix (lookups vs tensor cores, us): g = 32 q = 4 7.8 vs 11.0 on 512 x 1536,
+    // 13.7 vs 15.2 on 777 x 4128; q = 3 7.7 vs 9.6, 12.9 vs 12.7; q = 2 7.5 vs 8.2, 12.1
+    // vs 10.6; g = 64 q = 4 8.0 vs 9.9 on 300 x 2560, 13.9 vs 14.2 on 1000 x 3520; q = 3
+    // 7.8 vs 8.8, 12.9 vs 12.4; g = 128 q = 4 7.8 vs 8.8 on 512 x 1536, 7.7 vs 7.6 on
+    // 4096 x 512; other groups 7.2 vs 5.8 on 256 x 512, but q = 4, g = 512 9.6 vs 10.3
+    // on 100 x 8192 (fp32), and q = 3, 4 16.2 vs 17.4 on 1024 x 16384 (few row tiles).
+    // Two tokens where the 512-column kernels would run: 35.1 vs 20.2 us on 4096 x
+    // 11008 g = 64, but 8.4 vs 8.6 on 1024 x 8192 g = 512; of larger groups 25.5 vs
+    // 24.0 on 4096 x 14336 q = 3, but q = 4 33.9 vs 41.9, and 1024 x 16384 q = 2 10.9 vs
+    // 12.9.
+    const int64_t size = out * n_in, large = int64_t(1) << 24;
+    bool dense = batch >= 4;
+    if (n_in % kWideCols == 0 && g <= 256) {
+        dense |= batch == 3 && g >= 128;
+    } else if (batch == 4) {
+        dense = !(q == 4 && g <= 64 && size < int64_t(1) << 20);
+    } else if (batch == 3) {
+        const int least = g == 32 ? (q == 1 ? 0 : q == 2 ? 20 : 22) : g == 64 ? (q <= 2 ? 0 : q == 3 ? 20 : 22)
+                          : g == 128 ? (q == 4 ? 20 : 0) : q == 4 && g > 256 ? 24 : 0;
+        dense = size >= int64_t(1) << least && !(g > 256 && q >= 3 && size >= large && out < 2048);
+    } else if (batch == 2) {
+        dense = size >= large && (g <= 256 || (q <= 3 && out >= 2048));
+    }
+    if (dense) return launch_bcq_tc(planes, astar, zstar, out, n_in, q, g, x, xdtype, batch, y, work, st);
     switch (q) {
         case 1: return gemv_x<1>(planes, astar, zstar, out, n_in, g, x, xdtype, batch, y, work, st);
         case 2: return gemv_x<2>(planes, astar, zstar, out, n_in, g, x, xdtype, batch, y, work, st);

@@ -101,9 +101,10 @@ def test_gemv_many_rows(out, n_in, g, q):
     check(planes, a_star, z_star, x, g, label=f"{out} rows {n_in} g{g} q{q}")
 
 
-# The tensor-core product (3 tokens and more): row tiles of 128 with a remainder, one row, columns that are
-# no whole 128-column pass (per-thread loads), slices that begin inside a pass's four groups, every group
-# size class; 16, 32 and 64 matrix columns and several chunks of tokens (an fp32 token takes three columns)
+# The tensor-core product (5 tokens and more, 2 to 4 where it is the faster one): row tiles of 128 with a
+# remainder, one row, columns that are no whole 128-column pass (per-thread loads), slices that begin inside
+# a pass's four groups, every group size class; 16, 32 and 64 matrix columns and several chunks of tokens (an
+# fp32 token takes three columns)
 @pytest.mark.parametrize("out,n_in,g,q", [(1, 32, 32, 3), (127, 96, 32, 1), (129, 192, 64, 2), (300, 320, 64, 4),
                                           (128, 128, 128, 3), (257, 640, 128, 2), (65, 11008, 128, 3),
                                           (40, 1280, 256, 4), (31, 3072, 1024, 1), (2500, 6080, 32, 2)])
@@ -113,6 +114,40 @@ def test_gemv_tensor_core_product(out, n_in, g, q, batch, xdtype):
     planes, a_star, z_star = random_export(out, n_in, q, g, seed=out + batch)
     x = np.random.default_rng(batch + q).standard_normal((batch, n_in)).astype(F32)
     check(planes, a_star, z_star, x, g, xdtype, label=f"{out}x{n_in} g{g} q{q} batch {batch} {xdtype}")
+
+
+# Two to four tokens on both sides of the lines by size, bit-width and group between the lookup tables and the
+# tensor cores (the rows around a power of two of out * in, and of out = 2048 for larger groups)
+@pytest.mark.parametrize("out,n_in,g,q,batch", [
+    (2730, 1536, 32, 4, 3), (2731, 1536, 32, 3, 3), (682, 1536, 32, 2, 3), (683, 1536, 32, 2, 3), (682, 1536, 64, 3, 3),
+    (683, 1536, 64, 3, 3), (2731, 1536, 64, 4, 3), (683, 1536, 128, 4, 3), (682, 1536, 128, 4, 3), (682, 1536, 32, 4, 4),
+    (683, 1536, 64, 4, 4), (10922, 1536, 64, 2, 2), (10923, 1536, 64, 2, 2), (2047, 8704, 512, 3, 2),
+    (2048, 8704, 512, 3, 2), (2048, 8704, 512, 4, 2), (2047, 8704, 512, 3, 3)])
+def test_gemv_on_both_sides_of_a_path_line(out, n_in, g, q, batch):
+    planes, a_star, z_star = random_export(out, n_in, q, g, seed=out + q)
+    x = np.random.default_rng(batch).standard_normal((batch, n_in)).astype(F32)
+    check(planes, a_star, z_star, x, g, "f32" if out % 2 else "bf16", label=f"{out}x{n_in} g{g} q{q} batch {batch}")
+
+
+# Several row tiles per block with two and three warpgroups, planes through the ring of tensor copies: sizes the
+# product was built for, tile counts that are no multiple of the warpgroups, a last tile of one row; and two
+# groups of 256 loaded at a time, from slices that begin inside a four-pass window and at its start.  The rows
+# checked are a few of every tile (outputs of other rows depend on other planes only).
+@pytest.mark.parametrize("out,n_in,g,q,batch,xdtype", [
+    (14336, 4096, 128, 3, 64, "bf16"), (8192, 28672, 128, 3, 4, "f32"), (128 * 152 * 5 + 1, 1024, 128, 2, 16, "bf16"),
+    (128 * 152 * 4 - 100, 512, 64, 3, 30, "bf16"), (8192, 8192, 256, 3, 4, "bf16"), (6000, 8192, 256, 4, 22, "f32"),
+    (700, 28672, 256, 2, 6, "f32"), (300, 11264, 256, 1, 33, "bf16")])
+def test_gemv_tensor_core_product_of_many_tiles_and_slices(out, n_in, g, q, batch, xdtype):
+    planes, a_star, z_star = random_export(out, n_in, q, g, seed=out + q)
+    x = np.random.default_rng(q).standard_normal((batch, n_in)).astype(F32)
+    if xdtype == "bf16":
+        _, x = synth.bf16_round(x)
+    y = gpu_gemv(planes, a_star, z_star, x, g, xdtype)
+    assert np.isfinite(y).all()
+    first = np.arange(0, out, 128)
+    rows = np.unique(np.concatenate([first, np.minimum(first + 127, out - 1), np.random.default_rng(0).integers(0, out, 60)]))
+    err = np.abs(y[:, rows] - O.bcq_gemv(np.ascontiguousarray(planes[:, rows]), a_star[rows], z_star[rows], x, g))
+    assert (err <= TOL * mass(a_star[rows], z_star[rows], x, g)).all()
 
 
 @pytest.mark.parametrize("xdtype", ["f32", "bf16"])
@@ -219,3 +254,28 @@ def test_gemv_rejects_a_small_workspace():
         api.uq_bcq_gemv(torch.from_numpy(planes.view(np.int32)).to(d), torch.from_numpy(a_star).to(d),
                         torch.from_numpy(z_star).to(d), torch.zeros(1, 1024, device=d), y, 64, workspace=ws)
     assert e.value.status == api.UQ_ERR_ARG
+
+
+def test_gemv_tensor_core_product_in_a_cuda_graph():
+    """Captured products of three kinds (one slice, several slices, per-thread loads)
+    replay with the bits of the plain calls, on inputs changed in between."""
+    d = C.dev()
+    for out, n_in, g, batch in ((300, 512, 64, 8), (2000, 8192, 128, 5), (129, 192, 64, 6)):
+        planes, a_star, z_star = random_export(out, n_in, 3, g, seed=out)
+        pd, ad, zd = torch.from_numpy(planes.view(np.int32)).to(d), torch.from_numpy(a_star).to(d), torch.from_numpy(z_star).to(d)
+        x, y = torch.zeros(batch, n_in, device=d), torch.empty(batch, out, device=d)
+        ws = torch.empty(api.uq_bcq_gemv_workspace_bytes(out, n_in, batch) // 4, device=d)
+        api.uq_bcq_gemv(pd, ad, zd, x, y, g, workspace=ws)
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            api.uq_bcq_gemv(pd, ad, zd, x, y, g, workspace=ws)
+        for seed in (1, 2):
+            x.copy_(torch.from_numpy(np.random.default_rng(seed).standard_normal((batch, n_in)).astype(F32)))
+            graph.replay()
+            torch.cuda.synchronize()
+            got = y.clone()
+            y.fill_(float("nan"))
+            api.uq_bcq_gemv(pd, ad, zd, x, y, g, workspace=ws)
+            assert torch.equal(got, y)
+        api.uq_check_device()
