@@ -20,8 +20,10 @@ from tests import gpu_cases as C
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("out,n_in,g", [(37, 4096, 128), (19, 1024, 64), (11, 768, 32), (9, 1536, 384)])
-@pytest.mark.parametrize("q", [2, 3])
+# whole units, rows of partial units for every group size of the pipelined kernels, and the general kernel
+@pytest.mark.parametrize("out,n_in,g", [(37, 4096, 128), (19, 1024, 64), (11, 768, 32), (9, 1536, 384), (7, 32 * 11, 32),
+                                        (5, 64 * 13, 64), (9, 128 * 7, 128), (6, 256 * 3, 256), (5, 512 * 3, 512)])
+@pytest.mark.parametrize("q", [1, 2, 3, 4])
 def test_element_filter_backward(out, n_in, g, q):
     raw, W, P, codes, Gup = C.make_inputs(out, n_in, q, g, seed=out + q)
     d = C.dev()

@@ -352,6 +352,37 @@ def test_forward_on_both_sides_of_a_row_block_line(q, g, n_in, mode, step, line,
     api.uq_check_device()
 
 
+@pytest.mark.parametrize("out,n_in,q,g", [(40, 64 * 13, 4, 64), (8000, 512, 3, 256)])
+def test_pipelined_kernels_of_partial_units_in_a_cuda_graph(out, n_in, q, g):
+    """Captured forwards (remap, keep) and backward replay with the bits of the plain calls."""
+    raw, W, P, codes0, Gup = C.make_inputs(40, n_in, q, g, seed=q, init_G=2, init_T=1)
+    d, left = C.dev(), []
+    rows = torch.arange(out, device=d) % 40
+    Wd, pd = api.weights_tensor(raw, d)[rows].contiguous(), {k: v[rows].contiguous() for k, v in C.to_dev(P).items()}
+    Gd = torch.from_numpy(Gup).to(d)[rows].contiguous()
+    for captured in (False, True):
+        cd = torch.from_numpy(codes0).to(d)[rows].contiguous()
+        what, gr = torch.empty(out, n_in, device=d), api.empty_grads(out, n_in, q, g, d)
+        Qz = api.Quantizer(Wd, q, g, pd, cd, what, Gd, gr)
+
+        def calls():
+            Qz.fwd(0, 2, api.MAP_LOCAL_PERIODIC)
+            Qz.bwd()
+            Qz.fwd(1, 2, api.MAP_LOCAL_PERIODIC)
+        torch.cuda.synchronize()
+        if captured:
+            graph = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(graph):
+                calls()
+            graph.replay()
+        else:
+            calls()
+        api.uq_check_device()
+        left.append({**{k: v for k, v in gr.items()}, "codes": cd, "what": what})
+    for k in left[0]:
+        assert torch.equal(left[0][k], left[1][k]), k
+
+
 def test_deterministic_and_in_bounds():
     """Two identical calls give identical bits; outputs written into the middle
     of larger buffers leave the sentinel margins untouched."""

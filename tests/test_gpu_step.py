@@ -328,6 +328,32 @@ def test_quantizer_train_step_in_a_cuda_graph():
     assert np.array_equal(C.host(cd), ref[1]) and np.array_equal(C.host(what), ref[2])
 
 
+@pytest.mark.parametrize("n_in,wd", [(8192, "bf16"), (14336, "f32")])
+def test_cluster_step_in_a_cuda_graph(n_in, wd):
+    """Rows over two and four blocks: two captured steps leave what two calls leave."""
+    q, g, out, d = 3, 128, 21, C.dev()
+    raw, W, P, codes, Gup = C.make_inputs(out, n_in, q, g, seed=n_in, wdtype=wd, init_G=2, init_T=1)
+    Wd, Gd, left = api.weights_tensor(raw, d), torch.from_numpy(Gup).to(d), []
+    for captured in (False, True):
+        pd, cd = C.to_dev(P), torch.from_numpy(codes.copy()).to(d)
+        what = torch.empty(out, n_in, dtype=torch.float32, device=d)
+        Qz = api.Quantizer(Wd, q, g, pd, cd, what, Gd, None)
+        torch.cuda.synchronize()
+        if captured:
+            graph = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(graph):
+                Qz.train_step(0)
+                Qz.train_step(1)
+            graph.replay()
+        else:
+            Qz.train_step(0)
+            Qz.train_step(1)
+        api.uq_check_device()
+        left.append({**{k: C.host(v) for k, v in pd.items()}, "codes": C.host(cd), "what": C.host(what)})
+    for k in left[0]:
+        assert np.array_equal(left[0][k], left[1][k]), k
+
+
 # ---------------------------------------------------------------------------
 # full-size workloads, sampled rows (the launch configuration of the benchmark)
 # ---------------------------------------------------------------------------
