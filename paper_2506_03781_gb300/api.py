@@ -134,15 +134,18 @@ def uq_abi_version() -> int:
 
 def uq_selftest_wait_timeout(stream=None, device=None):
     """Launches the bounded-wait self-test (a wait that runs out after ~8 ms)."""
-    dev = torch.device("cuda", torch.cuda.current_device()) if device is None else device
-    _raise(lib().uq_selftest_wait_timeout(_stream(stream, dev)))
+    _raise(lib().uq_selftest_wait_timeout(_named_stream(stream, device)))
 
 
 def uq_check_device(stream=None, device=None):
     """Synchronises ``stream`` and raises UQError if a pipelined kernel's
     bounded wait ran out since the last check."""
-    dev = torch.device("cuda", torch.cuda.current_device()) if device is None else device
-    _raise(lib().uq_check_device(_stream(stream, dev)))
+    _raise(lib().uq_check_device(_named_stream(stream, device)))
+
+
+def _named_stream(stream, device):
+    """A stream's handle, by default the current one of whatever names a device to torch (None, an index, a string, ...)."""
+    return torch.cuda.current_stream(device).cuda_stream if stream is None else _stream(stream, None)
 
 
 # ---------------------------------------------------------------------------
@@ -152,8 +155,9 @@ def uq_check_device(stream=None, device=None):
 # The current device and a device's current stream, without the Stream and
 # device objects that torch.cuda builds on every call (a call on a small matrix
 # is shorter than its marshalling).
-_current_device = torch._C._cuda_getDevice
-_current_raw_stream = torch._C._cuda_getCurrentRawStream
+# (A PyTorch without CUDA has neither; there only the import has to work.)
+_current_device = getattr(torch._C, "_cuda_getDevice", None)
+_current_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 
 
 def _check(t, name, shape, dtype, device):

@@ -300,6 +300,45 @@ def test_binding_rejects_host_tensors_before_calling(libpath):
                             torch.zeros(4, 128))
 
 
+def test_device_arguments_of_every_kind(monkeypatch):
+    """uq_check_device and uq_selftest_wait_timeout take whatever names a device,
+    as torch does, and pass its current stream."""
+    import types
+    import torch
+    from paper_2506_03781_gb300 import api
+    seen = []
+    fake = types.SimpleNamespace(uq_check_device=lambda s: seen.append(s) or 0, uq_selftest_wait_timeout=lambda s: seen.append(s) or 0)
+    monkeypatch.setattr(api, "lib", lambda: fake)
+
+    def current_stream(device=None):                      # torch's, without a GPU
+        device = torch.device("cuda" if device is None else device)
+        if device.type != "cuda":
+            raise ValueError(f"Expected a cuda device, but got: {device}")
+        return types.SimpleNamespace(cuda_stream=1000 + (3 if device.index is None else device.index))
+    monkeypatch.setattr(torch.cuda, "current_stream", current_stream)
+    for device, stream in ((None, 1003), (0, 1000), (2, 1002), ("cuda:1", 1001), ("cuda", 1003), (torch.device("cuda"), 1003),
+                           (torch.device("cuda", 1), 1001)):
+        api.uq_check_device(device=device)
+        api.uq_selftest_wait_timeout(device=device)
+        assert seen == [stream, stream], device
+        seen.clear()
+    api.uq_check_device(7, device=0)                      # a stream given by its handle
+    assert seen == [7]
+    with pytest.raises(ValueError):
+        api.uq_check_device(device="cpu")
+
+
+def test_import_without_cuda_bindings_in_torch():
+    """A PyTorch built without CUDA lacks the device queries; importing the binding needs none."""
+    import subprocess
+    import sys
+    code = ("import torch\n"
+            "for n in ('_cuda_getDevice', '_cuda_getCurrentRawStream'):\n"
+            "    if hasattr(torch._C, n): delattr(torch._C, n)\n"
+            "import paper_2506_03781_gb300.api\n")
+    subprocess.run([sys.executable, "-c", code], check=True, cwd=ROOT)
+
+
 def test_oracle_and_product_are_independent():
     """The oracle imports nothing from the product package and vice versa;
     the only shared module is the seeded input generator."""
