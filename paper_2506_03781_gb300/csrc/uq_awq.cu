@@ -399,7 +399,8 @@ static cudaError_t run_awq_stream_fwd(const Shape& sh, const void* W, uq_params_
     int grid = 0;
     cudaError_t e = grid_for<AwqTag<St, MODE>>(kern, dyn, n_rb, grid);
     if (e != cudaSuccess) return e;
-    return launch_dependent(kern, grid, kThreads, dyn, st, W, p.sa, p.delta, p.za, p.alpha, p.zb, codes, what, sh.out, sh.n_in, R, n_rb);
+    return launch_dependent(kern, grid, kThreads, dyn, st, W, p.sa, p.delta, p.za, p.alpha, p.zb, codes, what, sh.out,
+                            sh.n_in, R, n_rb);
 }
 
 template <int Q, typename WT, int G_>
@@ -696,10 +697,11 @@ static cudaError_t run_awq_stream_bwd(const Shape& sh, const void* W, uq_params_
     auto kern = awq_stream_bwd_kernel<Q, WT, G_>;
     cudaError_t e = grid_for<AwqTag<St, 9>>(kern, dyn, n_rb, unused);    // shared-memory attribute (once)
     if (e != cudaSuccess) return e;
-    e = launch_dependent(kern, grid, kThreads, dyn, st, W, p.sa, p.delta, p.za, p.alpha, p.zb, codes, gup, gr.ddelta, gr.dza,
-                                      gr.dalpha, gr.dzb, work, sh.out, sh.n_in, R, n_rb);
+    e = launch_dependent(kern, grid, kThreads, dyn, st, W, p.sa, p.delta, p.za, p.alpha, p.zb, codes, gup, gr.ddelta,
+                         gr.dza, gr.dalpha, gr.dzb, work, sh.out, sh.n_in, R, n_rb);
     if (e != cudaSuccess) return e;
-    return launch_dependent(awq_colsum_kernel, (sh.n_in + 31) / 32, 32 * kColsumSlices, 0, st, work, gr.dsa, sh.n_in, grid * R);
+    return launch_dependent(awq_colsum_kernel, (sh.n_in + 31) / 32, 32 * kColsumSlices, 0, st, work, gr.dsa, sh.n_in,
+                            grid * R);
 }
 
 template <int Q, typename WT>
@@ -718,11 +720,12 @@ static cudaError_t awq_lpg(bool bwd, int mode, const Shape& sh, const void* W, u
     awq_grid(sh, LPG, cb, ranges, rpr);
     const dim3 grid(cb, (unsigned)ranges);
     if (bwd) {
-        cudaError_t e = launch_dependent(awq_bwd_kernel<Q, WT, LPG>, grid, kThreads, 0, st, W, p.sa, p.delta, p.za, p.alpha, p.zb, codes, gup,
-                                                             gr.ddelta, gr.dza, gr.dalpha, gr.dzb, work, sh.out,
-                                                             sh.n_in, sh.g, rpr);
+        cudaError_t e = launch_dependent(awq_bwd_kernel<Q, WT, LPG>, grid, kThreads, 0, st, W, p.sa, p.delta, p.za,
+                                         p.alpha, p.zb, codes, gup, gr.ddelta, gr.dza, gr.dalpha, gr.dzb, work,
+                                         sh.out, sh.n_in, sh.g, rpr);
         if (e != cudaSuccess) return e;
-        return launch_dependent(awq_colsum_kernel, (sh.n_in + 31) / 32, 32 * kColsumSlices, 0, st, work, gr.dsa, sh.n_in, (int)ranges);
+        return launch_dependent(awq_colsum_kernel, (sh.n_in + 31) / 32, 32 * kColsumSlices, 0, st, work, gr.dsa,
+                                sh.n_in, (int)ranges);
     }
     if (mode == FWD_KEEP)
         return launch_dependent(awq_fwd_kernel<Q, WT, LPG, FWD_KEEP>, grid, kThreads, 0, st, W, p.sa, p.delta, p.za,
@@ -730,8 +733,8 @@ static cudaError_t awq_lpg(bool bwd, int mode, const Shape& sh, const void* W, u
     if (mode == FWD_REMAP)
         return launch_dependent(awq_fwd_kernel<Q, WT, LPG, FWD_REMAP>, grid, kThreads, 0, st, W, p.sa, p.delta, p.za,
                                 p.alpha, p.zb, codes, what, sh.out, sh.n_in, sh.g, rpr);
-    return launch_dependent(awq_fwd_kernel<Q, WT, LPG, FWD_FULL>, grid, kThreads, 0, st, W, p.sa, p.delta, p.za, p.alpha,
-                            p.zb, codes, what, sh.out, sh.n_in, sh.g, rpr);
+    return launch_dependent(awq_fwd_kernel<Q, WT, LPG, FWD_FULL>, grid, kThreads, 0, st, W, p.sa, p.delta, p.za,
+                            p.alpha, p.zb, codes, what, sh.out, sh.n_in, sh.g, rpr);
 }
 
 template <int Q, typename WT>

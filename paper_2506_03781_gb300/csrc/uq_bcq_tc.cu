@@ -151,19 +151,23 @@ __device__ __forceinline__ void commit(uint32_t bar) {
 // 16 words per thread: lane i of the warp holds row i of its 32 rows
 __device__ __forceinline__ void load(uint32_t addr, float (&r)[16]) {
     asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, "
+        "[%16];\n\t"
         "tcgen05.wait::ld.sync.aligned;"
-        : "=f"(r[0]), "=f"(r[1]), "=f"(r[2]), "=f"(r[3]), "=f"(r[4]), "=f"(r[5]), "=f"(r[6]), "=f"(r[7]), "=f"(r[8]), "=f"(r[9]), "=f"(r[10]), "=f"(r[11]), "=f"(r[12]), "=f"(r[13]), "=f"(r[14]), "=f"(r[15])
+        : "=f"(r[0]), "=f"(r[1]), "=f"(r[2]), "=f"(r[3]), "=f"(r[4]), "=f"(r[5]), "=f"(r[6]), "=f"(r[7]),
+          "=f"(r[8]), "=f"(r[9]), "=f"(r[10]), "=f"(r[11]), "=f"(r[12]), "=f"(r[13]), "=f"(r[14]), "=f"(r[15])
         : "r"(addr)
         : "memory");
 }
 
 __device__ __forceinline__ void store(uint32_t addr, const uint32_t (&r)[16]) {
-    asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};" ::"r"(addr),
-                 "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
-                 : "memory");
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};" ::
+            "r"(addr),
+        "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]),
+        "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
+        : "memory");
 }
-
 
 // Instruction descriptor: fp32 sums, bf16 operands, both K-major, M = 128.
 __host__ __device__ constexpr uint32_t idesc(int n) {
@@ -765,8 +769,9 @@ cudaError_t run_tc(const uint32_t* planes, const float* astar, const float* zsta
     while (cols < p.groups * tc_tmem_cols(GB, N)) cols *= 2;
     int smem = 1024 + p.sb_per * tc_pass_bytes(GB, N) + (staged ? p.groups * kTcStages * tc_stage_bytes(Q, N) : 0);
     if (smem < kTcMinSmem) smem = kTcMinSmem;
-    e = launch_dependent(kern, dim3((unsigned)(p.n_ks * p.n_rb), (unsigned)chunks), dim3(p.groups * 160), (size_t)smem, st, map, planes, astar, zstar, x, x_bf16, p.n_ks > 1 ? work : y, out, n_in, g, batch,
-                           p.n_ks, p.sb_per, p.tiles, cols, staged ? 1 : 0, ex);
+    e = launch_dependent(kern, dim3((unsigned)(p.n_ks * p.n_rb), (unsigned)chunks), dim3(p.groups * 160),
+                         (size_t)smem, st, map, planes, astar, zstar, x, x_bf16,
+                         p.n_ks > 1 ? work : y, out, n_in, g, batch, p.n_ks, p.sb_per, p.tiles, cols, staged ? 1 : 0, ex);
     if (e != cudaSuccess || p.n_ks == 1) return e;
     return gemv_reduce(work, y, (int64_t)batch * out, p.n_ks, st);
 }

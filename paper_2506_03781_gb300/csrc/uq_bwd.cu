@@ -29,7 +29,9 @@ namespace uq {
 
 // ELEM: the whole-element filter (a filtered element drops out of every
 // gradient); otherwise the filter cuts the straight-through path only.
-template <int Q, typename WT, int LPG, bool ELEM>
+constexpr int kBwdLanes = 32;           // lanes per group
+
+template <int Q, typename WT, bool ELEM>
 __global__ void __launch_bounds__(kThreads, UQ_BWD_MIN_BLOCKS)
 bwd_kernel(const void* __restrict__ W, const float* __restrict__ S, const float* __restrict__ SR,
            const float* __restrict__ DELTA, const float* __restrict__ ZU, const float* __restrict__ ALPHA,
@@ -38,7 +40,7 @@ bwd_kernel(const void* __restrict__ W, const float* __restrict__ S, const float*
            float* __restrict__ DZB, float* __restrict__ DALPHA, int64_t out, int n_in, int g, int R) {
     inputs_ready();
     constexpr int L = 1 << Q;
-    constexpr int NG = 32 / LPG;                 // groups per unit
+    constexpr int LPG = kBwdLanes, NG = 32 / LPG;   // groups per unit
     using SR8 = SegReduce<LPG>;
     __shared__ LvTab<Q, NG> tabs[kWarps];
     __shared__ float tau_s[kWarps][NG];
@@ -149,16 +151,16 @@ bwd_kernel(const void* __restrict__ W, const float* __restrict__ S, const float*
     }
 }
 
-template <int Q, typename WT, int LPG, bool ELEM>
+template <int Q, typename WT, bool ELEM>
 static cudaError_t run_bwd(const Shape& sh, const void* W, uq_params p, const uint8_t* codes, const float* gup,
                            uq_grads gr, cudaStream_t st) {
-    constexpr int NG = 32 / LPG;
+    constexpr int NG = 32 / kBwdLanes;
     const int Gr = sh.n_in / sh.g;
     const int R = rows_per_block((Gr + NG - 1) / NG);
     const int64_t blocks = (sh.out + R - 1) / R;
-    return launch_dependent(bwd_kernel<Q, WT, LPG, ELEM>, dim3((unsigned)blocks), kThreads, 0, st, 
-        W, p.s, p.sr, p.delta, p.zu, p.alpha, p.zb, codes, gup, gr.ds, gr.dsr, gr.ddelta, gr.dzu, gr.dzb, gr.dalpha,
-        sh.out, sh.n_in, sh.g, R);
+    return launch_dependent(bwd_kernel<Q, WT, ELEM>, dim3((unsigned)blocks), kThreads, 0, st, W, p.s, p.sr, p.delta,
+                            p.zu, p.alpha, p.zb, codes, gup, gr.ds, gr.dsr, gr.ddelta, gr.dzu, gr.dzb, gr.dalpha,
+                            sh.out, sh.n_in, sh.g, R);
 }
 
 template <int Q>
@@ -166,10 +168,10 @@ static cudaError_t bwd_w(const Shape& sh, const void* W, uq_params p, const uint
                          uq_grads gr, int filter, cudaStream_t st) {
     const bool elem = filter == UQ_FILTER_ELEMENT;
     if (sh.wdtype == UQ_W_BF16)
-        return elem ? run_bwd<Q, WBF16, 32, true>(sh, W, p, codes, gup, gr, st)
-                    : run_bwd<Q, WBF16, 32, false>(sh, W, p, codes, gup, gr, st);
-    return elem ? run_bwd<Q, WF32, 32, true>(sh, W, p, codes, gup, gr, st)
-                : run_bwd<Q, WF32, 32, false>(sh, W, p, codes, gup, gr, st);
+        return elem ? run_bwd<Q, WBF16, true>(sh, W, p, codes, gup, gr, st)
+                    : run_bwd<Q, WBF16, false>(sh, W, p, codes, gup, gr, st);
+    return elem ? run_bwd<Q, WF32, true>(sh, W, p, codes, gup, gr, st)
+                : run_bwd<Q, WF32, false>(sh, W, p, codes, gup, gr, st);
 }
 
 cudaError_t launch_bwd(const Shape& sh, const void* W, uq_params p, const uint8_t* codes, const float* gup,

@@ -168,8 +168,8 @@ static cudaError_t run_export(const Shape& sh, const void* W, uq_params p, const
                               typename OT::T* astar, typename OT::T* zstar, cudaStream_t st) {
     const int64_t words = sh.n_in / 32;
     const int grid = export_grid(sh.out * (!EQ4 && (words & 3) == 0 ? words / 4 : words));
-    return launch_dependent(export_kernel<Q, WT, EQ4, OT>, grid, kThreads, 0, st, W, p.delta, p.zu, p.alpha, p.zb, codes, planes, astar,
-                                                             zstar, sh.out, sh.n_in, sh.g);
+    return launch_dependent(export_kernel<Q, WT, EQ4, OT>, grid, kThreads, 0, st, W, p.delta, p.zu, p.alpha, p.zb,
+                            codes, planes, astar, zstar, sh.out, sh.n_in, sh.g);
 }
 
 template <int Q, typename OT>

@@ -144,8 +144,8 @@ static cudaError_t run_fwd(const Shape& sh, const void* W, uq_params p, uint8_t*
     const int Gr = sh.n_in / sh.g;
     const int R = rows_per_block((Gr + NG - 1) / NG);
     const int64_t blocks = (sh.out + R - 1) / R;
-    return launch_dependent(fwd_kernel<Q, WT, LPG>, dim3((unsigned)blocks), kThreads, 0, st, 
-        W, p.s, p.sr, p.delta, p.zu, p.alpha, p.zb, codes, what, sh.out, sh.n_in, sh.g, R, mode);
+    return launch_dependent(fwd_kernel<Q, WT, LPG>, dim3((unsigned)blocks), kThreads, 0, st, W, p.s, p.sr, p.delta,
+                            p.zu, p.alpha, p.zb, codes, what, sh.out, sh.n_in, sh.g, R, mode);
 }
 
 template <int Q, typename WT>

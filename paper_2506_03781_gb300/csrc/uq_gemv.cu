@@ -955,8 +955,8 @@ static cudaError_t run_gemv(const uint32_t* planes, const float* astar, const fl
             if (e != cudaSuccess) return e;
             int64_t n_rb = 0, rpb = 0;
             gemv_row_blocks(out, n_tiles, per_sm, n_rb, rpb);
-            e = launch_dependent(kern, (unsigned)(n_rb * n_tiles), kGemvThreads, smem_tma, st, mp, ma, mz, x, work, out,
-                                 n_in, batch, n_tiles, rpb);
+            e = launch_dependent(kern, (unsigned)(n_rb * n_tiles), kGemvThreads, smem_tma, st, mp, ma, mz, x, work,
+                                 out, n_in, batch, n_tiles, rpb);
             if (e != cudaSuccess) return e;
             return gemv_reduce(work, y, (int64_t)batch * out, n_tiles, st);
         }
@@ -967,8 +967,8 @@ static cudaError_t run_gemv(const uint32_t* planes, const float* astar, const fl
     if (e != cudaSuccess) return e;
     int64_t n_rb = 0, rpb = 0;
     gemv_row_blocks(out, n_tiles, per_sm, n_rb, rpb);
-    e = launch_dependent(kern, (unsigned)(n_rb * n_tiles), kGemvThreads, smem, st, planes, astar, zstar, x, work, out, n_in,
-                         g, batch, n_tiles, rpb, pwide);
+    e = launch_dependent(kern, (unsigned)(n_rb * n_tiles), kGemvThreads, smem, st, planes, astar, zstar, x, work, out,
+                         n_in, g, batch, n_tiles, rpb, pwide);
     if (e != cudaSuccess) return e;
     return gemv_reduce(work, y, (int64_t)batch * out, n_tiles, st);
 }
@@ -998,8 +998,8 @@ static cudaError_t run_gemv_wide(const uint32_t* planes, const float* astar, con
         const int n_tiles = n_in / kWideCols;
         int64_t n_rb = 0, rpb = 0;
         gemv_row_blocks(out, n_tiles, per_sm, n_rb, rpb, (double)kWideLutRows);
-        e = launch_dependent(kern, (unsigned)(n_rb * n_tiles), NW * 32, DYN, st, mp, ma, mz, x, work, out, n_in, batch, n_tiles,
-                             rpb);
+        e = launch_dependent(kern, (unsigned)(n_rb * n_tiles), NW * 32, DYN, st, mp, ma, mz, x, work, out, n_in,
+                             batch, n_tiles, rpb);
         if (e != cudaSuccess) return e;
         return gemv_reduce(work, y, (int64_t)batch * out, n_tiles, st);
     } else {

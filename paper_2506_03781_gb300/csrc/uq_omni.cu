@@ -546,7 +546,8 @@ static cudaError_t run_omni_stream_fwd(const Shape& sh, const void* W, uq_params
     int grid = 0;
     cudaError_t e = grid_for<OmniTag<St, MODE>>(kern, dyn, n_rb, grid);
     if (e != cudaSuccess) return e;
-    return launch_dependent(kern, grid, kThreads, dyn, st, W, p.beta, p.gamma, p.alpha, p.zb, codes, what, sh.out, sh.n_in, R, n_rb);
+    return launch_dependent(kern, grid, kThreads, dyn, st, W, p.beta, p.gamma, p.alpha, p.zb, codes, what, sh.out,
+                            sh.n_in, R, n_rb);
 }
 
 template <int Q, typename WT, int G_>
@@ -561,8 +562,8 @@ static cudaError_t run_omni_stream_bwd(const Shape& sh, const void* W, uq_params
     int grid = 0;
     cudaError_t e = grid_for<OmniTag<St, 9>>(kern, dyn, n_rb, grid);
     if (e != cudaSuccess) return e;
-    return launch_dependent(kern, grid, kThreads, dyn, st, W, p.beta, p.gamma, p.alpha, p.zb, codes, gup, gr.dbeta, gr.dgamma, gr.dalpha,
-                                      gr.dzb, sh.out, sh.n_in, R, n_rb);
+    return launch_dependent(kern, grid, kThreads, dyn, st, W, p.beta, p.gamma, p.alpha, p.zb, codes, gup, gr.dbeta,
+                            gr.dgamma, gr.dalpha, gr.dzb, sh.out, sh.n_in, R, n_rb);
 }
 
 template <int Q, typename WT, int G_>
@@ -620,8 +621,8 @@ static cudaError_t run_omni_fwd(const Shape& sh, const void* W, uq_params_omni p
     const int Gr = sh.n_in / sh.g;
     const int R = rows_per_block((Gr + NG - 1) / NG);
     const int64_t blocks = (sh.out + R - 1) / R;
-    return launch_dependent(omni_fwd_kernel<Q, WT, LPG, MODE>, dim3((unsigned)blocks), kThreads, 0, st, 
-        W, p.beta, p.gamma, p.alpha, p.zb, codes, what, dout, zout, sh.out, sh.n_in, sh.g, R);
+    return launch_dependent(omni_fwd_kernel<Q, WT, LPG, MODE>, dim3((unsigned)blocks), kThreads, 0, st, W, p.beta,
+                            p.gamma, p.alpha, p.zb, codes, what, dout, zout, sh.out, sh.n_in, sh.g, R);
 }
 
 template <int Q, typename WT, int LPG>
@@ -631,9 +632,9 @@ static cudaError_t run_omni_bwd(const Shape& sh, const void* W, uq_params_omni p
     const int Gr = sh.n_in / sh.g;
     const int R = rows_per_block((Gr + NG - 1) / NG);
     const int64_t blocks = (sh.out + R - 1) / R;
-    return launch_dependent(omni_bwd_kernel<Q, WT, LPG>, dim3((unsigned)blocks), kThreads, 0, st, 
-        W, p.beta, p.gamma, p.alpha, p.zb, codes, gup, gr.dbeta, gr.dgamma, gr.dalpha, gr.dzb, sh.out, sh.n_in,
-        sh.g, R);
+    return launch_dependent(omni_bwd_kernel<Q, WT, LPG>, dim3((unsigned)blocks), kThreads, 0, st, W, p.beta, p.gamma,
+                            p.alpha, p.zb, codes, gup, gr.dbeta, gr.dgamma, gr.dalpha, gr.dzb, sh.out, sh.n_in, sh.g,
+                            R);
 }
 
 // kind: 0 forward (mode), 1 backward, 2 scales only

@@ -243,8 +243,8 @@ static cudaError_t run_ragged_bwd(const Shape& sh, const void* W, uq_params p, c
     if (e != cudaSuccess) return e;
     const RaggedSrc src{static_cast<const unsigned char*>(W), reinterpret_cast<const unsigned char*>(p.s),
                         reinterpret_cast<const unsigned char*>(gup), codes, p.delta, p.zu, p.zb, p.alpha};
-    return launch_dependent(kern, grid, kThreads, dyn, st, src, p.sr, gr.ds, gr.dsr, gr.ddelta, gr.dzu, gr.dzb, gr.dalpha, sh.out, sh.n_in,
-                                      R, n_rb);
+    return launch_dependent(kern, grid, kThreads, dyn, st, src, p.sr, gr.ds, gr.dsr, gr.ddelta, gr.dzu, gr.dzb,
+                            gr.dalpha, sh.out, sh.n_in, R, n_rb);
 }
 
 template <int Q, int G_>

@@ -536,9 +536,9 @@ static cudaError_t run_bwd_stream(const Shape& sh, const void* W, uq_params p, c
     // one occupancy cache (and shared-memory opt-in) per kernel variant
     cudaError_t e = grid_for<BwdTag<St, ELEM>>(kern, dyn, n_rb, grid);
     if (e != cudaSuccess) return e;
-    return launch_dependent(kern, grid, kThreads, dyn, st, W, p.s, p.sr, p.delta, p.zu, p.alpha, p.zb, codes, gup, gr.ds, gr.dsr,
-                                      gr.ddelta, gr.dzu, gr.dzb, gr.dalpha, sh.out, sh.n_in, R, n_rb,
-                                      U >= kBranchyUnits ? 1 : 0);
+    return launch_dependent(kern, grid, kThreads, dyn, st, W, p.s, p.sr, p.delta, p.zu, p.alpha, p.zb, codes, gup,
+                            gr.ds, gr.dsr, gr.ddelta, gr.dzu, gr.dzb, gr.dalpha, sh.out, sh.n_in, R, n_rb,
+                            U >= kBranchyUnits ? 1 : 0);
 }
 
 template <typename St, bool SEARCH>
@@ -556,8 +556,8 @@ static cudaError_t run_fwd_stream_mode(const Shape& sh, const void* W, uq_params
     int grid = 0;
     cudaError_t e = grid_for<FwdTag<St, SEARCH>>(kern, dyn, n_rb, grid);
     if (e != cudaSuccess) return e;
-    return launch_dependent(kern, grid, kThreads, dyn, st, W, p.s, p.sr, p.delta, p.zu, p.alpha, p.zb, codes, what, sh.out, sh.n_in, R,
-                                      n_rb);
+    return launch_dependent(kern, grid, kThreads, dyn, st, W, p.s, p.sr, p.delta, p.zu, p.alpha, p.zb, codes, what,
+                            sh.out, sh.n_in, R, n_rb);
 }
 
 template <int Q, int G_, int KU>
@@ -571,7 +571,8 @@ static cudaError_t run_keep_stream(const Shape& sh, uq_params p, const uint8_t* 
     int grid = 0;
     cudaError_t e = grid_for<St>(kern, dyn, n_rb, grid);
     if (e != cudaSuccess) return e;
-    return launch_dependent(kern, grid, kThreads, dyn, st, p.delta, p.zu, p.alpha, p.zb, codes, what, sh.out, sh.n_in, R, n_rb);
+    return launch_dependent(kern, grid, kThreads, dyn, st, p.delta, p.zu, p.alpha, p.zb, codes, what, sh.out, sh.n_in,
+                            R, n_rb);
 }
 
 // Units per keep item: as many adjacent units (up to 4 and kKeepMaxGroups
