@@ -396,19 +396,22 @@ uq_status uq_export_bcq_half(const void* W, uq_wdtype wdtype, int64_t out, int64
  * bitplanes [q, out, in/32] uint32, alpha_star [out, in/g, q] and
  * zb_star [out, in/g] fp32 as uq_export_bcq writes them; x [batch, in]
  * (xdtype fp32 or bf16), y [batch, out] fp32, both row-major.
- * One or two tokens: the columns are split into tiles, 1024 columns (32 per
- * lane) when in is a multiple of 1024 and g <= 256, else 512; each tile's
+ * Few tokens (one always, two to four by the shape: see launch_gemv): the
+ * columns are split into tiles, 1024 columns (32 per lane) when in is a
+ * multiple of 1024 and g <= 256, else 512; each tile's
  * contribution is formed from per-8-column partial sums of x (one table
- * lookup per plane byte).  Four tokens and more (and fewer of a large matrix
- * that the 1024-column tiles do not take): a +-1 matrix product per plane on
+ * lookup per plane byte).  Else (five tokens and more always, most products of
+ * three and four): a +-1 matrix product per plane on
  * the tensor cores, the activations as bf16 values (an fp32 one as the sum of
  * three; a token whose largest |x| in a column slice is below 2^-64 or 2^110 or
  * more is scaled there by a power of two, so that nothing above 2^-69 of it is
  * lost), fp32 sums scaled by alpha* per group.  Partial sums of tiles
  * or column slices go to `workspace` (caller-owned device memory of at least
  * uq_bcq_gemv_workspace_bytes(out, in, batch) bytes, overwritten) and are
- * summed in order into y.  Products of +-1 are exact and every sum is fp32, in
- * a fixed order for a given shape and batch: deterministic, and within a small
+ * summed in order into y.  The products of signs and activations are exact (with
+ * g >= 128 and at most 32 matrix columns but for at most 2^-33 of sum |x|, from
+ * clear bits that enter as 2^-64 or 2^-32) and every sum is fp32, in a fixed
+ * order for a given shape and batch: deterministic, and within a small
  * multiple of the fp32 unit roundoff of sum_i (sum_j |alpha*_j| + |z*|) |x_i|
  * of the exact product (the paths add in different orders, all within that
  * bound).

@@ -4,14 +4,14 @@
 // columns of one group (GB = 32, 64, or 128 for larger groups):
 //   y_r += sum_j alpha*_j (C_j x)_r + z* S,   S = sum of x over the block.
 //
-// The +-1 entries are exact in bf16 and so are the activations: a bf16 token
+// The entries are exact in bf16 and so are the activations: a bf16 token
 // is one column of the right-hand matrix, an fp32 token three (its value cut
-// into three bf16 pieces that add up to it exactly), so every product is
-// exact and the sums D_j are taken in fp32 (tcgen05.mma kind::f16, 128 rows by
+// into three bf16 pieces that add up to it), so every product is exact and the
+// sums D_j are taken in fp32 (tcgen05.mma kind::f16, 128 rows by
 // N columns, fp32 accumulators in tensor memory).  With 64 columns, or with
 // several blocks to a pass, the entries are +-1 themselves, made by two
-// operations per pair.  Else, where making them is what takes the time (450 of
-// 900 clocks), they are of four kinds, one operation
+// operations per pair.  Else, where making them is the longest part of the chain
+// (450 of 750 clocks), they are of four kinds, one operation
 // each wherever the bit lies (see expand16): +-0.5; 2 or 0, against half the
 // activation; 1 or 2^-64; 1 or 2^-32.  With S0 the sum of x over the columns
 // of the first kind, (C_j x)_r = 2 D_j + S0 - S then, but for the 2^-64 and
@@ -55,15 +55,18 @@
 // tensor memory that a kernel it waits for needs.  Deterministic; no atomics on
 // outputs.
 //
-// What bounds it: a plane of 128 x 128 takes the tensor cores 256 clocks with
-// 64 columns (measured 272) and 197 with 16, a warpgroup 1270 (700 to expand,
-// 430 to scale 64 sums) and 750: two or three warpgroups share the logic pipe,
-// which runs at half rate.  14336 x 4096, q = 3, g = 128, bf16: 64 tokens 447
-// -> 37.9 us (per-token lookup tables before), 16 tokens 114 -> 18.8 us, 4
-// tokens 30.4 -> 18.3 us (19.4 with +-1 entries); 8192 x 28672, 4 fp32 tokens:
-// 99.8 -> 70.2 us (76.4).  The same product with mma.sync and fragments in
-// registers took 72.5, 28.2, 20.6 and 108 us: every lane of a quad repeats
-// the loads and the scaling, and 64 columns are bound by that pipe (38 us).
+// What bounds it: latency.  A warpgroup takes each plane through one chain
+// (expand, store, wait for the products of the plane before, read the sums,
+// scale them: 1270 clocks with 64 columns, 750 with 16), and two or three share
+// an SM, which takes 1180 and 520 clocks a plane of 128 x 128 where the tensor
+// cores need 272 and 197.  Counters of 64 tokens of 14336 x 4096 and 4 fp32 tokens
+// of 8192 x 28672: tensor pipe 27 and 16 %, logic pipe 22 and 42 %, issue 0.47 and
+// 0.52, the largest stall the reads of tensor memory.  q = 3, g = 128, six sets of
+// inputs in turn: 64 bf16 tokens of 14336 x 4096 40.2 us (per-token lookup tables
+// 447), 16 tokens 21.4 (114), 4 tokens 20.5 (30); 8192 x 28672, 4 fp32 tokens 69.8
+// (99.8).  The same product with mma.sync and fragments in registers took 72.5 us
+// for 64 tokens and 108 for the 4: every lane of a quad repeats the loads and the
+// scaling, and 64 columns are bound by that pipe (38 us).
 // Error against 64 bits: 0.6e-7 to 1.3e-7, the lookup tables' 0.7e-7 to 1.7e-7.
 #include <cuda.h>   // CUtensorMap
 #include <cuda_bf16.h>
@@ -707,14 +710,17 @@ struct TcPlan {
 
 // Slices, tiles per block and warpgroups for the least estimated time (in SM
 // clocks): the waves of blocks, each with the operands it builds and its
-// rounds of tiles, and the slice sum where there is more than one slice.
+// rounds of tiles, and the slice sum where there is more than one slice.  The
+// constants order the plans and do not predict the time: a pass takes about
+// twice as long (64 tokens of 14336 x 4096 19 us estimated, 40.2 taken; 4 fp32
+// tokens of 8192 x 28672 34 and 69.8).
 template <int Q, int GB, int N>
 TcPlan tc_plan(int64_t out, int n_in, int chunks, bool staged) {
     const int sms = sm_count();
     const int n_sb = (n_in + kTcCols - 1) / kTcCols;
     const int64_t all = (out + kTcRows - 1) / kTcRows;
     const int most_ks = (n_in + 511) / 512;                // the workspace holds this many partials of every output
-    // a pass of one plane: alone (waits included), and what it takes of the SM among others
+    // a pass of one plane: alone, and what it takes of the SM among others
     const double alone = 450.0 + 7.0 * N, busy = 4.5 * N > 200.0 ? 4.5 * N : 200.0;
     TcPlan best{};
     double best_cost = -1.0;
