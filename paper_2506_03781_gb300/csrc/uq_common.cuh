@@ -41,15 +41,18 @@ constexpr unsigned kFull = 0xffffffffu;
 // 1.07 / 1.13 (g = 1024: 1.04 / 0.79), 300 x 11008 1.02 / 0.99 (full mapping 1.02 /
 // 0.82), 128 x 14336 1.04 / 0.83, 1024 x 8192 1.01 / 0.96, 4096 x 4096 1.01 /
 // 1.03.  Queued from the host (plain launches / now): a step of 1024 x 1024 30.6 /
-// 20.1 us, of 14336 x 4096 441 / 427 (432 without an early start).
+// 20.1 us, of 14336 x 4096 441 / 430.
 // Not for the initialization (one long launch) and the clusters of the fused
 // step (slower: see its launch).
 __device__ __forceinline__ void dependents_may_start() { asm volatile("griddepcontrol.launch_dependents;"); }
 __device__ __forceinline__ void inputs_ready() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // First thing in a pipelined per-step kernel of n_rb row blocks, of R rows of U
 // units each; many: the rounds from which on the grid evens out (0: never).
-// After a backward comes a forward, which has half its rounds (2048 x 5632: 6.7
-// and 4.5; 1.01 against 0.98 times a plain launch).
+// The forwards and the backward of partial units have such a line (4096 x 4096, g
+// = 256: 146.9 -> 143.6 us for two steps).  The backward of whole units never: it
+// is followed by a forward (14336 x 4096, two steps: 430 us against 427) or an
+// export, whose many small blocks crowd in (keep, backward and export of 14336 x
+// 4096 209.8 us against 217.1, of 4096 x 14336 223.4 against 230.8).
 constexpr int kFewBlocks = 64, kManyRounds = 6, kManyRoundsBwd = 8;
 __device__ __forceinline__ void let_next_start(int U, int R, int n_rb, int many) {
     const int blocks = (int)gridDim.x;

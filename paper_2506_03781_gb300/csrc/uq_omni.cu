@@ -415,7 +415,7 @@ omni_stream_bwd_kernel(const void* __restrict__ W, const float* __restrict__ BET
                        float* __restrict__ DALPHA, float* __restrict__ DZB, int64_t out, int n_in, int R, int n_rb) {
     using St = OmniBwdStage<Q, WT, G_>;
     constexpr int L = 1 << Q, LPG = St::LPG, NG = St::NG, NV = St::NV, UE = St::UE, NST = St::NST;
-    let_next_start(n_in / UE, R, n_rb, kManyRoundsBwd);
+    let_next_start(n_in / UE, R, n_rb, 0);
     using SR8 = SegReduce<LPG>;
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ __align__(8) unsigned long long bars[kWarps][NST];

@@ -67,7 +67,7 @@ bwd_stream_kernel(const void* __restrict__ W, const float* __restrict__ S, const
                   int n_in, int R, int n_rb, int branchy) {
     using St = Stage<Q, WT, G_, true, true, true, UQ_BWD_STAGE_BYTES>;
     constexpr int L = 1 << Q, LPG = St::LPG, NG = St::NG, NV = St::NV, UE = St::UE, NST = St::NST;
-    let_next_start(n_in / UE, R, n_rb, kManyRoundsBwd);
+    let_next_start(n_in / UE, R, n_rb, 0);
     constexpr uint32_t TX = St::TX;
     using SR8 = SegReduce<LPG>;
     extern __shared__ __align__(128) unsigned char smem[];
