@@ -34,8 +34,9 @@ constexpr unsigned kFull = 0xffffffffu;
 // have ended.  Blocks that are scheduled early go where there is room, two or
 // three of a grid to one SM, and what was one even round then takes up to twice
 // as long.  So the pipelined per-step kernels do so where they are few blocks of
-// one round (the fused step: up to two rounds), or, but for AWQ's, many rounds,
-// which even out; no other per-step kernel does.
+// one round (the fused step: up to two rounds), and the forwards (not AWQ's) and
+// the backward of partial units where they are many rounds, which even out; no
+// other per-step kernel does.
 // Captured steps (two forwards and backwards) against plain launches, with no
 // early start / with one always: 64 x 512 1.12 / 1.33 times as fast, 1024 x 1024
 // 1.07 / 1.13 (g = 1024: 1.04 / 0.79), 300 x 11008 1.02 / 0.99 (full mapping 1.02 /
